@@ -87,7 +87,10 @@ extern "C" {
 #define PT_ERR_INTERNAL  6   /* internal limit exceeded (message says which) */
 
 /* ---- precision of the pair arithmetic ---- */
-#define PT_FP64   0          /* everything in float64                        */
+#define PT_FP64   0          /* float64 results: pairs within r_out and all sums
+                                in float64, pairs outside it in float32
+                                expansions (three float32 per value), no less
+                                accurate than float64 instructions           */
 #define PT_MIXED  1          /* float64 storage, group-relative float32 pair
                                 arithmetic with float-float accumulation     */
 

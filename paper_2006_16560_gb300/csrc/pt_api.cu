@@ -163,6 +163,7 @@ struct pt_tree {
     Buf cells, pp;
     Buf pairs, nb_keys, nb_keys_s, nb_vals, nb_vals_s, nb_off, nb_idx, npairs_dev;
     Buf sort_k2, sort_v2, sort_counts, scan_sums;
+    Buf ffp, ffn;                                          // float64 force kernel's records
     Buf in_scale, scale_buf, set_mean, ssc, nd_thr, gr_thr;   // mass-dependent radii
     Buf orb_vel, orb_sv, orb_rnbf, orb_ndr, orb_ndthr, orb_grthr, orb_ctr, orb_rnb;   // orbit-dependent search
     Buf walk_spill;                                        // spill areas of the walk stacks
@@ -208,7 +209,7 @@ struct pt_tree {
                       &gr_b, &gr_nc, &gr_np, &gr_co, &gr_po, &gr_nf, &gr_fo, &gr_ord, &gpart, &red_part, &cells, &pp, &pairs,
                       &nb_keys, &nb_keys_s, &nb_vals, &nb_vals_s, &nb_off, &nb_idx, &npairs_dev,
                       &sort_k2, &sort_v2, &sort_counts, &scan_sums, &out_acc, &out_pot,
-                      &in_scale, &scale_buf, &set_mean, &ssc, &nd_thr, &gr_thr, &orb_vel, &orb_sv, &orb_rnbf, &walk_spill,
+                      &ffp, &ffn, &in_scale, &scale_buf, &set_mean, &ssc, &nd_thr, &gr_thr, &orb_vel, &orb_sv, &orb_rnbf, &walk_spill,
                       &orb_ndr, &orb_ndthr, &orb_grthr, &orb_ctr, &orb_rnb};
         for (Buf *b : all) b->release();
         d_tab.release(); d_totals.release(); d_acc.release(); d_pot.release();
@@ -332,6 +333,10 @@ int alloc_build(pt_tree *t, unsigned n, int nsets) {
     TRY(ensure(ctx, t->gpart, N * 32));
     TRY(ensure(ctx, t->red_part, (size_t)kRedBlocksMax * 48));     // reduction partials, one per block
     TRY(ensure(ctx, t->ssc, N * 8));
+    if (t->prm.precision == PT_FP64) {       // double-float records of the float64 force kernel
+        TRY(ensure(ctx, t->ffp, N * 48));
+        TRY(ensure(ctx, t->ffn, C * 96));
+    }
     TRY(ensure(ctx, t->set_mean, S * 8));
     if (t->prm.mass_dependent) {
         TRY(ensure(ctx, t->scale_buf, N * 8));
@@ -533,6 +538,10 @@ ForceArgs force_args(pt_tree *t, double *acc, double *pot, bool want_nb) {
     A.nd_c = t->nd_c.as<double4>();
     A.nd_q = t->nd_q.as<double4>();
     A.nd_f = t->nd_f.as<float4>();
+    A.nd_r = t->nd_r.as<uint2>();
+    A.sq = t->sq.as<uint4>();
+    A.ffp = t->ffp.as<float4>();
+    A.ffn = t->ffn.as<float4>();
     A.sets = t->sets.as<SetInfo>();
     A.perm = t->perm.as<unsigned>();
     A.ssc = t->ssc.as<double>();
@@ -681,7 +690,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             CK(cudaEventRecord(ctx->ev[3], st));
             ForceArgs F = force_args(t, acc, pot, want_nb);
             F.direct_groups = t->h.ngroups;           // known since the build's status read
-            nk += force_launch(F, t->prm.precision, st);
+            nk += force_launch(F, t->prm.precision, t->n, st);
             CK(cudaEventRecord(ctx->ev[4], st));
             TRY(copy_out());
             nk += force_reduce_launch(F, st);
@@ -730,7 +739,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
         CK(cudaEventRecord(ctx->ev[3], st));
         ForceArgs F = force_args(t, acc, pot, want_nb);
         F.direct_groups = t->h.ngroups;
-        nk += force_launch(F, t->prm.precision, st);
+        nk += force_launch(F, t->prm.precision, t->n, st);
         CK(cudaEventRecord(ctx->ev[4], st));
         TRY(copy_out());
         nk += force_reduce_launch(F, st);
@@ -868,7 +877,7 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
     const unsigned long long hint = t->h.ngroups ? t->h.ngroups + t->h.ngroups / 8 + 64 : 0;
     F.direct_groups = (unsigned)std::min<unsigned long long>(hint, 0x7fffffffull);
     F.count_hint = 1;
-    nk += force_launch(F, t->prm.precision, st);
+    nk += force_launch(F, t->prm.precision, t->n, st);
     nk += force_reduce_launch(F, st);
     if (want_nb) {
         nk += nb_launch(nb_args(t), st);

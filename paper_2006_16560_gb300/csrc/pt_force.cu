@@ -35,17 +35,14 @@
 // confirmed with the exact float64 test.
 #include <algorithm>
 
-#include "pt_kernels.cuh"
+#include "pt_force.cuh"
 
 namespace pt {
 
-constexpr int kFWarps = 4;
-constexpr int kFThreads = 32 * kFWarps;
 #ifndef PT_FORCE_TILE
 #define PT_FORCE_TILE 128
 #endif
 constexpr int kJ = PT_FORCE_TILE;   // list entries per warp tile of the mixed kernel
-constexpr int kJD = 64;             // list entries per warp tile of the float64 kernel
 #ifndef PT_FORCE_UNROLL_PAIRS
 #define PT_FORCE_UNROLL_PAIRS 1
 #endif
@@ -58,7 +55,6 @@ constexpr int kUnrollPP = PT_FORCE_UNROLL_PP;   // unroll of the near-segment PP
 #define PT_FORCE_UNROLL_FAR 4
 #endif
 constexpr int kUnrollFar = PT_FORCE_UNROLL_FAR;   // unroll of the far-segment PP-pair loop
-constexpr int kIB = 64;       // targets per pass of the float64 kernel (two per lane)
 constexpr int kSlotMax = 96;  // largest pass of the mixed kernel
 #ifndef PT_FORCE_MIN_BLOCKS
 #define PT_FORCE_MIN_BLOCKS 4     // resident CTAs per SM the register budget is sized for
@@ -105,34 +101,6 @@ __device__ __forceinline__ f2x fma2(f2x a, f2x b, f2x c) {
     f2x r;
     asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
-}
-
-__device__ __forceinline__ double exact_r2(double4 a, double4 b) {
-    const double dx = __dsub_rn(b.x, a.x), dy = __dsub_rn(b.y, a.y), dz = __dsub_rn(b.z, a.z);
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
-__device__ __forceinline__ void emit_pair(const ForceArgs &A, unsigned pi, unsigned pj) {
-    unsigned long long k = atomicAdd(&A.st->npairs, 1ull);
-    if (k < A.pair_cap) A.pairs[k] = make_uint2(pi, pj);
-}
-
-// Per-set constants of the changeover, float64 and float32.
-struct Chg {
-    double ri, ro, c2, lam, invw, c0, tiny, rout2;
-};
-__device__ __forceinline__ Chg make_chg(const SetInfo &S) {
-    Chg c;
-    c.ri = S.r_in;
-    c.ro = S.r_out;
-    c.c2 = 2.0 / (S.r_out + S.r_in);
-    c.lam = (S.r_out - S.r_in) / (S.r_out + S.r_in);
-    c.invw = 1.0 / (S.r_out - S.r_in);
-    c.c0 = -S.r_in * c.invw;
-    const double t = S.r_in > 0.0 ? S.r_in * (1.0 / 1024.0) : S.r_out * (1.0 / 1048576.0);
-    c.tiny = t * t;
-    c.rout2 = __dmul_rn(S.r_out, S.r_out);
-    return c;
 }
 
 // ===========================================================================
@@ -639,49 +607,6 @@ __device__ __forceinline__ void write_targets_ff(const ForceArgs &A, const uint2
     }
 }
 
-// Final per-target sums of the float64 kernel (threads 0..slots-1): fixed-order
-// float64 reduction over the warps, removal of the self entry, output in caller order.
-__device__ __forceinline__ void write_targets(const ForceArgs &A, const uint2 gr, unsigned i0,
-                                              unsigned slots, double c2, double (*red)[kSlotMax][4],
-                                              double (&ep)[4]) {
-    const unsigned t = threadIdx.x;
-    if (t < slots && i0 + t < gr.y) {
-        double s[4] = {0, 0, 0, 0};
-        for (int w = 0; w < kFWarps; w++)
-            for (int c = 0; c < 4; c++) s[c] += red[w][t][c];
-        const unsigned p = gr.x + i0 + t;
-        const double m = A.sp64[p].w;
-        // remove the self entry m_i 2 / (s_i (r_out + r_in))
-        const double P = s[3] - (A.massdep ? m * c2 / A.ssc[p] : m * c2);
-        const unsigned i = A.perm[p];
-        const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * P;
-        A.acc[3ull * i] = ax;
-        A.acc[3ull * i + 1] = ay;
-        A.acc[3ull * i + 2] = az;
-        A.pot[i] = phi;
-        ep[0] += 0.5 * m * phi;
-        ep[1] += m * ax;
-        ep[2] += m * ay;
-        ep[3] += m * az;
-    }
-}
-
-__device__ __forceinline__ void group_partials(const ForceArgs &A, unsigned g, double (&ep)[4],
-                                               double (*ered)[4]) {
-    const int w = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 4; c++) ep[c] = warp_sum(ep[c]);
-    if ((threadIdx.x & 31) == 0)
-        for (int c = 0; c < 4; c++) ered[w][c] = ep[c];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double e[4] = {0, 0, 0, 0};
-        for (int k = 0; k < kFWarps; k++)
-            for (int c = 0; c < 4; c++) e[c] += ered[k][c];
-        A.gpart[g] = make_double4(e[0], e[1], e[2], e[3]);
-    }
-}
-
 // Configuration class of a group's first pass (0: more than 64 targets, more
 // than one pass or the 96-slot one; then 64, 48, 32, 24 and 16 slots), in the
 // order the mixed kernel takes the groups.
@@ -780,251 +705,6 @@ __global__ void __launch_bounds__(kFThreads, PT_FORCE_MIN_BLOCKS) k_force_mixed(
             write_targets_ff(A, gr, i0, slots, c2, red, ep);
             __syncthreads();
             i0 += slots;
-        }
-        group_partials(A, g, ep, ered);
-    }
-}
-
-// ===========================================================================
-// Float64
-// ===========================================================================
-
-template <int NI, int ORDER>
-__device__ __forceinline__ void cells_tile_d(const double4 *sA, const double4 *sB, const double2 *sC,
-                                             int cnt, const double (&xx)[2], const double (&xy)[2],
-                                             const double (&xz)[2], double (&pa)[2][4]) {
-    for (int j = 0; j < cnt; j++) {
-        const double4 c = sA[j];
-        double4 q;
-        double2 q2;
-        if (ORDER == 2) {
-            q = sB[j];
-            q2 = sC[j];
-        }
-#pragma unroll
-        for (int s = 0; s < NI; s++) {
-            const double dx = c.x - xx[s], dy = c.y - xy[s], dz = c.z - xz[s];
-            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-            const double rinv = rsqrt(r2);
-            const double rinv2 = rinv * rinv;
-            const double mr = c.w * rinv;
-            const double mr3 = mr * rinv2;
-            if (ORDER == 2) {
-                const double qx = fma(q2.x, dz, fma(q.w, dy, q.x * dx));
-                const double qy = fma(q2.y, dz, fma(q.y, dy, q.w * dx));
-                const double qz = fma(q.z, dz, fma(q2.y, dy, q2.x * dx));
-                const double dqd = fma(dz, qz, fma(dy, qy, dx * qx));
-                const double rinv5 = rinv2 * rinv2 * rinv;
-                const double t = dqd * rinv5;
-                const double f = fma(2.5 * t, rinv2, mr3);
-                pa[s][0] = fma(-qx, rinv5, fma(f, dx, pa[s][0]));
-                pa[s][1] = fma(-qy, rinv5, fma(f, dy, pa[s][1]));
-                pa[s][2] = fma(-qz, rinv5, fma(f, dz, pa[s][2]));
-                pa[s][3] = fma(0.5, t, pa[s][3] + mr);
-            } else {
-                pa[s][0] = fma(mr3, dx, pa[s][0]);
-                pa[s][1] = fma(mr3, dy, pa[s][1]);
-                pa[s][2] = fma(mr3, dz, pa[s][2]);
-                pa[s][3] += mr;
-            }
-        }
-    }
-}
-
-template <int NI, bool NB, bool MD>
-__device__ __forceinline__ void pp_tile_d(const ForceArgs &A, const double4 *sP, const unsigned *sI,
-                                          const double *sS, int cnt, const Chg &C,
-                                          const double (&xx)[2], const double (&xy)[2],
-                                          const double (&xz)[2], const double (&st)[2],
-                                          const unsigned (&pid)[2], const bool (&valid)[2],
-                                          double (&pa)[2][4]) {
-    for (int j = 0; j < cnt; j++) {
-        const double4 P = sP[j];
-#pragma unroll
-        for (int s = 0; s < NI; s++) {
-            const double dx = __dsub_rn(P.x, xx[s]), dy = __dsub_rn(P.y, xy[s]), dz = __dsub_rn(P.z, xz[s]);
-            const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-            double rout2 = C.rout2, sij = 1.0;
-            if (MD) {                       // pair radii s_ij (r_in, r_out), s_ij = max(s_i, s_j)
-                sij = fmax(st[s], sS[j]);
-                const double ro = __dmul_rn(C.ro, sij);
-                rout2 = __dmul_rn(ro, ro);
-            }
-            if (NB && r2 < rout2) {
-                const unsigned pj = sI[j];
-                if (valid[s] && pj != pid[s]) emit_pair(A, pid[s], pj);
-            }
-            const double r2c = fmax(r2, C.tiny);
-            const double rinv = rsqrt(r2c);
-            const double r = MD ? (r2c * rinv) / sij : r2c * rinv;     // r / s_ij
-            const double xs = fmin(fmax(fma(r, C.invw, C.c0), 0.0), 1.0);
-            const double t = xs - 1.0;
-            const double t2 = t * t;
-            const double kq = fma(fma(fma(fma(35.0 * C.lam, xs, 20.0), xs, 10.0), xs, 4.0), xs, 1.0);
-            const double omk = fma(-t2 * t2, kq, 1.0);
-            const double x2 = xs * xs;
-            const double x5 = x2 * x2 * xs;
-            const double wp = fma(fma(fma(-5.0, xs, 20.0), xs, -28.0), xs, 14.0);
-            const double omw = fmin(fma(-C.lam * x5, wp, r * C.c2), 1.0);
-            const double mr = P.w * rinv;
-            const double fk = (omk * mr) * (rinv * rinv);
-            pa[s][0] = fma(fk, dx, pa[s][0]);
-            pa[s][1] = fma(fk, dy, pa[s][1]);
-            pa[s][2] = fma(fk, dz, pa[s][2]);
-            pa[s][3] = fma(omw, mr, pa[s][3]);
-        }
-    }
-}
-
-// Far PP entries in float64 (every pair at least r_out apart: K = W = 0):
-// plain Newtonian pairs.
-template <int NI>
-__device__ __forceinline__ void pp_tile_d_far(const double4 *sP, int cnt, const double (&xx)[2],
-                                              const double (&xy)[2], const double (&xz)[2],
-                                              double (&pa)[2][4]) {
-    for (int j = 0; j < cnt; j++) {
-        const double4 P = sP[j];
-#pragma unroll
-        for (int s = 0; s < NI; s++) {
-            const double dx = P.x - xx[s], dy = P.y - xy[s], dz = P.z - xz[s];
-            const double rinv = rsqrt(fma(dz, dz, fma(dy, dy, dx * dx)));
-            const double mr = P.w * rinv;
-            const double fk = mr * (rinv * rinv);
-            pa[s][0] = fma(fk, dx, pa[s][0]);
-            pa[s][1] = fma(fk, dy, pa[s][1]);
-            pa[s][2] = fma(fk, dz, pa[s][2]);
-            pa[s][3] += mr;
-        }
-    }
-}
-
-template <int NI, int ORDER, bool NB, bool MD>
-__device__ void group_pass_d(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0,
-                             const Chg &C, double4 (*sA)[kJD], double4 (*sB)[kJD],
-                             double2 (*sC)[kJD], unsigned (*sI)[kJD], double (*sS)[kJD],
-                             double (*red)[kSlotMax][4]) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double xx[2], xy[2], xz[2], st[2];
-    unsigned pid[2];
-    bool valid[2];
-#pragma unroll
-    for (int s = 0; s < 2; s++) {
-        const unsigned idx = i0 + lane + 32 * s;
-        valid[s] = idx < gr.y;
-        pid[s] = gr.x + (valid[s] ? idx : 0u);
-        const double4 P = A.sp64[pid[s]];
-        xx[s] = P.x; xy[s] = P.y; xz[s] = P.z;
-        st[s] = MD ? A.ssc[pid[s]] : 1.0;
-    }
-    double pa[2][4];
-#pragma unroll
-    for (int s = 0; s < 2; s++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) pa[s][c] = 0.0;
-    const unsigned nc = A.gr_nc[g];
-    const unsigned long long co = A.gr_co[g];
-    for (unsigned t = w * kJD; t < nc; t += kFWarps * kJD) {
-        const int cnt = (int)min((unsigned)kJD, nc - t);
-#pragma unroll
-        for (int h = 0; h < kJD / 32; h++) {
-            const int e = lane + 32 * h;
-            if (e < cnt) {
-                const unsigned v = A.cells[co + t + e];
-                sA[w][e] = A.nd_c[v];
-                if (ORDER == 2) {
-                    const double4 q0 = A.nd_q[2 * v], q1 = A.nd_q[2 * v + 1];
-                    sB[w][e] = q0;
-                    sC[w][e] = make_double2(q1.x, q1.y);
-                }
-            }
-        }
-        __syncwarp();
-        cells_tile_d<NI, ORDER>(sA[w], sB[w], sC[w], cnt, xx, xy, xz, pa);
-        __syncwarp();
-    }
-    // near PP segment (changeover and neighbour test per pair), then the far
-    // one (plain Newtonian pairs)
-    for (int seg = 0; seg < 2; seg++) {
-        const unsigned np = seg == 0 ? A.gr_np[g] : A.gr_nf[g];
-        const unsigned long long po = seg == 0 ? A.gr_po[g] : A.gr_fo[g];
-        for (unsigned t = w * kJD; t < np; t += kFWarps * kJD) {
-            const int cnt = (int)min((unsigned)kJD, np - t);
-#pragma unroll
-            for (int h = 0; h < kJD / 32; h++) {
-                const int e = lane + 32 * h;
-                if (e < cnt) {
-                    const unsigned p = A.pp[po + t + e];
-                    sA[w][e] = A.sp64[p];
-                    sI[w][e] = p;
-                    if (MD) sS[w][e] = A.ssc[p];
-                }
-            }
-            __syncwarp();
-            if (seg == 1)
-                pp_tile_d_far<NI>(sA[w], cnt, xx, xy, xz, pa);
-            else if (NB && A.want_nb)
-                pp_tile_d<NI, true, MD>(A, sA[w], sI[w], sS[w], cnt, C, xx, xy, xz, st, pid, valid, pa);
-            else
-                pp_tile_d<NI, false, MD>(A, sA[w], sI[w], sS[w], cnt, C, xx, xy, xz, st, pid, valid, pa);
-            __syncwarp();
-        }
-    }
-#pragma unroll
-    for (int s = 0; s < 2; s++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) red[w][lane + 32 * s][c] = (s < NI) ? pa[s][c] : 0.0;
-}
-
-template <int ORDER, bool NB, bool MD, bool TAIL>
-__global__ void __launch_bounds__(kFThreads) k_force_fp64(ForceArgs A) {
-    __shared__ double4 sA[kFWarps][kJD];
-    __shared__ double4 sB[kFWarps][kJD];
-    __shared__ double2 sC[kFWarps][kJD];
-    __shared__ unsigned sI[kFWarps][kJD];
-    __shared__ double sS[kFWarps][MD ? kJD : 1];
-    __shared__ double red[kFWarps][kSlotMax][4];
-    __shared__ double ered[kFWarps][4];
-    __shared__ unsigned gsh;
-    // lists left unusable by the walk (one-pass arrays exhausted, stack
-    // overflow): do nothing, the host re-runs the walk and the force
-    if (A.st->flags & (kErrListCap | kErrStack)) return;
-    const unsigned ng = A.st->ngroups;
-    for (unsigned it = 0;; it++) {
-        unsigned g;
-        if constexpr (!TAIL) {
-            if (A.direct_groups) {               // one group per CTA
-                if (it > 0 || blockIdx.x >= ng) break;
-                g = blockIdx.x;
-            } else {
-                __syncthreads();
-                if (threadIdx.x == 0) gsh = (unsigned)atomicAdd(&A.st->work[2], 1ull);
-                __syncthreads();
-                g = gsh;
-                if (g >= ng) break;
-            }
-        } else {                                 // see the mixed kernel
-            if (it == 0 && A.direct_groups && blockIdx.x < ng) {
-                g = blockIdx.x;
-            } else {
-                if (A.direct_groups >= ng) break;
-                __syncthreads();
-                if (threadIdx.x == 0) gsh = A.direct_groups + (unsigned)atomicAdd(&A.st->work[2], 1ull);
-                __syncthreads();
-                g = gsh;
-                if (g >= ng) break;
-            }
-        }
-        const uint2 gr = A.gr_r[g];
-        const Chg C = make_chg(A.sets[A.gr_a[g].w]);
-        double ep[4] = {0, 0, 0, 0};
-        for (unsigned i0 = 0; i0 < gr.y; i0 += kIB) {
-            if (gr.y - i0 > 32)
-                group_pass_d<2, ORDER, NB, MD>(A, g, gr, i0, C, sA, sB, sC, sI, (double (*)[kJD])sS, red);
-            else
-                group_pass_d<1, ORDER, NB, MD>(A, g, gr, i0, C, sA, sB, sC, sI, (double (*)[kJD])sS, red);
-            __syncthreads();
-            write_targets(A, gr, i0, kIB, C.c2, red, ep);
-            __syncthreads();
         }
         group_partials(A, g, ep, ered);
     }
@@ -1192,33 +872,24 @@ __global__ void __launch_bounds__(1024) k_group_order(const uint2 *gr_r, unsigne
 // get SMs within a group's time instead of waiting for the whole launch),
 // else a persistent grid that takes groups from an atomic counter.
 template <bool TAIL>
-static void force_launch_t(const ForceArgs &A, int precision, int blocks, cudaStream_t st) {
+static void force_launch_t(const ForceArgs &A, int blocks, cudaStream_t st) {
     const bool md = A.massdep != 0;
-    if (precision == 1) {
-        if (A.order == 2) {
-            if (md) k_force_mixed<2, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-            else k_force_mixed<2, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        } else {
-            if (md) k_force_mixed<0, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-            else k_force_mixed<0, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        }
+    if (A.order == 2) {
+        if (md) k_force_mixed<2, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+        else k_force_mixed<2, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
     } else {
-        if (A.order == 2) {
-            if (md) k_force_fp64<2, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-            else k_force_fp64<2, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        } else {
-            if (md) k_force_fp64<0, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-            else k_force_fp64<0, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        }
+        if (md) k_force_mixed<0, true, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+        else k_force_mixed<0, true, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
     }
 }
 
-int force_launch(const ForceArgs &A, int precision, cudaStream_t st) {
+int force_launch(const ForceArgs &A, int precision, unsigned n, cudaStream_t st) {
     const int blocks = A.direct_groups ? (int)A.direct_groups : sm_count() * 8;
-    if (precision == 1) k_group_order<<<1, 1024, 0, st>>>(A.gr_r, A.gr_ord, A.st);
-    if (A.count_hint && A.direct_groups) force_launch_t<true>(A, precision, blocks, st);
-    else force_launch_t<false>(A, precision, blocks, st);
-    return precision == 1 ? 2 : 1;
+    if (precision != 1) return force64_launch(A, n, blocks, st);
+    k_group_order<<<1, 1024, 0, st>>>(A.gr_r, A.gr_ord, A.st);
+    if (A.count_hint && A.direct_groups) force_launch_t<true>(A, blocks, st);
+    else force_launch_t<false>(A, blocks, st);
+    return 2;
 }
 
 int force_reduce_launch(const ForceArgs &A, cudaStream_t st) {

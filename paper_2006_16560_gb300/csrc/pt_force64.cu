@@ -1,0 +1,589 @@
+// pt_force64.cu -- the float64 force kernel (PT_FP64).
+//
+// GB300 has ~2 float64 lanes per SM and clock against 128 float32 ones, so a
+// kernel that evaluates every pair in float64 instructions is bound by that
+// pipe: 39 (monopole + quadrupole cell) to 22 (particle pair) float64
+// instructions at ~17 cycles per warp each.  Here every pair that is farther
+// apart than its changeover radius -- all cells and all but a few particle
+// pairs -- is evaluated in unevaluated sums of two or three float32 built
+// from error-free transformations (Knuth's TwoSum, Dekker's FastTwoSum, FMA
+// products): ~600 float32 instructions per cell and ~410 per particle pair.
+// Only pairs within r_out, whose changeover and neighbour test are defined in
+// float64 operations, take float64 instructions.
+//
+// Precision.  Coordinates enter as 63-bit fixed point relative to the
+// coordinate origin (exact for |x| >= 2^-9 of the largest coordinate, within
+// 2^-63 of it below), cut into three 21-bit limbs held as float32.  Limb
+// differences are exact, so a pair's separation is correct to ~2^-70 of
+// itself however close the pair is and wherever the group lies.  r^2, 1/r and
+// the products and sums of particle pairs and of short cell lists keep three
+// float32 (~2^-64); in a list of thousands of cells each cell's products keep
+// two and a half (~2^-49, averaged over the list), and a quadrupole term, at
+// most a few percent of its cell's monopole, always two.  The
+// sums are folded into float64 every 64 list entries.  Two float32 throughout
+// (~2^-47 per pair) were measured first: three times faster on the same
+// lists, but with results 2-5 times further from an extended-precision sum
+// than float64 instructions give, and so not used.
+//
+// Lengths are scaled by the power of two at or above the root box side and
+// masses by that of the set's mass, so no power up to r^-5 leaves float32's
+// range whatever the caller's units: separations below 2^-23 box sides go to
+// the float64 path, and accepted cells are at least a grid cell (2^-21) away.
+#include "pt_force.cuh"
+
+namespace pt {
+
+constexpr int kFfTile = 32;        // list entries per warp tile: one gathered by each lane
+constexpr int kFfFold = 2;         // tiles between folds of the float32 sums into float64
+constexpr unsigned kFfFewCells = 2048;   // cell lists below this take the full products (see ff_cells)
+constexpr int kFfQueue = 8;        // near pairs a lane may hold before the warp evaluates them
+constexpr float kFfTinyR2 = 0x1p-46f;   // smallest scaled r^2 evaluated in float32 expansions
+
+struct ff {            // h + l
+    float h, l;
+};
+struct ft {            // h + l + e, |l| <= ulp(h) / 2, e ~ the rounding of l
+    float h, l, e;
+};
+
+__device__ __forceinline__ ff ff_two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ ff ff_fast(float a, float b) {      // |a| >= |b| or a = 0
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ ff ff_prod(float a, float b) {      // exact
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+
+// ---- two float32 (quadrupole terms); low parts are not renormalised
+__device__ __forceinline__ ff ff_mul(ff a, ff b) {
+    const ff p = ff_prod(a.h, b.h);
+    return {p.h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l))};
+}
+__device__ __forceinline__ ff ff_sum3(ff x, ff y, ff z) {
+    const ff s = ff_two_sum(x.h, y.h), t = ff_two_sum(s.h, z.h);
+    return ff_fast(t.h, __fadd_rn(__fadd_rn(__fadd_rn(x.l, y.l), z.l), __fadd_rn(s.l, t.l)));
+}
+
+// ---- three float32
+// product: every rounding of the second word is kept in the third
+__device__ __forceinline__ ft ft_mul_raw(ft a, ft b) {         // h not renormalised against l
+    const ff p = ff_prod(a.h, b.h), q = ff_prod(a.h, b.l), r = ff_prod(a.l, b.h);
+    const ff c = ff_two_sum(q.h, r.h), d = ff_two_sum(p.l, c.h);
+    const float w = __fadd_rn(__fadd_rn(c.l, d.l), __fadd_rn(q.l, r.l));
+    return {p.h, d.h, __fmaf_rn(a.h, b.e, __fmaf_rn(a.e, b.h, __fmaf_rn(a.l, b.l, w)))};
+}
+__device__ __forceinline__ ft ft_mul(ft a, ft b) {
+    const ft x = ft_mul_raw(a, b);
+    const ff s = ff_fast(x.h, x.l);
+    return {s.h, s.l, x.e};
+}
+// the same with the cross terms rounded (~2^-49): cells
+__device__ __forceinline__ ft ft_mul_cell(ft a, ft b) {
+    const ff p = ff_prod(a.h, b.h), d = ff_two_sum(p.l, __fmaf_rn(a.l, b.h, __fmul_rn(a.h, b.l)));
+    const ff s = ff_fast(p.h, d.h);
+    return {s.h, s.l, __fmaf_rn(a.h, b.e, __fmaf_rn(a.e, b.h, __fmaf_rn(a.l, b.l, d.l)))};
+}
+// running sum of x.h + x.l + x.e
+__device__ __forceinline__ void ft_acc(ft &a, ft x) {
+    const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l), u = ff_two_sum(t.h, x.l);
+    a = {s.h, u.h, __fadd_rn(a.e, __fadd_rn(__fadd_rn(t.l, u.l), x.e))};
+}
+// the same with x.l added to the third word (~2^-49 of x): cells
+__device__ __forceinline__ void ft_acc_cell(ft &a, ff x) {
+    const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l);
+    a = {s.h, t.h, __fadd_rn(a.e, __fadd_rn(t.l, x.l))};
+}
+// float32 to float64 on the integer pipe (finite values; subnormals are 0)
+__device__ __forceinline__ double ff_widen(float f) {
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+    return __hiloint2double(e ? (int)hi : 0, e ? (int)(u << 29) : 0);
+}
+
+// Separation of two coordinates from their limbs: the limb differences are
+// exact (each limb is an integer of at most 21 bits in its unit), and each is
+// zero or at least as large as the next (FastTwoSum's condition).
+__device__ __forceinline__ ft ft_sep(float aj, float bj, float cj, float ai, float bi, float ci) {
+    const ff s = ff_fast(__fsub_rn(aj, ai), __fsub_rn(bj, bi)), t = ff_fast(s.l, __fsub_rn(cj, ci));
+    const ff r = ff_fast(s.h, t.h);
+    return {r.h, r.l, t.l};
+}
+
+// dx^2 + dy^2 + dz^2
+__device__ __forceinline__ ft ft_norm2(ft x, ft y, ft z) {
+    const ft d[3] = {x, y, z};
+    ff p[3], c[3];
+    float w[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        p[k] = ff_prod(d[k].h, d[k].h);
+        const float t = __fadd_rn(d[k].h, d[k].h);
+        const ff q = ff_prod(t, d[k].l);
+        c[k] = ff_two_sum(p[k].l, q.h);
+        w[k] = __fadd_rn(c[k].l, __fmaf_rn(t, d[k].e, __fmaf_rn(d[k].l, d[k].l, q.l)));
+    }
+    const ff s = ff_two_sum(p[0].h, p[1].h), t = ff_two_sum(s.h, p[2].h);
+    const ff a = ff_two_sum(c[0].h, c[1].h), b = ff_two_sum(c[2].h, s.l), e = ff_two_sum(a.h, b.h);
+    const ff g = ff_two_sum(e.h, t.l), r = ff_fast(t.h, g.h);
+    return {r.h, r.l, __fadd_rn(__fadd_rn(__fadd_rn(w[0], w[1]), w[2]),
+                                __fadd_rn(__fadd_rn(a.l, b.l), __fadd_rn(e.l, g.l)))};
+}
+
+// 1 / sqrt(r2): the float32 approximation, one float32 Newton step (so that
+// the correction is at most ~2^-24 of the result), then one third-order step
+// on the residual d = 1 - r2 y^2, whose leading part 1 - fl(r2.h y^2) is
+// exact.
+__device__ __forceinline__ ft ft_rsqrt(ft r2) {
+    float y = rsqrtf(r2.h);
+    const float h0 = __fmul_rn(0.5f, y);
+    y = __fmaf_rn(h0, __fmaf_rn(-r2.h, __fmul_rn(y, y), 1.0f), y);
+    const ff q = ff_prod(y, y), p = ff_prod(r2.h, q.h), u = ff_prod(r2.h, q.l), v = ff_prod(r2.l, q.h);
+    const ff g = ff_two_sum(u.h, v.h), k = ff_two_sum(g.h, p.l), d = ff_two_sum(__fsub_rn(1.0f, p.h), -k.h);
+    const float de = __fsub_rn(d.l, __fadd_rn(__fadd_rn(__fadd_rn(g.l, k.l), __fadd_rn(u.l, v.l)),
+                                              __fmaf_rn(r2.l, q.l, __fmul_rn(r2.e, q.h))));
+    const ff l = ff_prod(__fmul_rn(0.5f, y), d.h);
+    const ff r = ff_fast(y, l.h);
+    return {r.h, r.l, __fmaf_rn(__fmul_rn(0.5f, y), de, __fmaf_rn(__fmul_rn(l.h, 0.75f), d.h, l.l))};
+}
+
+// ---------------------------------------------------------------------------
+// Records of the float32 expansions, written once per force call from the
+// sorted float64 arrays (48 B per particle, 96 B per node)
+// ---------------------------------------------------------------------------
+
+// Exponents of a set's units: X = 2^ex above every |coordinate|, lengths in
+// 2^es >= box side (for coincident particles, whose box side is a stand-in,
+// not below 2^(ex - 60): the limbs then stay in range), masses in 2^em.
+struct FfUnits {
+    int ex, es, em;
+};
+__device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M) {
+    double X = S.S * 0x1p-60;
+    for (int d = 0; d < 3; d++) X = fmax(X, fmax(fabs(S.origin[d]), fabs(S.origin[d] + S.S)));
+    FfUnits u;
+    u.ex = ilogb(X) + 1;
+    u.es = max(ilogb(S.S) + 1, u.ex - 60);
+    u.em = M > 0.0 ? ilogb(M) + 1 : 0;
+    return u;
+}
+
+// The three limbs of x in units of 2^es: rounded to a multiple of 2^(ex - 62),
+// then cut 21 bits at a time, each limb rounded to nearest.
+__device__ __forceinline__ void ff_limbs(double x, const FfUnits &u, float &a, float &b, float &c) {
+    const long long f = __double2ll_rn(scalbn(x, 62 - u.ex));
+    const long long ia = (f + (1ll << 41)) >> 42, rem = f - (ia << 42);
+    const long long ib = (rem + (1ll << 20)) >> 21, ic = rem - (ib << 21);
+    const int k = u.ex - u.es;
+    a = scalbnf((float)ia, k - 20);
+    b = scalbnf((float)ib, k - 41);
+    c = scalbnf((float)ic, k - 62);
+}
+
+__device__ __forceinline__ float ff_split(double v, int k, float &h, float &l) {   // returns the third word
+    const double w = scalbn(v, k);
+    h = __double2float_rn(w);
+    l = __double2float_rn(w - (double)h);
+    return __double2float_rn((w - (double)h) - (double)l);
+}
+
+__global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
+    const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
+    for (unsigned p = t0; p < n; p += dt) {
+        const unsigned set = A.sq[p].w;
+        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
+        const double4 P = A.sp64[p];
+        float4 a, b, c;
+        ff_limbs(P.x, u, a.x, b.x, c.x);
+        ff_limbs(P.y, u, a.y, b.y, c.y);
+        ff_limbs(P.z, u, a.z, b.z, c.z);
+        c.w = ff_split(P.w, -u.em, a.w, b.w);
+        A.ffp[3ull * p] = a;
+        A.ffp[3ull * p + 1] = b;
+        A.ffp[3ull * p + 2] = c;
+    }
+    const unsigned nn = A.st->nnodes;
+    for (unsigned v = t0; v < nn; v += dt) {
+        const unsigned set = A.sq[A.nd_r[v].x].w;
+        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
+        const double4 P = A.nd_c[v];
+        float4 a, b, c;
+        ff_limbs(P.x, u, a.x, b.x, c.x);
+        ff_limbs(P.y, u, a.y, b.y, c.y);
+        ff_limbs(P.z, u, a.z, b.z, c.z);
+        c.w = ff_split(P.w, -u.em, a.w, b.w);
+        float4 *o = A.ffn + 6ull * v;
+        o[0] = a;
+        o[1] = b;
+        o[2] = c;
+        if (A.order == 2) {                  // Qxx Qyy Qzz Qxy | their low parts | Qxz, Qyz (high, low)
+            const double4 q0 = A.nd_q[2 * v], q1 = A.nd_q[2 * v + 1];
+            const int k = -u.em - 2 * u.es;
+            ff_split(q0.x, k, a.x, b.x);
+            ff_split(q0.y, k, a.y, b.y);
+            ff_split(q0.z, k, a.z, b.z);
+            ff_split(q0.w, k, a.w, b.w);
+            ff_split(q1.x, k, c.x, c.y);
+            ff_split(q1.y, k, c.z, c.w);
+            o[3] = a;
+            o[4] = b;
+            o[5] = c;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Force kernel
+// ---------------------------------------------------------------------------
+
+struct FfTarget {
+    float ax, ay, az, bx, by, bz, cx, cy, cz;
+};
+
+struct FfGroup {          // per group, formed by one thread
+    float hit2;           // scaled (r_out (1 + 2^-18))^2: a pair at or above it is outside r_out
+    double sa, sp;        // units of acceleration (mass / length^2) and potential (mass / length)
+    double ua, up;        // 1 / sa, 1 / sp
+    Chg C;
+};
+
+// A cell: a += (m/r^3 + 5/2 q/r^5) d - Q u/r^4, P += m/r + 1/2 q/r^3, with
+// u = d/r and q = u.Q.u (the unit-vector form keeps Q's products in range).
+// FULL: the monopole keeps three float32 throughout (short lists, whose few
+// terms do not average the cheaper products' rounding).
+template <int NI, int ORDER, bool FULL>
+__device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int cnt, const FfTarget (&T)[NI],
+                                         ft (&acc)[NI][4]) {
+    for (int j = 0; j < cnt; j++) {
+        const float4 A = sT[0][j], B = sT[1][j], Cc = sT[2][j];
+#pragma unroll
+        for (int k = 0; k < NI; k++) {
+            const ft d[3] = {ft_sep(A.x, B.x, Cc.x, T[k].ax, T[k].bx, T[k].cx),
+                             ft_sep(A.y, B.y, Cc.y, T[k].ay, T[k].by, T[k].cy),
+                             ft_sep(A.z, B.z, Cc.z, T[k].az, T[k].bz, T[k].cz)};
+            const ft ri = ft_rsqrt(ft_norm2(d[0], d[1], d[2]));
+            const ft m = {A.w, B.w, Cc.w};
+            const ft ri2 = FULL ? ft_mul(ri, ri) : ft_mul_cell(ri, ri), mr = FULL ? ft_mul(m, ri) : ft_mul_cell(m, ri);
+            ft f = FULL ? ft_mul(mr, ri2) : ft_mul_cell(mr, ri2), pot = mr;
+            ff w[3];
+            if (ORDER == 2) {
+                const float4 Q = sT[3][j], Ql = sT[4][j], Q2 = sT[5][j];
+                const ff xx = {Q.x, Ql.x}, yy = {Q.y, Ql.y}, zz = {Q.z, Ql.z}, xy = {Q.w, Ql.w};
+                const ff xz = {Q2.x, Q2.y}, yz = {Q2.z, Q2.w};
+                const ff r1 = {ri.h, ri.l}, r2 = {ri2.h, ri2.l};
+                const ff ux = ff_mul({d[0].h, d[0].l}, r1), uy = ff_mul({d[1].h, d[1].l}, r1);
+                const ff uz = ff_mul({d[2].h, d[2].l}, r1);
+                w[0] = ff_sum3(ff_mul(xx, ux), ff_mul(xy, uy), ff_mul(xz, uz));
+                w[1] = ff_sum3(ff_mul(xy, ux), ff_mul(yy, uy), ff_mul(yz, uz));
+                w[2] = ff_sum3(ff_mul(xz, ux), ff_mul(yz, uy), ff_mul(zz, uz));
+                const ff q3 = ff_mul(ff_sum3(ff_mul(ux, w[0]), ff_mul(uy, w[1]), ff_mul(uz, w[2])),
+                                     ff_mul(r2, r1));                        // q / r^3
+                const ff s = ff_two_sum(pot.h, 0.5f * q3.h);
+                const ff v = ff_two_sum(pot.l, __fmaf_rn(0.5f, q3.l, s.l));
+                pot = {s.h, v.h, __fadd_rn(pot.e, v.l)};
+                const ff t = ff_mul(q3, r2);                                 // q / r^5
+                const ff t25 = ff_prod(2.5f, t.h), g = ff_two_sum(f.h, t25.h);
+                const ff z = ff_two_sum(f.l, __fadd_rn(g.l, __fmaf_rn(2.5f, t.l, t25.l)));
+                const ff h = ff_fast(g.h, z.h);
+                f = {h.h, h.l, __fadd_rn(f.e, z.l)};
+                const ff r4 = ff_mul(r2, r2);
+#pragma unroll
+                for (int c = 0; c < 3; c++) w[c] = ff_mul(w[c], r4);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                if (FULL) {
+                    ft x = ft_mul_raw(f, d[c]);
+                    if (ORDER == 2) {
+                        const ff s = ff_two_sum(x.h, -w[c].h), v = ff_two_sum(x.l, __fsub_rn(s.l, w[c].l));
+                        x = {s.h, v.h, __fadd_rn(x.e, v.l)};
+                    }
+                    ft_acc(acc[k][c], x);
+                } else {
+                    const ff p = ff_prod(f.h, d[c].h);
+                    ff x = {p.h, __fmaf_rn(f.l, d[c].h, __fmaf_rn(f.h, d[c].l,
+                                 __fmaf_rn(f.h, d[c].e, __fmaf_rn(f.e, d[c].h, p.l))))};
+                    if (ORDER == 2) {
+                        const ff s = ff_two_sum(p.h, -w[c].h);
+                        x = {s.h, __fadd_rn(x.l, __fsub_rn(s.l, w[c].l))};
+                    }
+                    ft_acc_cell(acc[k][c], x);
+                }
+            }
+            if (FULL) ft_acc(acc[k][3], pot);
+            else ft_acc_cell(acc[k][3], {pot.h, __fadd_rn(pot.l, pot.e)});
+        }
+    }
+}
+
+// The lanes' queued near pairs, one float64 evaluation per lane at a time:
+// neighbour test and changeover (Sec. 6.1, Eqs. 15-17), into the lane's
+// float64 sums.  K = W = 0 beyond r_out, so a pair queued by the conservative
+// float32 bound is exact as well.
+template <int NI, bool MD>
+__device__ __forceinline__ void ff_near(const ForceArgs &A, const FfGroup &G, const unsigned *queue, int &qn,
+                                        const unsigned (&pid)[NI], double (*sD)[4][32]) {
+    const int lane = threadIdx.x & 31;
+    for (int e = 0; __any_sync(0xffffffffu, e < qn); e++) {
+        if (e >= qn) continue;
+        const unsigned code = queue[e * 32 + lane];
+        const int k = NI > 1 ? (int)(code >> 31) : 0;
+        const unsigned pj = code & 0x7fffffffu, pi = NI > 1 && k ? pid[NI - 1] : pid[0];
+        const double4 xi = A.sp64[pi], xj = A.sp64[pj];
+        const double dx = __dsub_rn(xj.x, xi.x), dy = __dsub_rn(xj.y, xi.y), dz = __dsub_rn(xj.z, xi.z);
+        const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+        const Chg &C = G.C;
+        double rout2 = C.rout2, sij = 1.0;
+        if (MD) {                       // pair radii s_ij (r_in, r_out), s_ij = max(s_i, s_j)
+            sij = fmax(A.ssc[pi], A.ssc[pj]);
+            const double ro = __dmul_rn(C.ro, sij);
+            rout2 = __dmul_rn(ro, ro);
+        }
+        if (A.want_nb && r2 < rout2) emit_pair(A, pi, pj);
+        const double r2c = fmax(r2, C.tiny);
+        const double rinv = rsqrt(r2c);
+        const double r = MD ? (r2c * rinv) / sij : r2c * rinv;     // r / s_ij
+        const double xs = fmin(fmax(fma(r, C.invw, C.c0), 0.0), 1.0);
+        const double t = xs - 1.0;
+        const double t2 = t * t;
+        const double kq = fma(fma(fma(fma(35.0 * C.lam, xs, 20.0), xs, 10.0), xs, 4.0), xs, 1.0);
+        const double omk = fma(-t2 * t2, kq, 1.0);
+        const double x2 = xs * xs;
+        const double x5 = x2 * x2 * xs;
+        const double wp = fma(fma(fma(-5.0, xs, 20.0), xs, -28.0), xs, 14.0);
+        const double omw = fmin(fma(-C.lam * x5, wp, r * C.c2), 1.0);
+        const double mr = xj.w * rinv;
+        const double fk = (omk * mr) * (rinv * rinv) * G.ua;
+        sD[k][0][lane] = fma(fk, dx, sD[k][0][lane]);
+        sD[k][1][lane] = fma(fk, dy, sD[k][1][lane]);
+        sD[k][2][lane] = fma(fk, dz, sD[k][2][lane]);
+        sD[k][3][lane] = fma(omw * G.up, mr, sD[k][3][lane]);
+    }
+    qn = 0;
+    __syncwarp();
+}
+
+// Particle pairs outside r_out: a += m d/r^3, P += m/r.  Closer ones (and
+// those below kFfTinyR2) are queued for ff_near and weigh nothing here; the
+// target's own entry is skipped.
+template <int NI, bool MD>
+__device__ __forceinline__ void ff_pairs(const ForceArgs &A, const FfGroup &G, const float4 (*sT)[kFfTile],
+                                         const unsigned *sI, const float *sW, int cnt, const FfTarget (&T)[NI],
+                                         const float (&invs)[NI], const unsigned (&pid)[NI],
+                                         const bool (&valid)[NI], unsigned *queue, int &qn,
+                                         double (*sD)[4][32], ft (&acc)[NI][4]) {
+    const int lane = threadIdx.x & 31;
+    for (int j = 0; j < cnt; j++) {
+        const float4 P = sT[0][j], B = sT[1][j], Cc = sT[2][j];
+        const unsigned pj = sI[j];
+#pragma unroll
+        for (int k = 0; k < NI; k++) {
+            const ft dx = ft_sep(P.x, B.x, Cc.x, T[k].ax, T[k].bx, T[k].cx);
+            const ft dy = ft_sep(P.y, B.y, Cc.y, T[k].ay, T[k].by, T[k].cy);
+            const ft dz = ft_sep(P.z, B.z, Cc.z, T[k].az, T[k].bz, T[k].cz);
+            ft r2 = ft_norm2(dx, dy, dz);
+            float q2 = r2.h;
+            if (MD) {
+                const float w = fminf(invs[k], sW[j]);        // 1 / s_ij
+                q2 *= w * w;
+            }
+            const bool hit = q2 < G.hit2 || r2.h < kFfTinyR2;
+            if (hit && pj != pid[k] && valid[k]) queue[qn++ * 32 + lane] = pj | (k ? 0x80000000u : 0u);
+            r2.h = hit ? 1.0f : r2.h;
+            const ft m = {hit ? 0.0f : P.w, hit ? 0.0f : B.w, hit ? 0.0f : Cc.w};
+            const ft ri = ft_rsqrt(r2);
+            const ft mr = ft_mul(m, ri);
+            const ft f = ft_mul(mr, ft_mul(ri, ri));
+            ft_acc(acc[k][0], ft_mul_raw(f, dx));
+            ft_acc(acc[k][1], ft_mul_raw(f, dy));
+            ft_acc(acc[k][2], ft_mul_raw(f, dz));
+            ft_acc(acc[k][3], mr);
+        }
+        if (__any_sync(0xffffffffu, qn > kFfQueue - NI)) ff_near<NI, MD>(A, G, queue, qn, pid, sD);
+    }
+}
+
+struct FfShared {
+    float4 T[kFWarps][6][kFfTile];
+    unsigned I[kFWarps][kFfTile];
+    float W[kFWarps][kFfTile];             // 1 / s_j (mass-dependent radii)
+    unsigned queue[kFWarps][kFfQueue * 32];
+    double D[kFWarps][2][4][32];           // float64 sums: warp, target of the lane, component, lane
+    double ered[kFWarps][4];
+    FfGroup G;
+    unsigned g;
+};
+
+// One pass over up to 32 NI targets; every warp takes every fourth tile of
+// each list segment.  Leaves the warps' float64 sums in S.D.
+template <int NI, int ORDER, bool MD>
+__device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, FfShared &S) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    FfTarget T[NI];
+    float invs[NI];
+    unsigned pid[NI];
+    bool valid[NI];
+    ft acc[NI][4];
+#pragma unroll
+    for (int k = 0; k < NI; k++) {
+        const unsigned idx = i0 + lane + 32 * k;
+        valid[k] = idx < gr.y;
+        pid[k] = gr.x + (valid[k] ? idx : 0u);
+        const float4 a = A.ffp[3ull * pid[k]], b = A.ffp[3ull * pid[k] + 1], c = A.ffp[3ull * pid[k] + 2];
+        T[k] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z};
+        invs[k] = MD ? A.spL[pid[k]].w : 1.0f;
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[k][q] = {0.0f, 0.0f, 0.0f};
+    }
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) S.D[w][k][q][lane] = 0.0;
+    const FfGroup &G = S.G;
+    auto fold = [&]() {
+#pragma unroll
+        for (int k = 0; k < NI; k++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                S.D[w][k][q][lane] += ff_widen(acc[k][q].h) + (ff_widen(acc[k][q].l) + ff_widen(acc[k][q].e));
+                acc[k][q] = {0.0f, 0.0f, 0.0f};
+            }
+    };
+    int tiles = 0, qn = 0;
+    {
+        const unsigned nc = A.gr_nc[g];
+        const unsigned long long co = A.gr_co[g];
+        for (unsigned t = w * kFfTile; t < nc; t += kFWarps * kFfTile) {
+            const int cnt = (int)min((unsigned)kFfTile, nc - t);
+            if (lane < cnt) {
+                const float4 *o = A.ffn + 6ull * A.cells[co + t + lane];
+#pragma unroll
+                for (int r = 0; r < (ORDER == 2 ? 6 : 3); r++) S.T[w][r][lane] = o[r];
+            }
+            __syncwarp();
+            if (nc < kFfFewCells) ff_cells<NI, ORDER, true>(S.T[w], cnt, T, acc);
+            else ff_cells<NI, ORDER, false>(S.T[w], cnt, T, acc);
+            __syncwarp();
+            if (++tiles % kFfFold == 0) fold();
+        }
+    }
+    // near PP segment, then the far one (whose pairs are all outside r_out)
+    for (int seg = 0; seg < 2; seg++) {
+        const unsigned np = seg == 0 ? A.gr_np[g] : A.gr_nf[g];
+        const unsigned long long po = seg == 0 ? A.gr_po[g] : A.gr_fo[g];
+        for (unsigned t = w * kFfTile; t < np; t += kFWarps * kFfTile) {
+            const int cnt = (int)min((unsigned)kFfTile, np - t);
+            if (lane < cnt) {
+                const unsigned p = A.pp[po + t + lane];
+                S.I[w][lane] = p;
+                if (MD) S.W[w][lane] = A.spL[p].w;
+#pragma unroll
+                for (int r = 0; r < 3; r++) S.T[w][r][lane] = A.ffp[3ull * p + r];
+            }
+            __syncwarp();
+            ff_pairs<NI, MD>(A, G, S.T[w], S.I[w], S.W[w], cnt, T, invs, pid, valid, S.queue[w], qn, S.D[w], acc);
+            __syncwarp();
+            if (++tiles % kFfFold == 0) fold();
+        }
+    }
+    ff_near<NI, MD>(A, G, S.queue[w], qn, pid, S.D[w]);
+    fold();
+}
+
+// Final per-target sums (threads 0..63): fixed-order float64 reduction over
+// the warps, output in caller order.
+__device__ __forceinline__ void ff_write(const ForceArgs &A, const uint2 gr, unsigned i0, const FfShared &S,
+                                         double (&ep)[4]) {
+    const unsigned t = threadIdx.x;
+    if (t < 64 && i0 + t < gr.y) {
+        double s[4] = {0, 0, 0, 0};
+        for (int w = 0; w < kFWarps; w++)
+            for (int c = 0; c < 4; c++) s[c] += S.D[w][t >> 5][c][t & 31];
+        for (int c = 0; c < 4; c++) s[c] *= c < 3 ? S.G.sa : S.G.sp;
+        const unsigned p = gr.x + i0 + t;
+        const double m = A.sp64[p].w;
+        const unsigned i = A.perm[p];
+        const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * s[3];
+        A.acc[3ull * i] = ax;
+        A.acc[3ull * i + 1] = ay;
+        A.acc[3ull * i + 2] = az;
+        A.pot[i] = phi;
+        ep[0] += 0.5 * m * phi;
+        ep[1] += m * ax;
+        ep[2] += m * ay;
+        ep[3] += m * az;
+    }
+}
+
+template <int ORDER, bool MD, bool TAIL>
+__global__ void __launch_bounds__(kFThreads, 4) k_force_ff(ForceArgs A) {
+    __shared__ FfShared S;
+    // lists left unusable by the walk (one-pass arrays exhausted, stack
+    // overflow): do nothing, the host re-runs the walk and the force
+    if (A.st->flags & (kErrListCap | kErrStack)) return;
+    const unsigned ng = A.st->ngroups;
+    for (unsigned it = 0;; it++) {
+        unsigned g;
+        if (TAIL ? (it == 0 && A.direct_groups && blockIdx.x < ng) : A.direct_groups != 0) {
+            if (it > 0 || blockIdx.x >= ng) break;           // one group per CTA
+            g = blockIdx.x;
+        } else {
+            // persistent CTAs, or (a grid sized from a count hint) the groups beyond the grid
+            const unsigned first = TAIL ? A.direct_groups : 0u;
+            if (first >= ng) break;
+            __syncthreads();
+            if (threadIdx.x == 0) S.g = first + (unsigned)atomicAdd(&A.st->work[2], 1ull);
+            __syncthreads();
+            g = S.g;
+            if (g >= ng) break;
+        }
+        const uint2 gr = A.gr_r[g];
+        if (threadIdx.x == 0) {
+            const SetInfo &I = A.sets[A.gr_a[g].w];
+            const FfUnits u = ff_units(I, A.nd_c[A.gr_b[g].w].w);
+            FfGroup G;
+            G.C = make_chg(I);
+            const double h = scalbn(I.r_out, -u.es) * (1.0 + 0x1p-18);
+            G.hit2 = __double2float_ru(fmin(h * h, 1e30));
+            G.sa = scalbn(1.0, u.em - 2 * u.es);
+            G.sp = scalbn(1.0, u.em - u.es);
+            G.ua = scalbn(1.0, 2 * u.es - u.em);
+            G.up = scalbn(1.0, u.es - u.em);
+            S.G = G;
+        }
+        __syncthreads();
+        double ep[4] = {0, 0, 0, 0};
+        for (unsigned i0 = 0; i0 < gr.y; i0 += 64) {
+            if (gr.y - i0 > 32) ff_pass<2, ORDER, MD>(A, g, gr, i0, S);
+            else ff_pass<1, ORDER, MD>(A, g, gr, i0, S);
+            __syncthreads();
+            ff_write(A, gr, i0, S, ep);
+            __syncthreads();
+        }
+        group_partials(A, g, ep, S.ered);
+    }
+}
+
+template <bool TAIL>
+static void force64_t(const ForceArgs &A, int blocks, cudaStream_t st) {
+    if (A.order == 2) {
+        if (A.massdep) k_force_ff<2, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+        else k_force_ff<2, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+    } else {
+        if (A.massdep) k_force_ff<0, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+        else k_force_ff<0, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+    }
+}
+
+int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st) {
+    k_ff_records<<<sm_count() * 8, 256, 0, st>>>(A, n);
+    if (A.count_hint && A.direct_groups) force64_t<true>(A, blocks, st);
+    else force64_t<false>(A, blocks, st);
+    return 2;
+}
+
+}  // namespace pt

@@ -97,6 +97,9 @@ struct ForceArgs {
     const float4 *spH, *spL;
     const double4 *nd_c, *nd_q;
     const float4 *nd_f;
+    const uint2 *nd_r;
+    const uint4 *sq;
+    float4 *ffp, *ffn;               // float64 kernel: double-float records (3 per particle, 6 per node)
     const SetInfo *sets;
     const unsigned *perm;
     const double *ssc;               // sorted radius factors (massdep)
@@ -193,7 +196,8 @@ int ctx_fail(pt_ctx *ctx, int code, const char *msg);
 int walk_warps(unsigned stack_cap);   // warps of a walk launch with this stack size
 constexpr unsigned kWalkSpill = 4096;    // per-warp spill entries of the walk stack (global memory)
 int walk_launch(const WalkArgs &A, int phase, cudaStream_t st);    // 0 count+scan, 1 fill, 2 one pass
-int force_launch(const ForceArgs &A, int precision, cudaStream_t st);
+int force_launch(const ForceArgs &A, int precision, unsigned n, cudaStream_t st);
+int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st);
 constexpr int kRedBlocksMax = 256;    // partial-sum slots of the force's energy / momentum reduction
 int force_reduce_launch(const ForceArgs &A, cudaStream_t st);
 int nb_launch(const NbArgs &A, cudaStream_t st);
