@@ -153,13 +153,14 @@ struct pt_tree {
     std::vector<SetInfo> h_sets;
     // capacities
     unsigned cap_n = 0, cap_nodes = 0, cap_sets = 0;
+    unsigned cap_items = 0, cap_parts = 0;                 // force work items, partial records
     unsigned long long cap_cells = 0, cap_pp = 0, cap_pairs = 0, cap_sort = 0;
     // device buffers
     Buf status, sets, set_of, bmin, bmax, n_dev;
     Buf in_pos, in_mass;                                   // staging for host inputs
     Buf keys_in, vals_in, qbuf, skey, perm, sp64, spH, spL, sq;
     Buf nd_a, nd_b, nd_r, nd_c, nd_q, nd_t, nd_f, nd_bnd, nd_int, topo_bs, tmp_a, tmp_b, lcp;
-    Buf gflag, gbegin, gr_r, gr_a, gr_b, gr_nc, gr_np, gr_co, gr_po, gr_nf, gr_fo, gr_ord, gpart, red_part;
+    Buf gflag, gbegin, gr_r, gr_a, gr_b, gr_nc, gr_np, gr_co, gr_po, gr_nf, gr_fo, gr_wide, gr_pb, items, parts, gpart, red_part;
     Buf cells, pp;
     Buf pairs, nb_keys, nb_keys_s, nb_vals, nb_vals_s, nb_off, nb_idx, npairs_dev;
     Buf sort_k2, sort_v2, sort_counts, scan_sums;
@@ -196,6 +197,8 @@ struct pt_tree {
     // list sizes of the last successful walk of this tree: the one-pass walk
     // sizes its arrays from them (0: no estimate yet, walk in two passes)
     unsigned long long est_cells = 0, est_pp = 0;
+    long long est_extra = -1;                  // force items beyond one per group (-1: no step yet)
+    unsigned est_parts = 0;                    // partial records of its split groups
     unsigned long long chunk_cells = kWalkChunkEntries, chunk_pp = kWalkChunkEntries;
     const double *scale_in = nullptr;          // device radius factors of the current build
     bool built = false, lists_valid = false;
@@ -206,7 +209,7 @@ struct pt_tree {
         Buf *all[] = {&status, &sets, &set_of, &bmin, &bmax, &n_dev, &in_pos, &in_mass, &keys_in,
                       &vals_in, &qbuf, &skey, &perm, &sp64, &spH, &spL, &sq, &nd_a, &nd_b, &nd_r,
                       &nd_c, &nd_q, &nd_t, &nd_f, &nd_bnd, &nd_int, &topo_bs, &tmp_a, &tmp_b, &lcp, &gflag, &gbegin, &gr_r, &gr_a,
-                      &gr_b, &gr_nc, &gr_np, &gr_co, &gr_po, &gr_nf, &gr_fo, &gr_ord, &gpart, &red_part, &cells, &pp, &pairs,
+                      &gr_b, &gr_nc, &gr_np, &gr_co, &gr_po, &gr_nf, &gr_fo, &gr_wide, &gr_pb, &items, &parts, &gpart, &red_part, &cells, &pp, &pairs,
                       &nb_keys, &nb_keys_s, &nb_vals, &nb_vals_s, &nb_off, &nb_idx, &npairs_dev,
                       &sort_k2, &sort_v2, &sort_counts, &scan_sums, &out_acc, &out_pot,
                       &ffp, &ffn, &in_scale, &scale_buf, &set_mean, &ssc, &nd_thr, &gr_thr, &orb_vel, &orb_sv, &orb_rnbf, &walk_spill,
@@ -327,7 +330,8 @@ int alloc_build(pt_tree *t, unsigned n, int nsets) {
     TRY(ensure(ctx, t->gr_np, N * 4));
     TRY(ensure(ctx, t->gr_nf, N * 4));
     TRY(ensure(ctx, t->gr_fo, (N + 1) * 8));
-    TRY(ensure(ctx, t->gr_ord, N * 4));
+    TRY(ensure(ctx, t->gr_pb, N * 8));
+    TRY(ensure(ctx, t->gr_wide, N * 4));
     TRY(ensure(ctx, t->gr_co, (N + 1) * 8));
     TRY(ensure(ctx, t->gr_po, (N + 1) * 8));
     TRY(ensure(ctx, t->gpart, N * 32));
@@ -393,6 +397,7 @@ BuildArgs build_args(pt_tree *t, const double *pos, const double *mass) {
     A.gr_r = t->gr_r.as<uint2>();
     A.gr_a = t->gr_a.as<uint4>();
     A.gr_b = t->gr_b.as<uint4>();
+    A.gr_wide = t->gr_wide.as<unsigned>();
     A.n_leaf = t->prm.n_leaf;
     A.n_group = t->prm.n_group;
     A.scale = t->scale_in;
@@ -493,6 +498,7 @@ WalkArgs walk_args(pt_tree *t) {
     A.gr_r = t->gr_r.as<uint2>();
     A.gr_a = t->gr_a.as<uint4>();
     A.gr_b = t->gr_b.as<uint4>();
+    A.gr_wide = t->gr_wide.as<unsigned>();
     A.sets = t->sets.as<SetInfo>();
     A.nd_thr = t->nd_thr.as<long long>();
     A.gr_thr = t->gr_thr.as<long long>();
@@ -518,6 +524,28 @@ WalkArgs walk_args(pt_tree *t) {
     return A;
 }
 
+// Targets per partial record of a split group (a walk group holds at most
+// n_group particles; larger depth-capped leaves are never split).
+unsigned part_stride(const pt_tree *t) { return (unsigned)std::min(t->prm.n_group, 1 << 16); }
+
+// Room for the force work items: one per group (at most n) and the extra
+// parts of the split groups, as many as the last step's with a quarter and 64
+// head room (before the first: an eighth of the groups).  A step that needs
+// more is flagged (kErrItemCap, with the counts in the status) and repeated.
+// Returns the items of `ngroups` groups in *grid.
+int size_items(pt_tree *t, unsigned ngroups, unsigned *grid) {
+    pt_ctx *ctx = t->ctx;
+    const unsigned long long extra = t->est_extra < 0 ? ngroups / 8 : (unsigned long long)t->est_extra;
+    const unsigned long long parts = t->est_extra < 0 ? ngroups / 4 : t->est_parts;
+    const unsigned long long more = extra + extra / 4 + 64;
+    t->cap_items = (unsigned)std::min<unsigned long long>(t->n + more, 0x7fffffffull);
+    t->cap_parts = (unsigned)std::min<unsigned long long>(parts + parts / 4 + 64, 0x7fffffffull);
+    *grid = (unsigned)std::min<unsigned long long>(ngroups + more, t->cap_items);
+    TRY(ensure(ctx, t->items, (size_t)t->cap_items * 8));
+    TRY(ensure(ctx, t->parts, (size_t)t->cap_parts * part_stride(t) * 32));
+    return PT_OK;
+}
+
 ForceArgs force_args(pt_tree *t, double *acc, double *pot, bool want_nb) {
     ForceArgs A{};
     A.gr_r = t->gr_r.as<uint2>();
@@ -529,7 +557,13 @@ ForceArgs force_args(pt_tree *t, double *acc, double *pot, bool want_nb) {
     A.gr_po = t->gr_po.as<unsigned long long>();
     A.gr_nf = t->gr_nf.as<unsigned>();
     A.gr_fo = t->gr_fo.as<unsigned long long>();
-    A.gr_ord = t->gr_ord.as<unsigned>();
+    A.items = t->items.as<uint2>();
+    A.gr_pb = t->gr_pb.as<uint2>();
+    A.item_bsum = t->topo_bs.as<unsigned>();   // free once the build is done
+    A.parts = t->parts.as<double4>();
+    A.part_stride = part_stride(t);
+    A.item_cap = t->cap_items;
+    A.part_cap = t->cap_parts;
     A.cells = t->cells.as<unsigned>();
     A.pp = t->pp.as<unsigned>();
     A.sp64 = t->sp64.as<double4>();
@@ -624,8 +658,10 @@ int size_onepass(pt_tree *t) {
     t->chunk_pp = granule(t->est_pp);
     const unsigned long long warps =
         std::min<unsigned long long>((unsigned long long)walk_warps(t->walk_stack), ngr);
-    const unsigned long long need_c = t->est_cells + t->est_cells / 4 + warps * t->chunk_cells * 3 / 2;
-    const unsigned long long need_p = t->est_pp + t->est_pp / 4 + warps * t->chunk_pp * 3;
+    // a wide group (walked by its block) takes chunks of its own
+    const unsigned long long wide = t->h.nwide + t->h.nwide / 4ull + 16;
+    const unsigned long long need_c = t->est_cells + t->est_cells / 4 + (warps * 3 / 2 + wide) * t->chunk_cells;
+    const unsigned long long need_p = t->est_pp + t->est_pp / 4 + (warps * 3 + wide * 2) * t->chunk_pp;
     if (need_c > t->cap_cells || !t->cells.p) {
         t->cap_cells = need_c;
         TRY(ensure(ctx, t->cells, t->cap_cells * 4));
@@ -675,21 +711,15 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
     Status *dS = t->status.as<Status>();
     TRY(ensure(ctx, t->nb_off, ((size_t)t->n + 1) * 8));
     TRY(alloc_pairs(t, std::max<unsigned long long>(nb_cap_hint, 2ull * t->n)));
-    bool onepass = t->est_cells > 0 && t->est_pp > 0;
-    for (int attempt = 0; attempt < 6; attempt++) {
-        CK(cudaMemsetAsync(&dS->flags, 0, sizeof(unsigned), st));
-        CK(cudaMemsetAsync(&dS->max_stack, 0, sizeof(unsigned), st));
-        CK(cudaMemsetAsync(&dS->work, 0, sizeof(dS->work), st));
-        CK(cudaMemsetAsync(&dS->npairs, 0, 3 * sizeof(unsigned long long), st));   // npairs, pp_full, pp_fast
-        if (onepass) {
-            TRY(size_onepass(t));
-            CK(cudaMemsetAsync(&dS->cell_total, 0, 2 * sizeof(unsigned long long), st));   // cell, pp totals
-            CK(cudaEventRecord(ctx->ev[2], st));
-            WalkArgs W = walk_args(t);
-            int nk = walk_launch(W, 2, st);
-            CK(cudaEventRecord(ctx->ev[3], st));
+    // force kernel, sums and CSR on the lists of the walk just enqueued (nk
+    // kernels so far), repeated with more room for work items when flagged
+    auto force_stage = [&](int nk) -> int {
+        const unsigned ngroups = t->h.ngroups;         // known since the build's status read
+        for (int k = 0;; k++) {
+            unsigned grid = 0;
+            TRY(size_items(t, ngroups, &grid));
             ForceArgs F = force_args(t, acc, pot, want_nb);
-            F.direct_groups = t->h.ngroups;           // known since the build's status read
+            F.direct_items = F.item_cap = grid;
             nk += force_launch(F, t->prm.precision, t->n, st);
             CK(cudaEventRecord(ctx->ev[4], st));
             TRY(copy_out());
@@ -699,6 +729,30 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             CK(cudaGetLastError());
             CK(cudaEventRecord(ctx->ev[5], st));
             TRY(read_status(t));
+            if (t->h.flags & (kErrStack | kErrListCap)) return PT_OK;     // the walk is repeated
+            t->est_extra = (long long)t->h.nitems - (long long)t->h.ngroups;
+            t->est_parts = t->h.nparts;
+            if (!(t->h.flags & kErrItemCap)) return PT_OK;
+            if (k == 2) return fail(ctx, PT_ERR_INTERNAL, "force work items did not fit after being sized");
+            CK(cudaMemsetAsync(&dS->flags, 0, sizeof(unsigned), st));
+            CK(cudaMemsetAsync(&dS->npairs, 0, 3 * sizeof(unsigned long long), st));
+        }
+    };
+    bool onepass = t->est_cells > 0 && t->est_pp > 0;
+    for (int attempt = 0; attempt < 6; attempt++) {
+        CK(cudaMemsetAsync(&dS->flags, 0, sizeof(unsigned), st));
+        CK(cudaMemsetAsync(&dS->max_stack, 0, sizeof(unsigned), st));
+        CK(cudaMemsetAsync(&dS->wide_next, 0, sizeof(dS->wide_next), st));
+        CK(cudaMemsetAsync(&dS->work, 0, sizeof(dS->work), st));
+        CK(cudaMemsetAsync(&dS->npairs, 0, 3 * sizeof(unsigned long long), st));   // npairs, pp_full, pp_fast
+        if (onepass) {
+            TRY(size_onepass(t));
+            CK(cudaMemsetAsync(&dS->cell_total, 0, 2 * sizeof(unsigned long long), st));   // cell, pp totals
+            CK(cudaEventRecord(ctx->ev[2], st));
+            WalkArgs W = walk_args(t);
+            const int nk = walk_launch(W, 2, st);
+            CK(cudaEventRecord(ctx->ev[3], st));
+            TRY(force_stage(nk));
             const unsigned f = t->h.flags;
             if (f & (kErrStack | kErrListCap)) {
                 if (f & kErrStack) TRY(on_walk_overflow(t));
@@ -737,17 +791,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
         W = walk_args(t);
         nk += walk_launch(W, 1, st);
         CK(cudaEventRecord(ctx->ev[3], st));
-        ForceArgs F = force_args(t, acc, pot, want_nb);
-        F.direct_groups = t->h.ngroups;
-        nk += force_launch(F, t->prm.precision, t->n, st);
-        CK(cudaEventRecord(ctx->ev[4], st));
-        TRY(copy_out());
-        nk += force_reduce_launch(F, st);
-        if (want_nb) nk += nb_launch(nb_args(t), st);
-        t->launches_force = nk;
-        CK(cudaGetLastError());
-        CK(cudaEventRecord(ctx->ev[5], st));
-        TRY(read_status(t));
+        TRY(force_stage(nk));
         const unsigned f = t->h.flags;
         if (f & kErrStack) {                            // cannot happen after the counting pass
             TRY(on_walk_overflow(t));
@@ -873,9 +917,9 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
     nk += walk_launch(W, 2, st);              // one pass (arrays sized before the capture)
     ForceArgs F = force_args(t, t->d_acc.as<double>(), t->d_pot.as<double>(), want_nb);
     // this step's group count is on the device: a grid sized from the last
-    // step's, with head room (groups beyond it are taken from a counter)
-    const unsigned long long hint = t->h.ngroups ? t->h.ngroups + t->h.ngroups / 8 + 64 : 0;
-    F.direct_groups = (unsigned)std::min<unsigned long long>(hint, 0x7fffffffull);
+    // step's, with head room (items beyond it are taken from a counter)
+    const unsigned long long hint = t->h.ngroups ? t->h.ngroups + t->h.ngroups / 8 + 64 + (t->est_extra > 0 ? t->est_extra : 0) : 0;
+    F.direct_items = (unsigned)std::min<unsigned long long>(hint, t->cap_items);
     F.count_hint = 1;
     nk += force_launch(F, t->prm.precision, t->n, st);
     nk += force_reduce_launch(F, st);
@@ -1008,7 +1052,7 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
         const bool pair_short = want_nb && t->h.npairs > t->cap_pairs && t->h.npairs <= nb_hint;
         if (f & (kErrNonFinite | kErrNegMass | kErrBadScale))
             return fail(ctx, PT_ERR_ARG, "non-finite position, negative mass or radius factor not finite and positive");
-        if (!(f & (kErrNodeCap | kErrStack | kErrListCap)) && !pair_short) {
+        if (!(f & (kErrNodeCap | kErrStack | kErrListCap | kErrItemCap)) && !pair_short) {
             done = true;
             cudaEventElapsedTime(&ms[2], ctx->ev[6], ctx->ev[7]);
         } else {
@@ -1056,6 +1100,8 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
                 TRY(alloc_build(t, n, C));
             }
             if (want_nb) TRY(alloc_pairs(t, std::max<unsigned long long>(t->cap_pairs, t->h.npairs * 2 + 1024)));
+            unsigned grid = 0;
+            TRY(size_items(t, t->h.ngroups, &grid));
             if (t->gexec) cudaGraphExecDestroy(t->gexec);
             t->gexec = nullptr;
             const Status keep = t->h;

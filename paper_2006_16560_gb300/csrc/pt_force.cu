@@ -371,7 +371,7 @@ __device__ __forceinline__ float2 ff_sum(float2 a, float2 b) {
 }
 
 template <int NI, int J, int ORDER, bool NB, bool MD>
-__device__ void group_pass_f(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0,
+__device__ void group_pass_f(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, unsigned lo, unsigned hi,
                              const ChgF &C, double rout2, double rout, ulonglong2 (*sP)[5][kJ / 2],
                              unsigned (*sI)[kJ], float2 (*sF)[3][4][32], float2 (*red)[kSlotMax][4]) {
     constexpr int L = 32 / J;
@@ -411,10 +411,13 @@ __device__ void group_pass_f(const ForceArgs &A, unsigned g, const uint2 gr, uns
 #pragma unroll
             for (int c = 0; c < 4; c++) PA[k][c] = 0ull;
         }
-        const unsigned nc = A.gr_nc[g];
+        unsigned cb, ce;
+        seg_range(lo, hi, 0, A.gr_nc[g], cb, ce);
         const unsigned long long co = A.gr_co[g];
-        for (unsigned t = w * kJ; t < nc; t += kFWarps * kJ) {
-            const int cnt = (int)min((unsigned)kJ, nc - t);
+        for (unsigned r = cb; r < ce; r += kFWarps * kJ) {
+            const unsigned q = warp_share<kJ, 2 * J>(ce - r), t = r + w * q;
+            if (t >= ce) break;
+            const int cnt = (int)min(q, ce - t);
             const int cnt2 = (cnt + 2 * J - 1) / (2 * J) * (2 * J);   // <= kJ: kJ is a multiple of 2J
             // lane -> pairs P = lane, lane + 32, ..: entries a = (P / J) 2J + P mod J and
             // b = a + J; each row of a pair is one 128-bit store
@@ -493,10 +496,13 @@ __device__ void group_pass_f(const ForceArgs &A, unsigned g, const uint2 gr, uns
         const unsigned ntarg = min((unsigned)(NI * L), gr.y - i0);   // targets of this pass
         // the near segment (changeover test per iteration), then the far one
         for (int seg = 0; seg < 2; seg++) {
-            const unsigned np = seg == 0 ? A.gr_np[g] : A.gr_nf[g];
+            unsigned pb, pe;
+            seg_range(lo, hi, A.gr_nc[g] + (seg == 0 ? 0u : A.gr_np[g]), seg == 0 ? A.gr_np[g] : A.gr_nf[g], pb, pe);
             const unsigned long long po = seg == 0 ? A.gr_po[g] : A.gr_fo[g];
-            for (unsigned t = w * kJ; t < np; t += kFWarps * kJ) {
-                const int cnt = (int)min((unsigned)kJ, np - t);
+            for (unsigned r = pb; r < pe; r += kFWarps * kJ) {
+                const unsigned q = warp_share<kJ, 2 * J>(pe - r), t = r + w * q;
+                if (t >= pe) break;
+                const int cnt = (int)min(q, pe - t);
                 const int cnt2 = (cnt + 2 * J - 1) / (2 * J) * (2 * J);   // <= kJ: kJ is a multiple of 2J
 #pragma unroll
                 for (int h = 0; h < kJ / 64; h++) {
@@ -576,12 +582,30 @@ __device__ void group_pass_f(const ForceArgs &A, unsigned g, const uint2 gr, uns
         }
 }
 
-// Final per-target sums of the mixed kernel (threads 0..slots-1): the warps'
-// float-float partials added in a fixed order, converted to float64 once;
-// removal of the self entry, output in caller order.
-__device__ __forceinline__ void write_targets_ff(const ForceArgs &A, const uint2 gr, unsigned i0,
-                                                 unsigned slots, double c2, float2 (*red)[kSlotMax][4],
-                                                 double (&ep)[4]) {
+// Results of target p (sorted index) from its sums s, in caller order: the
+// self entry is removed and the energy and momentum terms are added to ep.
+__device__ __forceinline__ void write_target(const ForceArgs &A, unsigned p, double c2, const double (&s)[4],
+                                             double (&ep)[4]) {
+    const double m = A.sp64[p].w;
+    const double P = s[3] - (A.massdep ? m * c2 / A.ssc[p] : m * c2);
+    const unsigned i = A.perm[p];
+    const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * P;
+    A.acc[3ull * i] = ax;
+    A.acc[3ull * i + 1] = ay;
+    A.acc[3ull * i + 2] = az;
+    A.pot[i] = phi;
+    ep[0] += 0.5 * m * phi;
+    ep[1] += m * ax;
+    ep[2] += m * ay;
+    ep[3] += m * az;
+}
+
+// Per-target sums of a pass of the mixed kernel (threads 0..slots-1): the
+// warps' float-float partials added in a fixed order, converted to float64
+// once, then written out or, for one part of several, stored.
+__device__ __forceinline__ void write_targets_ff(const ForceArgs &A, unsigned g, unsigned part, unsigned parts,
+                                                 const uint2 gr, unsigned i0, unsigned slots, double c2,
+                                                 float2 (*red)[kSlotMax][4], double (&ep)[4]) {
     const unsigned t = threadIdx.x;
     if (t < slots && i0 + t < gr.y) {
         double s[4];
@@ -591,19 +615,8 @@ __device__ __forceinline__ void write_targets_ff(const ForceArgs &A, const uint2
             for (int w = 1; w < kFWarps; w++) v = ff_sum(v, red[w][t][c]);
             s[c] = (double)v.x + (double)v.y;
         }
-        const unsigned p = gr.x + i0 + t;
-        const double m = A.sp64[p].w;
-        const double P = s[3] - (A.massdep ? m * c2 / A.ssc[p] : m * c2);
-        const unsigned i = A.perm[p];
-        const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * P;
-        A.acc[3ull * i] = ax;
-        A.acc[3ull * i + 1] = ay;
-        A.acc[3ull * i + 2] = az;
-        A.pot[i] = phi;
-        ep[0] += 0.5 * m * phi;
-        ep[1] += m * ax;
-        ep[2] += m * ay;
-        ep[3] += m * az;
+        if (parts == 1) write_target(A, gr.x + i0 + t, c2, s, ep);
+        else store_part(A, g, part, i0 + t, s);
     }
 }
 
@@ -613,21 +626,21 @@ __device__ __forceinline__ void write_targets_ff(const ForceArgs &A, const uint2
 __device__ __forceinline__ int pass_class(unsigned n) {
     return n > 64 ? 0 : n > 48 ? 1 : n > 32 ? 2 : n > 24 ? 3 : n > 16 ? 4 : 5;
 }
-constexpr int kPassClasses = 6;
+constexpr int kItemClasses = 7;       // split groups, then the six pass classes
 
 // Pass configuration for `rem` remaining targets: returns the slot count and
 // runs the matching instantiation.
 template <int ORDER, bool NB, bool MD>
-__device__ unsigned mixed_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0,
+__device__ unsigned mixed_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, unsigned lo, unsigned hi,
                                const ChgF &C, double rout2, double rout, ulonglong2 (*sP)[5][kJ / 2],
                                unsigned (*sI)[kJ], float2 (*sF)[3][4][32], float2 (*red)[kSlotMax][4]) {
     const unsigned rem = gr.y - i0;
-    if (rem <= 16) { group_pass_f<2, 4, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red); return 16; }
-    if (rem <= 24) { group_pass_f<3, 4, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red); return 24; }
-    if (rem <= 32) { group_pass_f<2, 2, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red); return 32; }
-    if (rem <= 48) { group_pass_f<3, 2, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red); return 48; }
-    if (rem <= 64) { group_pass_f<2, 1, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red); return 64; }
-    group_pass_f<3, 1, ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red);
+    if (rem <= 16) { group_pass_f<2, 4, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red); return 16; }
+    if (rem <= 24) { group_pass_f<3, 4, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red); return 24; }
+    if (rem <= 32) { group_pass_f<2, 2, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red); return 32; }
+    if (rem <= 48) { group_pass_f<3, 2, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red); return 48; }
+    if (rem <= 64) { group_pass_f<2, 1, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red); return 64; }
+    group_pass_f<3, 1, ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red);
     return 96;
 }
 
@@ -645,37 +658,45 @@ __global__ void __launch_bounds__(kFThreads, PT_FORCE_MIN_BLOCKS) k_force_mixed(
     __shared__ double sRout2, sRout, sC2;
     // lists left unusable by the walk (one-pass arrays exhausted, stack
     // overflow): do nothing, the host re-runs the walk and the force
-    if (A.st->flags & (kErrListCap | kErrStack)) return;
-    const unsigned ng = A.st->ngroups;
+    if (A.st->flags & (kErrListCap | kErrStack | kErrItemCap)) return;
+    const unsigned ni = A.st->nitems;
     for (unsigned it = 0;; it++) {
         unsigned gi;
         if constexpr (!TAIL) {
-            if (A.direct_groups) {               // one group per CTA, in group order
-                if (it > 0 || blockIdx.x >= ng) break;
+            if (A.direct_items) {                // one item per CTA, in order
+                if (it > 0 || blockIdx.x >= ni) break;
                 gi = blockIdx.x;
             } else {                             // persistent CTAs
                 __syncthreads();
                 if (threadIdx.x == 0) gsh = (unsigned)atomicAdd(&A.st->work[2], 1ull);
                 __syncthreads();
                 gi = gsh;
-                if (gi >= ng) break;
+                if (gi >= ni) break;
             }
         } else {
-            // the CTA's own group first, then the groups beyond a grid sized
+            // the CTA's own item first, then the items beyond a grid sized
             // from a count hint (a separate instantiation: the loop that may
             // run again compiled the single-set kernel 2.4% slower)
-            if (it == 0 && A.direct_groups && blockIdx.x < ng) {
+            if (it == 0 && A.direct_items && blockIdx.x < ni) {
                 gi = blockIdx.x;
             } else {
-                if (A.direct_groups >= ng) break;
+                if (A.direct_items >= ni) break;
                 __syncthreads();
-                if (threadIdx.x == 0) gsh = A.direct_groups + (unsigned)atomicAdd(&A.st->work[2], 1ull);
+                if (threadIdx.x == 0) gsh = A.direct_items + (unsigned)atomicAdd(&A.st->work[2], 1ull);
                 __syncthreads();
                 gi = gsh;
-                if (gi >= ng) break;
+                if (gi >= ni) break;
             }
         }
-        const unsigned g = A.gr_ord[gi];
+        const uint2 item = A.items[gi];
+        const unsigned g = item.x, part = item.y & 0xffffu, parts = item.y >> 16;
+        unsigned lo = 0, hi = 0xffffffffu;
+        if (parts > 1) {
+            const unsigned S = part_length(A.gr_nc[g] + A.gr_np[g] + A.gr_nf[g],
+                                           part_entries(A.sets[A.gr_a[g].w].n, A.part_shift), kFWarps * kJ);
+            lo = part * S;
+            hi = lo + S;
+        }
         const uint2 gr = A.gr_r[g];
         if (threadIdx.x == 0) {
             const Chg C64 = make_chg(A.sets[A.gr_a[g].w]);
@@ -700,11 +721,19 @@ __global__ void __launch_bounds__(kFThreads, PT_FORCE_MIN_BLOCKS) k_force_mixed(
         const double rout2 = sRout2, rout = sRout, c2 = sC2;
         double ep[4] = {0, 0, 0, 0};
         for (unsigned i0 = 0; i0 < gr.y;) {
-            const unsigned slots = mixed_pass<ORDER, NB, MD>(A, g, gr, i0, C, rout2, rout, sP, sI, sF, red);
+            const unsigned slots = mixed_pass<ORDER, NB, MD>(A, g, gr, i0, lo, hi, C, rout2, rout, sP, sI, sF, red);
             __syncthreads();
-            write_targets_ff(A, gr, i0, slots, c2, red, ep);
+            write_targets_ff(A, g, part, parts, gr, i0, slots, c2, red, ep);
             __syncthreads();
             i0 += slots;
+        }
+        if (parts > 1) {
+            if (!last_part(A, g, parts, &gsh)) continue;
+            for (unsigned t = threadIdx.x; t < gr.y; t += kFThreads) {
+                double s[4];
+                sum_parts(A, g, parts, t, s);
+                write_target(A, gr.x + t, c2, s, ep);
+            }
         }
         group_partials(A, g, ep, ered);
     }
@@ -793,84 +822,122 @@ __global__ void __launch_bounds__(32) k_force_reduce(const double4 *red_e, const
     }
 }
 
-// Order in which the mixed kernel takes the groups: class by class (largest
-// pass configuration first), group order within a class.  Consecutive groups
-// then run the same instantiation, which keeps one code path in the SMs'
-// instruction caches, and the largest groups start first, which shortens the
-// tail of the atomic work queue.  One CTA: thread t classifies a contiguous
-// chunk of groups, a block-wide exclusive scan per class gives each chunk its
-// output positions, and a second pass over the chunk writes them (stable).
-__global__ void __launch_bounds__(1024) k_group_order(const uint2 *gr_r, unsigned *gr_ord,
-                                                      const Status *st) {
-    __shared__ unsigned wsum[32][kPassClasses];
-    __shared__ unsigned base[kPassClasses];
-    const unsigned ng = st->ngroups;
-    const unsigned t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const unsigned per = (ng + 1023) / 1024;
-    const unsigned b = min(t * per, ng), e = min(b + per, ng);
-    unsigned c[kPassClasses], x[kPassClasses];
-#pragma unroll
-    for (int k = 0; k < kPassClasses; k++) c[k] = 0;
-#pragma unroll 4
-    for (unsigned g = b; g < e; g++) {
-        const int k = pass_class(gr_r[g].y);
-#pragma unroll
-        for (int j = 0; j < kPassClasses; j++) c[j] += j == k ? 1u : 0u;   // stays in registers
-    }
-#pragma unroll
-    for (int k = 0; k < kPassClasses; k++) {       // inclusive scan within the warp
-        unsigned v = c[k];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned u = __shfl_up_sync(0xffffffffu, v, d);
-            if (lane >= (unsigned)d) v += u;
-        }
-        x[k] = v;
-        if (lane == 31) wsum[w][k] = v;
+// The force kernels' work items: every group in one part or several (see
+// part_entries), split groups first, then class by class (largest pass
+// configuration first), group order within a class.  Consecutive items then
+// run the same instantiation, which keeps one code path in the SMs'
+// instruction caches, and the longest start first, which shortens the launch's
+// tail.  Two launches over the same even chunks of groups, one per block: the
+// chunk's items per class, then their positions (the classes and blocks
+// before, then a stable rank within the block).  (One CTA for all groups took
+// 87 us for the 20,700 groups of 2^20 particles, these two 8.)
+constexpr int kItemThreads = 256;
+
+// Parts and item class of group g.  A group larger than a partial record (a
+// leaf at the depth limit) is never split, nor is any when the walk left the
+// lists unusable.
+__device__ __forceinline__ unsigned group_parts(const ForceArgs &A, unsigned g, unsigned unit, bool usable, int &cls) {
+    const unsigned n = A.gr_r[g].y, L = A.gr_nc[g] + A.gr_np[g] + A.gr_nf[g];
+    const unsigned most = part_entries(A.sets[A.gr_a[g].w].n, A.part_shift);
+    cls = 1 + pass_class(n);
+    if (L <= most || n > A.part_stride || !usable) return 1u;
+    const unsigned S = part_length(L, most, unit), K = (L + S - 1) / S;
+    if (K > 1) cls = 0;
+    return K;
+}
+
+__device__ __forceinline__ void item_chunk(unsigned ng, unsigned &b, unsigned &e) {
+    const unsigned per = (ng + gridDim.x - 1) / gridDim.x;
+    b = min(blockIdx.x * per, ng);
+    e = min(b + per, ng);
+}
+
+__global__ void __launch_bounds__(kItemThreads) k_items_count(ForceArgs A, unsigned unit, unsigned *bcnt) {
+    __shared__ unsigned sh[kItemClasses];
+    if (threadIdx.x < kItemClasses) sh[threadIdx.x] = 0;
+    __syncthreads();
+    const bool usable = (A.st->flags & (kErrListCap | kErrStack)) == 0;
+    unsigned b, e;
+    item_chunk(A.st->ngroups, b, e);
+    for (unsigned g = b + threadIdx.x; g < e; g += kItemThreads) {
+        int cls;
+        const unsigned K = group_parts(A, g, unit, usable, cls);
+        atomicAdd(&sh[cls], K);
     }
     __syncthreads();
-    if (w == 0) {                                   // inclusive scan over the warps
-        unsigned v[kPassClasses];
-#pragma unroll
-        for (int k = 0; k < kPassClasses; k++) v[k] = wsum[lane][k];
-#pragma unroll
-        for (int k = 0; k < kPassClasses; k++) {
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned u = __shfl_up_sync(0xffffffffu, v[k], d);
-                if (lane >= (unsigned)d) v[k] += u;
-            }
+    if (threadIdx.x < kItemClasses) bcnt[blockIdx.x * kItemClasses + threadIdx.x] = sh[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(kItemThreads) k_items_write(ForceArgs A, unsigned unit, const unsigned *bcnt) {
+    constexpr int kW = kItemThreads / 32;
+    static_assert(kW >= kItemClasses, "one warp per class sums the blocks' counts");
+    __shared__ unsigned tot[kItemClasses], pre[kItemClasses], next[kItemClasses];
+    __shared__ unsigned wcnt[kW][kItemClasses];
+    const unsigned t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (w < kItemClasses) {
+        unsigned all = 0, before = 0;
+        for (unsigned k = lane; k < gridDim.x; k += 32) {
+            const unsigned v = bcnt[k * kItemClasses + w];
+            all += v;
+            before += k < blockIdx.x ? v : 0u;
         }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kPassClasses; k++) wsum[lane][k] = v[k];
+        all = __reduce_add_sync(0xffffffffu, all);
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0) {
+            tot[w] = all;
+            pre[w] = before;
+        }
     }
     __syncthreads();
     if (t == 0) {
         unsigned sum = 0;
-        for (int k = 0; k < kPassClasses; k++) {
-            base[k] = sum;
-            sum += wsum[31][k];
+        for (int k = 0; k < kItemClasses; k++) {
+            next[k] = sum + pre[k];
+            sum += tot[k];
+        }
+        if (blockIdx.x == 0) {
+            A.st->nitems = sum;
+            A.st->nparts = tot[0];
+            if (sum > A.item_cap || tot[0] > A.part_cap) atomicOr(&A.st->flags, kErrItemCap);
         }
     }
-    __syncthreads();
-    unsigned o[kPassClasses];
+    const bool usable = (A.st->flags & (kErrListCap | kErrStack)) == 0;
+    unsigned b, e;
+    item_chunk(A.st->ngroups, b, e);
+    for (unsigned r = b; r < e; r += kItemThreads) {          // uniform across the block
+        const unsigned g = r + t;
+        int cls = -1;
+        const unsigned K = g < e ? group_parts(A, g, unit, usable, cls) : 0u;
+        unsigned rank = 0;
 #pragma unroll
-    for (int k = 0; k < kPassClasses; k++) o[k] = base[k] + (w ? wsum[w - 1][k] : 0u) + x[k] - c[k];
-    for (unsigned g = b; g < e; g++) {
-        const int k = pass_class(gr_r[g].y);
+        for (int j = 1; j < kItemClasses; j++) {
+            const unsigned m = __ballot_sync(0xffffffffu, cls == j);
+            if (cls == j) rank = __popc(m & lanemask_lt());
+            if (lane == 0) wcnt[w][j] = __popc(m);
+        }
+        const unsigned k0 = cls == 0 ? K : 0u, inc = warp_incl_scan(k0);
+        if (cls == 0) rank = inc - k0;
+        if (lane == 31) wcnt[w][0] = inc;
+        __syncthreads();
         unsigned pos = 0;
-#pragma unroll
-        for (int j = 0; j < kPassClasses; j++)      // register-indexed: no local-memory array
-            if (j == k) pos = o[j]++;
-        gr_ord[pos] = g;
+        if (cls >= 0) {
+            pos = next[cls] + rank;
+            for (unsigned k = 0; k < w; k++) pos += wcnt[k][cls];
+            for (unsigned q = 0; q < K; q++)
+                if (pos + q < A.item_cap) A.items[pos + q] = make_uint2(g, q | (K << 16));
+            if (cls == 0) A.gr_pb[g] = make_uint2(pos, 0u);   // class 0 comes first: item index = record index
+        }
+        __syncthreads();
+        if (t < kItemClasses)
+            for (int k = 0; k < kW; k++) next[t] += wcnt[k][t];
+        __syncthreads();
     }
 }
 
-// One CTA per group when the host knows the group count (CTAs then retire
-// group by group, so kernels of other streams -- other batches of a server --
-// get SMs within a group's time instead of waiting for the whole launch),
-// else a persistent grid that takes groups from an atomic counter.
+// One CTA per item when the host has a grid for them (CTAs then retire item
+// by item, so kernels of other streams -- other batches of a server --
+// get SMs within an item's time instead of waiting for the whole launch),
+// else a persistent grid that takes items from an atomic counter.
 template <bool TAIL>
 static void force_launch_t(const ForceArgs &A, int blocks, cudaStream_t st) {
     const bool md = A.massdep != 0;
@@ -883,13 +950,17 @@ static void force_launch_t(const ForceArgs &A, int blocks, cudaStream_t st) {
     }
 }
 
-int force_launch(const ForceArgs &A, int precision, unsigned n, cudaStream_t st) {
-    const int blocks = A.direct_groups ? (int)A.direct_groups : sm_count() * 8;
-    if (precision != 1) return force64_launch(A, n, blocks, st);
-    k_group_order<<<1, 1024, 0, st>>>(A.gr_r, A.gr_ord, A.st);
-    if (A.count_hint && A.direct_groups) force_launch_t<true>(A, blocks, st);
+int force_launch(const ForceArgs &A0, int precision, unsigned n, cudaStream_t st) {
+    ForceArgs A = A0;
+    A.part_shift = precision == 1 ? kPartShiftMixed : kPartShift64;
+    const int blocks = A.direct_items ? (int)A.direct_items : sm_count() * 8;
+    const unsigned unit = precision == 1 ? kFWarps * kJ : kForce64Unit;
+    k_items_count<<<sm_count(), kItemThreads, 0, st>>>(A, unit, A.item_bsum);
+    k_items_write<<<sm_count(), kItemThreads, 0, st>>>(A, unit, A.item_bsum);
+    if (precision != 1) return 2 + force64_launch(A, n, blocks, st);
+    if (A.count_hint && A.direct_items) force_launch_t<true>(A, blocks, st);
     else force_launch_t<false>(A, blocks, st);
-    return 2;
+    return 3;
 }
 
 int force_reduce_launch(const ForceArgs &A, cudaStream_t st) {

@@ -37,6 +37,75 @@ __device__ __forceinline__ Chg make_chg(const SetInfo &S) {
     return c;
 }
 
+// ---------------------------------------------------------------------------
+// Parts: a group whose lists are long for its set is evaluated by several
+// CTAs, each over a range of the concatenated lists (cells, near PP, far PP);
+// the last one to finish adds the partial sums in part order.  One group in a
+// thousand or so sits in the sparse halo with a box that reaches the core and
+// has lists 8 to 16 times the mean; alone it ran as long as the rest of the
+// launch (100,003 Kroupa Plummer particles: 1.1 of 1.1 ms), and a set of a
+// few thousand particles has fewer groups than the GPU has SMs.  The part
+// length depends on the set's own size and on the precision only, so a set's
+// results do not depend on what else is in a batch or on the launch.
+//
+// Entries per part at most: about 1.5 times the mean list at the upper end of
+// each range of set sizes, so that ordinary groups of large sets stay whole
+// (a part costs its targets' loads and a reduction again).  The float64
+// kernel's entries cost ~15 times as much, so its parts are an eighth as long.
+__device__ __forceinline__ unsigned part_entries(unsigned n, unsigned shift) {
+    return (n < 8192u ? 32u : n < 32768u ? 128u : n < 262144u ? 256u : 1024u) << shift;
+}
+constexpr unsigned kPartShiftMixed = 6, kPartShift64 = 3;
+
+// Length of the parts of a list of L entries and their number; parts are
+// multiples of `unit` (one tile of every warp).
+__device__ __forceinline__ unsigned part_length(unsigned L, unsigned most, unsigned unit) {
+    const unsigned k = min((L + most - 1) / most, 0xffffu);
+    return ((L + k - 1) / k + unit - 1) / unit * unit;
+}
+
+// The part of [base, base + len) that lies in [lo, hi), relative to base.
+__device__ __forceinline__ void seg_range(unsigned lo, unsigned hi, unsigned base, unsigned len, unsigned &b,
+                                          unsigned &e) {
+    b = lo > base ? min(lo - base, len) : 0u;
+    e = hi > base ? min(hi - base, len) : 0u;
+}
+
+// Entries each warp takes of the next `left` list entries: a whole tile while
+// every warp can have one, else a quarter, rounded up to `step` (a partial
+// last round left to the first warps costs half a round per list segment on
+// average, 3 to 5% of lists of a few thousand entries).
+template <int TILE, int STEP>
+__device__ __forceinline__ unsigned warp_share(unsigned left) {
+    if (left >= (unsigned)(kFWarps * TILE)) return TILE;
+    return ((left + kFWarps - 1) / kFWarps + STEP - 1) / STEP * STEP;
+}
+
+// A split group: stores the target's partial sums; the part that finishes
+// last returns true in every thread.
+__device__ __forceinline__ void store_part(const ForceArgs &A, unsigned g, unsigned part, unsigned target,
+                                           const double (&s)[4]) {
+    A.parts[(size_t)(A.gr_pb[g].x + part) * A.part_stride + target] = make_double4(s[0], s[1], s[2], s[3]);
+}
+__device__ __forceinline__ bool last_part(const ForceArgs &A, unsigned g, unsigned parts, unsigned *flag) {
+    __threadfence();                     // this thread's partial sums, before the count
+    __syncthreads();
+    if (threadIdx.x == 0) *flag = atomicAdd(&A.gr_pb[g].y, 1u) == parts - 1 ? 1u : 0u;
+    __syncthreads();
+    __threadfence();
+    return *flag != 0;
+}
+__device__ __forceinline__ void sum_parts(const ForceArgs &A, unsigned g, unsigned parts, unsigned target,
+                                          double (&s)[4]) {
+    for (int c = 0; c < 4; c++) s[c] = 0.0;
+    const double4 *p = A.parts + (size_t)A.gr_pb[g].x * A.part_stride + target;
+    for (unsigned k = 0; k < parts; k++, p += A.part_stride) {
+        const double2 u = __ldcg(reinterpret_cast<const double2 *>(p));
+        const double2 v = __ldcg(reinterpret_cast<const double2 *>(p) + 1);
+        s[0] += u.x; s[1] += u.y; s[2] += v.x; s[3] += v.y;
+    }
+}
+
 __device__ __forceinline__ void group_partials(const ForceArgs &A, unsigned g, double (&ep)[4],
                                                double (*ered)[4]) {
     const int w = threadIdx.x >> 5;

@@ -421,7 +421,8 @@ struct FfShared {
 // One pass over up to 32 NI targets; every warp takes every fourth tile of
 // each list segment.  Leaves the warps' float64 sums in S.D.
 template <int NI, int ORDER, bool MD>
-__device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, FfShared &S) {
+__device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, unsigned lo,
+                                        unsigned hi, FfShared &S) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     FfTarget T[NI];
     float invs[NI];
@@ -457,8 +458,12 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
     {
         const unsigned nc = A.gr_nc[g];
         const unsigned long long co = A.gr_co[g];
-        for (unsigned t = w * kFfTile; t < nc; t += kFWarps * kFfTile) {
-            const int cnt = (int)min((unsigned)kFfTile, nc - t);
+        unsigned cb, ce;
+        seg_range(lo, hi, 0, nc, cb, ce);
+        for (unsigned r = cb; r < ce; r += kFWarps * kFfTile) {
+            const unsigned q = warp_share<kFfTile, 1>(ce - r), t = r + w * q;
+            if (t >= ce) break;
+            const int cnt = (int)min(q, ce - t);
             if (lane < cnt) {
                 const float4 *o = A.ffn + 6ull * A.cells[co + t + lane];
 #pragma unroll
@@ -473,10 +478,13 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
     }
     // near PP segment, then the far one (whose pairs are all outside r_out)
     for (int seg = 0; seg < 2; seg++) {
-        const unsigned np = seg == 0 ? A.gr_np[g] : A.gr_nf[g];
+        unsigned pb, pe;
+        seg_range(lo, hi, A.gr_nc[g] + (seg == 0 ? 0u : A.gr_np[g]), seg == 0 ? A.gr_np[g] : A.gr_nf[g], pb, pe);
         const unsigned long long po = seg == 0 ? A.gr_po[g] : A.gr_fo[g];
-        for (unsigned t = w * kFfTile; t < np; t += kFWarps * kFfTile) {
-            const int cnt = (int)min((unsigned)kFfTile, np - t);
+        for (unsigned r = pb; r < pe; r += kFWarps * kFfTile) {
+            const unsigned q = warp_share<kFfTile, 1>(pe - r), t = r + w * q;
+            if (t >= pe) break;
+            const int cnt = (int)min(q, pe - t);
             if (lane < cnt) {
                 const unsigned p = A.pp[po + t + lane];
                 S.I[w][lane] = p;
@@ -494,29 +502,19 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
     fold();
 }
 
-// Final per-target sums (threads 0..63): fixed-order float64 reduction over
-// the warps, output in caller order.
-__device__ __forceinline__ void ff_write(const ForceArgs &A, const uint2 gr, unsigned i0, const FfShared &S,
-                                         double (&ep)[4]) {
-    const unsigned t = threadIdx.x;
-    if (t < 64 && i0 + t < gr.y) {
-        double s[4] = {0, 0, 0, 0};
-        for (int w = 0; w < kFWarps; w++)
-            for (int c = 0; c < 4; c++) s[c] += S.D[w][t >> 5][c][t & 31];
-        for (int c = 0; c < 4; c++) s[c] *= c < 3 ? S.G.sa : S.G.sp;
-        const unsigned p = gr.x + i0 + t;
-        const double m = A.sp64[p].w;
-        const unsigned i = A.perm[p];
-        const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * s[3];
-        A.acc[3ull * i] = ax;
-        A.acc[3ull * i + 1] = ay;
-        A.acc[3ull * i + 2] = az;
-        A.pot[i] = phi;
-        ep[0] += 0.5 * m * phi;
-        ep[1] += m * ax;
-        ep[2] += m * ay;
-        ep[3] += m * az;
-    }
+// Results of target p (sorted index) from its sums, in caller order.
+__device__ __forceinline__ void ff_write(const ForceArgs &A, unsigned p, const double (&s)[4], double (&ep)[4]) {
+    const double m = A.sp64[p].w;
+    const unsigned i = A.perm[p];
+    const double ax = A.G * s[0], ay = A.G * s[1], az = A.G * s[2], phi = -A.G * s[3];
+    A.acc[3ull * i] = ax;
+    A.acc[3ull * i + 1] = ay;
+    A.acc[3ull * i + 2] = az;
+    A.pot[i] = phi;
+    ep[0] += 0.5 * m * phi;
+    ep[1] += m * ax;
+    ep[2] += m * ay;
+    ep[3] += m * az;
 }
 
 template <int ORDER, bool MD, bool TAIL>
@@ -524,22 +522,31 @@ __global__ void __launch_bounds__(kFThreads, 4) k_force_ff(ForceArgs A) {
     __shared__ FfShared S;
     // lists left unusable by the walk (one-pass arrays exhausted, stack
     // overflow): do nothing, the host re-runs the walk and the force
-    if (A.st->flags & (kErrListCap | kErrStack)) return;
-    const unsigned ng = A.st->ngroups;
+    if (A.st->flags & (kErrListCap | kErrStack | kErrItemCap)) return;
+    const unsigned ni = A.st->nitems;
     for (unsigned it = 0;; it++) {
-        unsigned g;
-        if (TAIL ? (it == 0 && A.direct_groups && blockIdx.x < ng) : A.direct_groups != 0) {
-            if (it > 0 || blockIdx.x >= ng) break;           // one group per CTA
-            g = blockIdx.x;
+        unsigned gi;
+        if (TAIL ? (it == 0 && A.direct_items && blockIdx.x < ni) : A.direct_items != 0) {
+            if (it > 0 || blockIdx.x >= ni) break;           // one item per CTA
+            gi = blockIdx.x;
         } else {
-            // persistent CTAs, or (a grid sized from a count hint) the groups beyond the grid
-            const unsigned first = TAIL ? A.direct_groups : 0u;
-            if (first >= ng) break;
+            // persistent CTAs, or (a grid sized from a count hint) the items beyond the grid
+            const unsigned first = TAIL ? A.direct_items : 0u;
+            if (first >= ni) break;
             __syncthreads();
             if (threadIdx.x == 0) S.g = first + (unsigned)atomicAdd(&A.st->work[2], 1ull);
             __syncthreads();
-            g = S.g;
-            if (g >= ng) break;
+            gi = S.g;
+            if (gi >= ni) break;
+        }
+        const uint2 item = A.items[gi];
+        const unsigned g = item.x, part = item.y & 0xffffu, parts = item.y >> 16;
+        unsigned lo = 0, hi = 0xffffffffu;
+        if (parts > 1) {
+            const unsigned len = part_length(A.gr_nc[g] + A.gr_np[g] + A.gr_nf[g],
+                                             part_entries(A.sets[A.gr_a[g].w].n, A.part_shift), kForce64Unit);
+            lo = part * len;
+            hi = lo + len;
         }
         const uint2 gr = A.gr_r[g];
         if (threadIdx.x == 0) {
@@ -557,12 +564,28 @@ __global__ void __launch_bounds__(kFThreads, 4) k_force_ff(ForceArgs A) {
         }
         __syncthreads();
         double ep[4] = {0, 0, 0, 0};
+        const unsigned t = threadIdx.x;
         for (unsigned i0 = 0; i0 < gr.y; i0 += 64) {
-            if (gr.y - i0 > 32) ff_pass<2, ORDER, MD>(A, g, gr, i0, S);
-            else ff_pass<1, ORDER, MD>(A, g, gr, i0, S);
+            if (gr.y - i0 > 32) ff_pass<2, ORDER, MD>(A, g, gr, i0, lo, hi, S);
+            else ff_pass<1, ORDER, MD>(A, g, gr, i0, lo, hi, S);
             __syncthreads();
-            ff_write(A, gr, i0, S, ep);
+            if (t < 64 && i0 + t < gr.y) {                   // fixed-order sums over the warps
+                double s[4] = {0, 0, 0, 0};
+                for (int w = 0; w < kFWarps; w++)
+                    for (int c = 0; c < 4; c++) s[c] += S.D[w][t >> 5][c][t & 31];
+                for (int c = 0; c < 4; c++) s[c] *= c < 3 ? S.G.sa : S.G.sp;
+                if (parts == 1) ff_write(A, gr.x + i0 + t, s, ep);
+                else store_part(A, g, part, i0 + t, s);
+            }
             __syncthreads();
+        }
+        if (parts > 1) {
+            if (!last_part(A, g, parts, &S.g)) continue;
+            for (unsigned k = t; k < gr.y; k += kFThreads) {
+                double s[4];
+                sum_parts(A, g, parts, k, s);
+                ff_write(A, gr.x + k, s, ep);
+            }
         }
         group_partials(A, g, ep, S.ered);
     }
@@ -581,7 +604,7 @@ static void force64_t(const ForceArgs &A, int blocks, cudaStream_t st) {
 
 int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st) {
     k_ff_records<<<sm_count() * 8, 256, 0, st>>>(A, n);
-    if (A.count_hint && A.direct_groups) force64_t<true>(A, blocks, st);
+    if (A.count_hint && A.direct_items) force64_t<true>(A, blocks, st);
     else force64_t<false>(A, blocks, st);
     return 2;
 }

@@ -8,8 +8,9 @@
 //              spL   float4  (lo(x), lo(y), lo(z), 0) 16 B   (float-float)
 //              sq    uint4   (q_x, q_y, q_z, set id)  16 B
 //              skey  u64, perm u32 (sorted slot -> original index)
-//   nodes      nd_a  uint4 (qmin xyz, meta = level | leaf<<5 | nchild<<6)
-//              nd_b  uint4 (qmax xyz, first child)
+//   nodes      nd_a  uint4 (qmin xyz, meta = level | leaf<<5 | nchild<<6
+//                    | a leaf's particle count<<10)
+//              nd_b  uint4 (qmax xyz, first child; a leaf's first particle)
 //              nd_r  uint2 (begin, count)
 //              nd_c  double4 (com xyz, M);  nd_q double4 x 2 (Q xx yy zz xy, xz yz T-trace 0)
 //              nd_f  float4 x 3 (hi(com) M | lo(com) -Qxx | -Qyy -Qxy -Qxz -Qyz), 48 B
@@ -40,6 +41,7 @@ enum : unsigned {
     kErrNegMass = 1u << 5,    // negative mass
     kErrGroupCap = 1u << 6,   // group arrays too small
     kErrBadScale = 1u << 7,   // radius factor not finite and positive
+    kErrItemCap = 1u << 8,    // more force work items or partial records than the launch holds
 };
 
 // Per-set (cluster) table entry.
@@ -59,6 +61,9 @@ struct Status {
     unsigned ngroups;
     unsigned max_level;
     unsigned max_stack;              // deepest walk stack seen (entries per warp)
+    unsigned nitems, nparts;         // force work items, partial records of split groups
+    unsigned nwide;                  // groups walked by whole blocks (listed in gr_wide)
+    unsigned wide_next[2];           // their work counters (counting, filling)
     unsigned pad0;
     unsigned long long cell_total, pp_total;
     unsigned long long cell_inter, pp_inter;
@@ -83,6 +88,15 @@ __host__ __device__ inline unsigned meta_leaf(unsigned m) { return (m >> 5) & 1u
 __host__ __device__ inline unsigned meta_nchild(unsigned m) { return (m >> 6) & 15u; }
 __host__ __device__ inline unsigned make_meta(unsigned level, unsigned leaf, unsigned nchild) {
     return level | (leaf << 5) | (nchild << 6);
+}
+
+// A leaf's particle count in its meta word (from the multipole pass on), so
+// that a walk finds a leaf's range in the two records it has loaded anyway;
+// kMetaManyParticles: that many or more, see nd_r.
+constexpr unsigned kMetaManyParticles = (1u << 22) - 1u;
+__host__ __device__ inline unsigned meta_count(unsigned m) { return m >> 10; }
+__host__ __device__ inline unsigned meta_with_count(unsigned m, unsigned count) {
+    return (m & 0x3ffu) | ((count < kMetaManyParticles ? count : kMetaManyParticles) << 10);
 }
 
 // Order-preserving map of a double to an unsigned 64-bit integer (for

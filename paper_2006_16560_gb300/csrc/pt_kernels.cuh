@@ -14,6 +14,18 @@ constexpr unsigned kOrbitStack = 2048;       // per-warp stack of the orbit-depe
 constexpr unsigned kWalkMaxIters = 1u << 24;   // safety cap on walk iterations per group
 constexpr unsigned long long kWalkChunkEntries = 8192;   // one-pass list allocation granule
 
+// A group is wide when a side of its grid box is at least 2^-kWalkWideShift of
+// the root box: it is listed by the build and walked by a whole block (see
+// pt_walk.cu).  2^-4 finds the groups with many times the mean list (a box
+// that reaches the core from the halo) among about 2% of a Plummer sphere's
+// groups; 2^-5 lists twice as many at the same walk times.  Sets below
+// kWalkWideMin particles have none: their walks take a few dozen steps, and a
+// block's steps cost more than a warp's (1,000 particles: 39 against 32 us).
+constexpr unsigned kWalkWideShift = 4, kWalkWideMin = 2048;
+__device__ __forceinline__ bool walk_wide(const uint4 ga, const uint4 gb, unsigned set_n) {
+    return set_n >= kWalkWideMin && max(max(gb.x - ga.x, gb.y - ga.y), gb.z - ga.z) >= (kGrid >> kWalkWideShift);
+}
+
 struct BuildArgs {
     unsigned n;                      // particles (all sets)
     const unsigned *n_dev;           // device copy of n
@@ -45,6 +57,7 @@ struct BuildArgs {
     unsigned *gflag, *gbegin;        // n each
     uint2 *gr_r;
     uint4 *gr_a, *gr_b;
+    unsigned *gr_wide;               // groups with a wide box, in any order
     int n_leaf, n_group;
     // mass-dependent changeover radii (Eq. 12): per-particle factors in input
     // order (NULL: computed from the masses when massdep, else all 1)
@@ -64,6 +77,7 @@ struct WalkArgs {
     const uint2 *nd_r;
     const uint2 *gr_r;
     const uint4 *gr_a, *gr_b;
+    const unsigned *gr_wide;             // groups walked by whole blocks, in any order
     const SetInfo *sets;
     const long long *nd_thr, *gr_thr;    // per node / group gap thresholds (massdep)
     int massdep;
@@ -91,7 +105,16 @@ struct ForceArgs {
     const unsigned long long *gr_co, *gr_po;
     const unsigned *gr_nf;           // far PP segment (no pair within r_out)
     const unsigned long long *gr_fo;
-    unsigned *gr_ord;                // mixed kernel: group processing order (written per launch)
+    // work items, written per launch by k_items_write in processing order: (group,
+    // part | parts << 16); groups of more than one part also have a slot in gr_pb
+    // (index of their first partial record, parts finished)
+    uint2 *items;
+    uint2 *gr_pb;
+    unsigned *item_bsum;             // items per block and class (8 per SM)
+    double4 *parts;                  // partial sums: part_stride targets per record
+    unsigned part_stride;
+    unsigned item_cap, part_cap;     // items the launch can take, records in parts
+    unsigned part_shift;             // log2 of the part length's unit: see part_entries
     const unsigned *cells, *pp;
     const double4 *sp64;
     const float4 *spH, *spL;
@@ -110,14 +133,15 @@ struct ForceArgs {
     int want_nb;
     uint2 *pairs;                    // (sorted i, sorted j)
     unsigned long long pair_cap;
-    // CTAs of the launch, each first taking the group of its own index: the
-    // group count when the host knows it (after the build), else a hint (a
-    // batch's count from its previous step, with head room: the count is on
-    // the device when a step is enqueued or captured); groups beyond the grid
-    // go to CTAs that take them from an atomic counter.  0: a persistent
-    // launch taking every group from the counter.
-    unsigned direct_groups;
-    unsigned count_hint;             // 1: direct_groups is a hint (take groups beyond it)
+    // CTAs of the launch, each first taking the item of its own index.  The
+    // item count is on the device: a single set's grid holds the group count
+    // (known after the build) and the extra parts of the last step with head
+    // room, and a step that needs more is flagged and repeated; a batch's
+    // grid is a hint from its previous step (count_hint = 1: items beyond
+    // the grid go to CTAs that take them from an atomic counter).  0: a
+    // persistent launch taking every item from the counter.
+    unsigned direct_items;
+    unsigned count_hint;
     double4 *gpart;                  // per group: sum m phi / 2, sum m a
     double4 *red_e;                  // per reduction block: partial sums of gpart
     unsigned long long *red_c;       // per reduction block: cell and PP interaction counts
@@ -197,6 +221,7 @@ int walk_warps(unsigned stack_cap);   // warps of a walk launch with this stack 
 constexpr unsigned kWalkSpill = 4096;    // per-warp spill entries of the walk stack (global memory)
 int walk_launch(const WalkArgs &A, int phase, cudaStream_t st);    // 0 count+scan, 1 fill, 2 one pass
 int force_launch(const ForceArgs &A, int precision, unsigned n, cudaStream_t st);
+constexpr unsigned kForce64Unit = 128;    // list entries of one tile of every warp of the float64 kernel
 int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st);
 constexpr int kRedBlocksMax = 256;    // partial-sum slots of the force's energy / momentum reduction
 int force_reduce_launch(const ForceArgs &A, cudaStream_t st);
