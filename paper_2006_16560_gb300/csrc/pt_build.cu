@@ -274,6 +274,7 @@ __global__ void k_topo_roots(const SetInfo *sets, int nsets, uint4 *nd_a, uint4 
         }
         for (int l = 0; l <= kLevels; l++) st->lvl_int[l] = 0;
         for (int b = 0; b < kLeafBuckets; b++) st->leaf_hist[b] = st->leaf_fill[b] = 0;
+        st->nwide = 0;
     }
 }
 
@@ -577,8 +578,10 @@ __device__ __forceinline__ void leaf_moments(unsigned v, const double4 *sp64, co
                                              uint4 *nd_b, const uint2 *nd_r, double4 *nd_c, double4 *nd_q,
                                              double4 *nd_t, float4 *nd_f, const double *ssc,
                                              const SetInfo *sets, long long *nd_thr) {
-    const uint4 a = nd_a[v], bb = nd_b[v];
+    uint4 a = nd_a[v], bb = nd_b[v];
     const uint2 r = nd_r[v];
+    a.w = meta_with_count(a.w, r.y);
+    bb.w = r.x;
     double s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0}, T[6] = {0, 0, 0, 0, 0, 0}, com[3];
     const double4 p0 = sp64[r.x];
     const uint4 q0 = sq[r.x];
@@ -823,8 +826,8 @@ __global__ void __launch_bounds__(kT) k_group_emit(const unsigned *gflag, const 
 // One warp per group: range, grid box, set, root node, reference point.
 __global__ void __launch_bounds__(kT) k_group_info(const unsigned *gbegin, unsigned n,
                                                    const uint4 *sq, uint2 *gr_r, uint4 *gr_a,
-                                                   uint4 *gr_b, const double *ssc, const SetInfo *sets,
-                                                   long long *gr_thr, const Status *st) {
+                                                   uint4 *gr_b, unsigned *gr_wide, const double *ssc,
+                                                   const SetInfo *sets, long long *gr_thr, Status *st) {
     const unsigned ng = st->ngroups;
     const unsigned lane = threadIdx.x & 31;
     for (unsigned g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < ng;
@@ -851,6 +854,9 @@ __global__ void __launch_bounds__(kT) k_group_info(const unsigned *gbegin, unsig
             gr_r[g] = make_uint2(b, e - b);
             gr_a[g] = make_uint4(mn[0], mn[1], mn[2], set);
             gr_b[g] = make_uint4(mx[0], mx[1], mx[2], set /* root node of the set */);
+            if (walk_wide(make_uint4(mn[0], mn[1], mn[2], 0), make_uint4(mx[0], mx[1], mx[2], 0),
+                          sets[set].n))
+                gr_wide[atomicAdd(&st->nwide, 1u)] = g;
         }
     }
 }
@@ -931,7 +937,7 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     nk++;
     nk += scan_exclusive<unsigned>(A.gflag, A.tmp_u32b, A.n_dev, nullptr, &S->ngroups, A.scan_tmp, st);
     k_group_emit<<<grid_for(n, kT, gmax), kT, 0, st>>>(A.gflag, A.tmp_u32b, n, A.gbegin);
-    k_group_info<<<gmax, kT, 0, st>>>(A.gbegin, n, A.sq, A.gr_r, A.gr_a, A.gr_b, A.ssc, A.sets,
+    k_group_info<<<gmax, kT, 0, st>>>(A.gbegin, n, A.sq, A.gr_r, A.gr_a, A.gr_b, A.gr_wide, A.ssc, A.sets,
                                       A.massdep ? A.gr_thr : nullptr, S);
     nk += 2;
     return nk;

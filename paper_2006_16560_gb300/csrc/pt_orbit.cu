@@ -232,9 +232,9 @@ __global__ void __launch_bounds__(kOrbThreads) k_orbit_search(OrbitArgs A) {
                 }
                 if (gap2 < max(gthr, A.nd_thr[v])) {
                     if (meta_leaf(a.w)) {
-                        const uint2 r = A.nd_r[v];
-                        pbegin = r.x;
-                        pcount = r.y;
+                        pbegin = b.w;
+                        pcount = meta_count(a.w);
+                        if (pcount == kMetaManyParticles) pcount = A.nd_r[v].y;
                     } else {
                         nch = meta_nchild(a.w);
                         first = b.w;

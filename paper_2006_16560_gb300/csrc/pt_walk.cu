@@ -20,7 +20,8 @@
 //   group order.  The arrays are sized from the previous walk of the tree;
 //   if they run out, the kernel flags it and the host falls back to two
 //   passes.
-// Warps take groups from an atomic work counter (persistent grid).
+// Warps take groups from an atomic work counter (persistent grid), after the
+// blocks have taken the wide groups.
 #include "pt_kernels.cuh"
 
 namespace pt {
@@ -54,12 +55,227 @@ __device__ __forceinline__ bool grow_list(unsigned *arr, unsigned long long cap,
     return true;
 }
 
+// What the walk does with a node: accept it as a cell, open it (its children
+// first .. first + nch - 1 go on the stack) or take its particles (pcount from
+// `first`; far: its box is at least r_out from the group's, so it was opened
+// for the opening angle alone).
+struct WalkNode {
+    bool accept = false, far = false;
+    unsigned nch = 0, first = 0, pcount = 0;
+};
+
+template <bool MD>
+__device__ __forceinline__ WalkNode walk_test(const WalkArgs &A, const long long *ithr, const int (&glo)[3],
+                                              const int (&ghi)[3], long long r2thr, unsigned v) {
+    WalkNode N;
+    const uint4 a = A.nd_a[v], b = A.nd_b[v];
+    const unsigned level = meta_level(a.w);
+    const int sh = kBits - (int)level;
+    const unsigned qmn[3] = {a.x, a.y, a.z}, qmx[3] = {b.x, b.y, b.z};
+    long long d2 = 0, gap2 = 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const int p = (int)(qmn[d] >> sh);
+        const int c2 = (2 * p + 1) << sh;          // cube centre, half cells
+        int dd = glo[d] - c2;
+        dd = max(dd, c2 - ghi[d]);
+        dd = max(dd, 0);
+        d2 += (long long)dd * dd;
+        int gg = (int)qmn[d] - (ghi[d] >> 1);      // C.qmin - (G.qmax + 1)
+        gg = max(gg, (glo[d] >> 1) - (int)qmx[d] - 1);
+        gg = max(gg, 0);
+        gap2 += (long long)gg * gg;
+    }
+    // mass-dependent radii: the larger of the group's and the cell's threshold
+    const long long thr = MD ? max(r2thr, A.nd_thr[v]) : r2thr;
+    N.accept = (d2 >= ithr[level]) && (gap2 >= thr);
+    if (!N.accept) {
+        N.first = b.w;
+        if (meta_leaf(a.w)) {
+            N.pcount = meta_count(a.w);
+            if (N.pcount == kMetaManyParticles) N.pcount = A.nd_r[v].y;
+            N.far = gap2 >= thr;
+        } else {
+            N.nch = meta_nchild(a.w);
+        }
+    }
+    return N;
+}
+
+// A wide group (walk_wide) is walked by the whole block, 128 nodes a step: its
+// box reaches far beyond its own neighbourhood, so it may open most of the
+// tree, and one warp then took longer with it than the others with all the
+// other groups (walk of 100,003 Kroupa Plummer particles 0.95 -> 0.42 ms, of
+// 400,000 binary members 1.58 -> 0.74 ms).  Same tests, the stack shared by
+// the block's warps; a step takes fewer nodes when their children might not
+// fit, so the stack never spills.  Not inlined, and short of registers like
+// k_walk itself, whose loop must not spill for it: batched list moves here, or
+// a kernel of 111 registers on a second stream beside k_walk, slowed the
+// ordinary groups' walk of 2^20 particles from 1.55 to 2.8 and 1.8 ms.
+constexpr int kWalkReserve = 7 * kLevels + 6;
+
+struct WalkShared {
+    unsigned cnt[4][kWalkWarps];            // cells, near, far, children per warp
+    unsigned long long chunk;
+    unsigned group;
+};
+
+// As grow_list, by the whole block.
+__device__ __forceinline__ bool grow_list_block(WalkShared &S, unsigned *arr, unsigned long long cap,
+                                                unsigned long long *cursor, unsigned long long &g0,
+                                                unsigned long long &end, unsigned have, unsigned long long need,
+                                                unsigned long long chunk, unsigned *flags) {
+    unsigned long long size = 2 * need;
+    if (size < chunk) size = chunk;
+    if (threadIdx.x == 0) S.chunk = atomicAdd(cursor, size);
+    __syncthreads();
+    const unsigned long long nb = S.chunk;
+    __syncthreads();
+    if (nb + size > cap) {
+        if (threadIdx.x == 0) atomicOr(flags, kErrListCap);
+        return false;
+    }
+    for (unsigned e = threadIdx.x; e < have; e += kWalkThreads) arr[nb + e] = arr[g0 + e];
+    __syncthreads();
+    g0 = nb;
+    end = nb + size;
+    return true;
+}
+
+template <bool FILL, bool MD, bool ONEPASS>
+__device__ __noinline__ void walk_block(const WalkArgs &A, unsigned g, const long long *ithr, unsigned *stk, int cap,
+                                        WalkShared &S) {
+    const unsigned w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint4 ga = A.gr_a[g], gb = A.gr_b[g];
+    const long long r2thr = MD ? A.gr_thr[g] : A.sets[ga.w].r2thr;
+    const int glo[3] = {2 * (int)ga.x, 2 * (int)ga.y, 2 * (int)ga.z};
+    const int ghi[3] = {2 * (int)gb.x + 2, 2 * (int)gb.y + 2, 2 * (int)gb.z + 2};
+    unsigned long long cbase = 0, pbase = 0, fbase = 0, c_end = 0, p_end = 0, f_end = 0;
+    if (!ONEPASS && FILL) {
+        cbase = A.gr_co[g];
+        pbase = A.gr_po[g];
+        fbase = pbase + (A.gr_np[g] - A.gr_nf[g]);
+    }
+    unsigned nc = 0, nn = 0, nf = 0, iters = 0;
+    bool dead = false, overflow = false;
+    __syncthreads();
+    if (threadIdx.x == 0) stk[0] = gb.w;
+    __syncthreads();
+    int sp = 1, max_sp = 1;
+    while (sp > 0) {
+        if (++iters > kWalkMaxIters) {
+            overflow = true;
+            break;
+        }
+        // a node is replaced by at most eight; one at a time, the stack grows
+        // by at most seven per level, which the reserve holds
+        const int k = min(min(sp, kWalkThreads), max(1, (cap - kWalkReserve - sp) / 7));
+        sp -= k;
+        WalkNode N;
+        unsigned v = 0;
+        if ((int)threadIdx.x < k) {
+            v = stk[sp + threadIdx.x];
+            N = walk_test<MD>(A, ithr, glo, ghi, r2thr, v);
+        }
+        const unsigned amask = __ballot_sync(0xffffffffu, N.accept);
+        const unsigned pn = N.far ? 0u : N.pcount, pf = N.far ? N.pcount : 0u;
+        const unsigned nincl = warp_incl_scan(pn), fincl = warp_incl_scan(pf), cincl = warp_incl_scan(N.nch);
+        if (lane == 31) {
+            S.cnt[0][w] = __popc(amask);
+            S.cnt[1][w] = nincl;
+            S.cnt[2][w] = fincl;
+            S.cnt[3][w] = cincl;
+        }
+        __syncthreads();
+        unsigned before[4], tot[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            before[q] = tot[q] = 0;
+#pragma unroll
+            for (unsigned i = 0; i < (unsigned)kWalkWarps; i++) {
+                const unsigned c = S.cnt[q][i];
+                before[q] += i < w ? c : 0u;
+                tot[q] += c;
+            }
+        }
+        if (ONEPASS) {                  // uniform across the block
+            if (tot[0] && !dead && cbase + nc + tot[0] > c_end)
+                dead = !grow_list_block(S, A.cells, A.cap_cells, &A.st->work[0], cbase, c_end, nc, nc + tot[0],
+                                        A.chunk_cells, &A.st->flags);
+            if (tot[1] && !dead && pbase + nn + tot[1] > p_end)
+                dead = !grow_list_block(S, A.pp, A.cap_pp, &A.st->work[3], pbase, p_end, nn, nn + tot[1],
+                                        A.chunk_pp, &A.st->flags);
+            if (tot[2] && !dead && fbase + nf + tot[2] > f_end)
+                dead = !grow_list_block(S, A.pp, A.cap_pp, &A.st->work[3], fbase, f_end, nf, nf + tot[2],
+                                        A.chunk_pp, &A.st->flags);
+        }
+        if (FILL && !dead) {
+            if (N.accept) {
+                const unsigned long long pos = cbase + nc + before[0] + __popc(amask & lanemask_lt());
+                if (pos < A.cap_cells) A.cells[pos] = v;
+                else atomicOr(&A.st->flags, kErrListCap);
+            }
+            if (N.pcount) {
+                const unsigned long long at = N.far ? fbase + nf + before[2] + (fincl - pf)
+                                                    : pbase + nn + before[1] + (nincl - pn);
+                if (at + N.pcount <= A.cap_pp) {
+                    unsigned *to = A.pp + at;
+#pragma unroll 4
+                    for (unsigned e = 0; e < N.pcount; e++) to[e] = N.first + e;
+                } else {
+                    atomicOr(&A.st->flags, kErrListCap);
+                }
+            }
+        }
+        nc += tot[0];
+        nn += tot[1];
+        nf += tot[2];
+        const int at = sp + (int)(before[3] + cincl - N.nch);
+#pragma unroll
+        for (unsigned j = 0; j < 8; j++)
+            if (j < N.nch) stk[at + j] = N.first + j;   // every popped entry has been read
+        sp += (int)tot[3];
+        max_sp = max(max_sp, sp);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        if (overflow) atomicOr(&A.st->flags, kErrStack);
+        if (!FILL || ONEPASS) atomicMax(&A.st->max_stack, (unsigned)max_sp);
+        if (!FILL) {                 // counting pass: gr_np holds the total for the scan
+            A.gr_nc[g] = nc;
+            A.gr_np[g] = nn + nf;
+            A.gr_nf[g] = nf;
+        } else {
+            A.gr_np[g] = nn;
+            A.gr_nf[g] = nf;
+            A.gr_fo[g] = fbase;
+            if (ONEPASS) {
+                A.gr_nc[g] = nc;
+                A.gr_co[g] = cbase;
+                A.gr_po[g] = pbase;
+                atomicAdd(&A.st->cell_total, (unsigned long long)nc);
+                atomicAdd(&A.st->pp_total, (unsigned long long)(nn + nf));
+            }
+        }
+    }
+}
+
 template <bool FILL, bool MD, bool ONEPASS>
 // 14 blocks per SM: the most the small stacks' shared memory allows (32 registers)
 __global__ void __launch_bounds__(kWalkThreads, 14) k_walk(WalkArgs A) {
     extern __shared__ unsigned stack_mem[];      // kWalkWarps x A.stack_cap entries
     __shared__ long long ithr[kLevels];
     if (threadIdx.x < kLevels) ithr[threadIdx.x] = A.wp.ithr[threadIdx.x];
+    __syncthreads();
+    __shared__ WalkShared S;
+    for (const unsigned nwide = A.st->nwide;;) {       // the wide groups first, a block each
+        if (threadIdx.x == 0) S.group = atomicAdd(&A.st->wide_next[FILL ? 1 : 0], 1u);
+        __syncthreads();
+        const unsigned i = S.group;
+        if (i >= nwide) break;
+        walk_block<FILL, MD, ONEPASS>(A, A.gr_wide[i], ithr, stack_mem, (int)(kWalkWarps * A.stack_cap), S);
+        __syncthreads();
+    }
     __syncthreads();
     const unsigned w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned ng = A.st->ngroups;
@@ -81,6 +297,7 @@ __global__ void __launch_bounds__(kWalkThreads, 14) k_walk(WalkArgs A) {
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= ng) break;
         const uint4 ga = A.gr_a[g], gb = A.gr_b[g];
+        if (walk_wide(ga, gb, A.sets[ga.w].n)) continue;
         const long long r2thr = MD ? A.gr_thr[g] : A.sets[ga.w].r2thr;
         const int glo[3] = {2 * (int)ga.x, 2 * (int)ga.y, 2 * (int)ga.z};
         const int ghi[3] = {2 * (int)gb.x + 2, 2 * (int)gb.y + 2, 2 * (int)gb.z + 2};
@@ -122,43 +339,10 @@ __global__ void __launch_bounds__(kWalkThreads, 14) k_walk(WalkArgs A) {
             const bool valid = (int)lane < k;
             const unsigned v = valid ? stk[sp + lane] : 0u;
             __syncwarp();
-            bool accept = false, leaf = false, pfar = false;
-            unsigned nch = 0, first = 0, pcount = 0, pbegin = 0;
-            if (valid) {
-                const uint4 a = A.nd_a[v], b = A.nd_b[v];
-                const unsigned level = meta_level(a.w);
-                const int sh = kBits - (int)level;
-                const unsigned qmn[3] = {a.x, a.y, a.z}, qmx[3] = {b.x, b.y, b.z};
-                long long d2 = 0, gap2 = 0;
-#pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    const int p = (int)(qmn[d] >> sh);
-                    const int c2 = (2 * p + 1) << sh;          // cube centre, half cells
-                    int dd = glo[d] - c2;
-                    dd = max(dd, c2 - ghi[d]);
-                    dd = max(dd, 0);
-                    d2 += (long long)dd * dd;
-                    int gg = (int)qmn[d] - (ghi[d] >> 1);      // C.qmin - (G.qmax + 1)
-                    gg = max(gg, (glo[d] >> 1) - (int)qmx[d] - 1);
-                    gg = max(gg, 0);
-                    gap2 += (long long)gg * gg;
-                }
-                // mass-dependent radii: the larger of the group's and the cell's threshold
-                const long long thr = MD ? max(r2thr, A.nd_thr[v]) : r2thr;
-                accept = (d2 >= ithr[level]) && (gap2 >= thr);
-                leaf = meta_leaf(a.w);
-                if (!accept) {
-                    if (leaf) {
-                        const uint2 r = A.nd_r[v];
-                        pbegin = r.x;
-                        pcount = r.y;
-                        pfar = gap2 >= thr;      // opened for the opening angle only
-                    } else {
-                        nch = meta_nchild(a.w);
-                        first = b.w;
-                    }
-                }
-            }
+            WalkNode N;
+            if (valid) N = walk_test<MD>(A, ithr, glo, ghi, r2thr, v);
+            const bool accept = N.accept, pfar = N.far;
+            const unsigned nch = N.nch, first = N.first, pcount = N.pcount, pbegin = N.first;
             // accepted cells
             const unsigned amask = __ballot_sync(0xffffffffu, accept);
             if (ONEPASS && amask && !dead && cbase + nc + __popc(amask) > c_end)
@@ -203,7 +387,9 @@ __global__ void __launch_bounds__(kWalkThreads, 14) k_walk(WalkArgs A) {
                 // every lane writes its own leaf's particle range at its offset
                 const unsigned long long at = pfar ? fbase + nf + (fincl - pf) : pbase + nn + (nincl - pn);
                 if (at + pcount <= A.cap_pp) {
-                    for (unsigned e = 0; e < pcount; e++) A.pp[at + e] = pbegin + e;
+                    unsigned *to = A.pp + at;
+#pragma unroll 4
+                    for (unsigned e = 0; e < pcount; e++) to[e] = pbegin + e;
                 } else if (pcount) {
                     atomicOr(&A.st->flags, kErrListCap);
                 }
