@@ -186,6 +186,8 @@ struct pt_tree {
     cudaGraphExec_t gbuild = nullptr;
     BuildArgs gbuild_args{}, last_build_args{};
     bool have_last_build = false;
+    int levels = kMaxLevel;                    // deepest level the next build's launches cover
+    int level_margin = 2;                      // levels beyond the last tree's depth
     std::vector<unsigned> gkey_n;
     std::vector<double> gkey_r;
     pt_params gkey_p{};
@@ -400,6 +402,7 @@ BuildArgs build_args(pt_tree *t, const double *pos, const double *mass) {
     A.gr_wide = t->gr_wide.as<unsigned>();
     A.n_leaf = t->prm.n_leaf;
     A.n_group = t->prm.n_group;
+    A.levels = t->levels;
     A.scale = t->scale_in;
     A.massdep = t->prm.mass_dependent;
     A.scale_buf = t->scale_buf.as<double>();
@@ -476,6 +479,11 @@ int run_build(pt_tree *t, const double *pos, const double *mass) {
         if (f & kErrNonFinite) return fail(ctx, PT_ERR_ARG, "non-finite position or mass in the input");
         if (f & kErrNegMass) return fail(ctx, PT_ERR_ARG, "negative mass in the input");
         if (f & kErrBadScale) return fail(ctx, PT_ERR_ARG, "radius factor not finite and positive");
+        if (f & kErrLevels) {                  // deeper than expected: every level now, more room from now on
+            t->levels = kMaxLevel;
+            t->level_margin = std::min(2 * t->level_margin, kMaxLevel);
+            continue;
+        }
         if (f & kErrNodeCap) {
             unsigned long long c = 2ull * t->cap_nodes;
             if (c > 0x7fffffffull) return fail(ctx, PT_ERR_INTERNAL, "tree node count exceeds 2^31");
@@ -483,6 +491,11 @@ int run_build(pt_tree *t, const double *pos, const double *mass) {
             // node arrays are re-allocated for the new capacity by alloc_build
             continue;
         }
+        // the next build's depth, kept while this tree's is near it: a changed
+        // launch sequence is captured again
+        const int depth = (int)t->h.max_level;
+        if (t->levels > depth + 2 * t->level_margin || t->levels < depth + 1)
+            t->levels = std::min(depth + t->level_margin, kMaxLevel);
         t->built = true;
         t->lists_valid = false;
         return PT_OK;
@@ -1052,7 +1065,7 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
         const bool pair_short = want_nb && t->h.npairs > t->cap_pairs && t->h.npairs <= nb_hint;
         if (f & (kErrNonFinite | kErrNegMass | kErrBadScale))
             return fail(ctx, PT_ERR_ARG, "non-finite position, negative mass or radius factor not finite and positive");
-        if (!(f & (kErrNodeCap | kErrStack | kErrListCap | kErrItemCap)) && !pair_short) {
+        if (!(f & (kErrNodeCap | kErrLevels | kErrStack | kErrListCap | kErrItemCap)) && !pair_short) {
             done = true;
             cudaEventElapsedTime(&ms[2], ctx->ev[6], ctx->ev[7]);
         } else {
@@ -1542,6 +1555,8 @@ int pt_orbit_neighbours(pt_tree *t, const double *vel, const pt_orbit_params *op
         A.ctr = t->orb_ctr.as<unsigned long long>();
         A.stack_cap = stack;
         A.cap_nodes = t->cap_nodes;
+        A.max_level = (int)t->h.max_level;
+        A.gr_wide = t->gr_wide.as<unsigned>();
         A.st = dS;
         if (orbit_launch(A, st) < 0) return fail(ctx, PT_ERR_CUDA, "orbit search: kernel attribute refused");
         CK(cudaGetLastError());

@@ -379,13 +379,17 @@ __device__ __forceinline__ void topo_chunk(unsigned cnt, unsigned &k0, unsigned 
 __global__ void __launch_bounds__(kT) k_topo_count(int l, const unsigned long long *skey,
                                                    const unsigned char *lcp, uint4 *nd_a,
                                                    const uint2 *nd_r, unsigned *nch, uint4 *bnd,
-                                                   unsigned *bsum, int n_leaf, unsigned cap,
-                                                   const Status *st) {
+                                                   unsigned *bsum, int n_leaf, int levels, unsigned cap,
+                                                   Status *st) {
     __shared__ unsigned sh[kT / 32];
     unsigned b0, cnt, k0, k1;
     level_range(st, l, cap, b0, cnt);
     topo_chunk(cnt, k0, k1);
-    const bool can_split = l < kMaxLevel;
+    const bool can_split = l < levels;
+    if (l == levels && l < kMaxLevel) {      // the launch ends here: nothing may be left to split
+        for (unsigned k = k0 + threadIdx.x; k < k1; k += blockDim.x)
+            if ((int)nd_r[b0 + k].y > n_leaf) atomicOr(&st->flags, kErrLevels);
+    }
     for (unsigned k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
         const unsigned v = b0 + k;
         const uint2 r = nd_r[v];
@@ -906,11 +910,11 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     nk++;
     k_topo_roots<<<(A.nsets + 127) / 128, 128, 0, st>>>(A.sets, A.nsets, A.nd_a, A.nd_b, A.nd_r, S);
     nk += 2;
-    for (int l = 0; l <= kMaxLevel; l++) {
+    for (int l = 0; l <= A.levels; l++) {
         k_topo_count<<<gmax, kT, 0, st>>>(l, A.skey, A.lcp, A.nd_a, A.nd_r, A.tmp_u32a, A.nd_bnd,
-                                          A.topo_bsum, A.n_leaf, A.cap_nodes, S);
+                                          A.topo_bsum, A.n_leaf, A.levels, A.cap_nodes, S);
         nk++;
-        if (l == kMaxLevel) break;
+        if (l == A.levels) break;
         k_topo_emit<<<gmax, kT, 0, st>>>(l, A.nd_bnd, A.nd_a, A.nd_b, A.nd_r, A.tmp_u32a, A.topo_bsum,
                                          A.nd_int, A.cap_nodes, S);
         nk++;
@@ -928,7 +932,7 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     // ones, and a level's internal nodes are few (the larger grid ran in
     // waves of idle blocks)
     const int mgrid = sm_count() * 2;
-    for (int l = kMaxLevel - 1; l >= 0; l--, nk++)
+    for (int l = A.levels - 1; l >= 0; l--, nk++)
         k_moments_level<<<mgrid, kT, 0, st>>>(l, A.sq, A.nd_a, A.nd_b, A.nd_r, A.nd_c, A.nd_q, A.nd_t,
                                              A.nd_f, A.sets, thr, A.nd_int, A.cap_nodes, S);
     // groups

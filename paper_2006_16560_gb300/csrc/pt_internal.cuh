@@ -41,6 +41,7 @@ enum : unsigned {
     kErrNegMass = 1u << 5,    // negative mass
     kErrGroupCap = 1u << 6,   // group arrays too small
     kErrBadScale = 1u << 7,   // radius factor not finite and positive
+    kErrLevels = 1u << 9,     // a node above n_leaf particles at the deepest level launched
     kErrItemCap = 1u << 8,    // more force work items or partial records than the launch holds
 };
 

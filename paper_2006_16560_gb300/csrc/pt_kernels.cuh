@@ -59,6 +59,10 @@ struct BuildArgs {
     uint4 *gr_a, *gr_b;
     unsigned *gr_wide;               // groups with a wide box, in any order
     int n_leaf, n_group;
+    // deepest level the launch sequence covers (kMaxLevel: every tree): the
+    // depth of the tree's last build and two more, since an empty level still
+    // costs its three kernels; a deeper tree is flagged (kErrLevels)
+    int levels;
     // mass-dependent changeover radii (Eq. 12): per-particle factors in input
     // order (NULL: computed from the masses when massdep, else all 1)
     const double *scale;
@@ -190,6 +194,8 @@ struct OrbitArgs {
     unsigned long long *ctr;             // [0] work counter, [1] candidates
     unsigned stack_cap;
     unsigned cap_nodes;
+    const unsigned *gr_wide;             // wide groups
+    int max_level;                       // deepest level of the tree
     Status *st;
 };
 int orbit_launch(const OrbitArgs &A, cudaStream_t st);
