@@ -122,6 +122,11 @@ __device__ __forceinline__ int orbit_pair(const OrbitArgs &A, unsigned pi, unsig
 }
 
 constexpr int kOrbChunk = 128;     // opened-leaf particles staged per warp
+// Warps that share a wide group (walk_wide: its box overlaps much of the tree,
+// so its members are tested against most of the set): each walks the whole
+// tree and tests every kOrbParts-th staged chunk.  One warp alone took as long
+// as the rest of the search (250,007 Kroupa Plummer particles: 2.85 -> 1.27 ms).
+constexpr unsigned kOrbParts = 16;
 
 // Candidate tests of the staged particles against every member of group g:
 // a float32 prefilter on float-float differences with a 2^-10 margin on
@@ -191,12 +196,19 @@ __global__ void __launch_bounds__(kOrbThreads) k_orbit_search(OrbitArgs A) {
     const unsigned ng = A.st->ngroups;
     unsigned *stk = ostack + (size_t)w * A.stack_cap;
     const int cap = (int)A.stack_cap;
+    // items: kOrbParts parts of every wide group, then the groups
+    const unsigned nparts = A.st->nwide * kOrbParts;
     for (;;) {
-        unsigned g = 0;
-        if (lane == 0) g = (unsigned)atomicAdd(&A.ctr[0], 1ull);
-        g = __shfl_sync(0xffffffffu, g, 0);
-        if (g >= ng) break;
+        unsigned i = 0;
+        if (lane == 0) i = (unsigned)atomicAdd(&A.ctr[0], 1ull);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= nparts + ng) break;
+        const unsigned g = i < nparts ? A.gr_wide[i / kOrbParts] : i - nparts;
         const uint4 ga = A.gr_a[g], gb = A.gr_b[g];
+        if (i >= nparts && walk_wide(ga, gb, A.sets[ga.w].n)) continue;
+        const unsigned part = i < nparts ? i % kOrbParts : 0u;
+        unsigned chunk = 0;          // staged chunks so far (a wide group's part takes every kOrbParts-th)
+        auto mine = [&]() { return i >= nparts || chunk++ % kOrbParts == part; };
         const uint2 gr = A.gr_r[g];
         const long long gthr = A.gr_thr[g];
         unsigned long long ncand = 0;
@@ -267,7 +279,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orbit_search(OrbitArgs A) {
                     done += take;
                     __syncwarp();
                     if (fill == kOrbChunk) {
-                        orbit_chunk(A, gr, fill, cH[w], cL[w], cR[w], cI[w], ncand);
+                        if (mine()) orbit_chunk(A, gr, fill, cH[w], cL[w], cR[w], cI[w], ncand);
                         fill = 0;
                         __syncwarp();
                     }
@@ -284,7 +296,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orbit_search(OrbitArgs A) {
             sp += (int)ctot;
             __syncwarp();
         }
-        if (fill > 0 && !overflow) orbit_chunk(A, gr, fill, cH[w], cL[w], cR[w], cI[w], ncand);
+        if (fill > 0 && !overflow && mine()) orbit_chunk(A, gr, fill, cH[w], cL[w], cR[w], cI[w], ncand);
         __syncwarp();
         ncand = warp_sum(ncand);
         if (lane == 0) {
@@ -301,7 +313,7 @@ int orbit_launch(const OrbitArgs &A, cudaStream_t st) {
         return -1;
     k_orbit_prep<<<sm_count() * 8, 256, 0, st>>>(A);
     int nk = 1;
-    for (int l = kLevels - 1; l >= 0; l--, nk++) k_orbit_nodes<<<sm_count() * 4, 256, 0, st>>>(A, l);
+    for (int l = A.max_level; l >= 0; l--, nk++) k_orbit_nodes<<<sm_count() * 4, 256, 0, st>>>(A, l);
     k_orbit_groups<<<sm_count() * 4, 256, 0, st>>>(A);
     int per_sm = (int)((200u * 1024u) / (smem + 24u * 1024u));
     per_sm = per_sm < 1 ? 1 : (per_sm > 12 ? 12 : per_sm);
