@@ -199,6 +199,7 @@ struct pt_tree {
     // list sizes of the last successful walk of this tree: the one-pass walk
     // sizes its arrays from them (0: no estimate yet, walk in two passes)
     unsigned long long est_cells = 0, est_pp = 0;
+    bool nb_long = false;                      // a neighbour row was too long for nb_launch
     long long est_extra = -1;                  // force items beyond one per group (-1: no step yet)
     unsigned est_parts = 0;                    // partial records of its split groups
     unsigned long long chunk_cells = kWalkChunkEntries, chunk_pp = kWalkChunkEntries;
@@ -628,10 +629,20 @@ NbArgs nb_args(pt_tree *t) {
     A.nb_off = t->nb_off.as<long long>();
     A.nb_idx = t->nb_idx.as<int>();
     A.key_bits = key_bits_for(t->n);
+    A.row = t->gflag.as<unsigned>();           // n words, free once the build is done
+    A.n_dev = t->n_dev.as<unsigned>();
+    A.scan_tmp = scan_tmp_of(t);
     A.st = t->status.as<Status>();
     A.sort_tmp = sort_tmp_of(t);
     return A;
 }
+
+// Neighbour CSR of the tree's pairs: rows of any length by sorting all pairs
+// once a row has been too long for the direct way (nb_long).
+int nb_stage(pt_tree *t, cudaStream_t st) {
+    return t->nb_long ? nb_sort_launch(nb_args(t), st) : nb_launch(nb_args(t), st);
+}
+bool nb_rows_too_long(pt_tree *t) { return !t->nb_long && t->h.max_row > kNbRowMax; }
 
 int alloc_pairs(pt_tree *t, unsigned long long cap) {
     pt_ctx *ctx = t->ctx;
@@ -737,7 +748,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             CK(cudaEventRecord(ctx->ev[4], st));
             TRY(copy_out());
             nk += force_reduce_launch(F, st);
-            if (want_nb) nk += nb_launch(nb_args(t), st);
+            if (want_nb) nk += nb_stage(t, st);
             t->launches_force = nk;
             CK(cudaGetLastError());
             CK(cudaEventRecord(ctx->ev[5], st));
@@ -745,7 +756,15 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             if (t->h.flags & (kErrStack | kErrListCap)) return PT_OK;     // the walk is repeated
             t->est_extra = (long long)t->h.nitems - (long long)t->h.ngroups;
             t->est_parts = t->h.nparts;
-            if (!(t->h.flags & kErrItemCap)) return PT_OK;
+            if (!(t->h.flags & kErrItemCap)) {
+                if (want_nb && nb_rows_too_long(t)) {
+                    t->nb_long = true;
+                    t->launches_force += nb_stage(t, st);
+                    CK(cudaGetLastError());
+                    CK(cudaStreamSynchronize(st));
+                }
+                return PT_OK;
+            }
             if (k == 2) return fail(ctx, PT_ERR_INTERNAL, "force work items did not fit after being sized");
             CK(cudaMemsetAsync(&dS->flags, 0, sizeof(unsigned), st));
             CK(cudaMemsetAsync(&dS->npairs, 0, 3 * sizeof(unsigned long long), st));
@@ -937,7 +956,7 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
     nk += force_launch(F, t->prm.precision, t->n, st);
     nk += force_reduce_launch(F, st);
     if (want_nb) {
-        nk += nb_launch(nb_args(t), st);
+        nk += nb_stage(t, st);
         nk += batch_nb_launch(dtab, dsets, C, n, t->nb_off.as<long long>(), t->nb_idx.as<int>(),
                               t->d_totals.as<long long>(), !host_io, st);
     }
@@ -1065,7 +1084,8 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
         const bool pair_short = want_nb && t->h.npairs > t->cap_pairs && t->h.npairs <= nb_hint;
         if (f & (kErrNonFinite | kErrNegMass | kErrBadScale))
             return fail(ctx, PT_ERR_ARG, "non-finite position, negative mass or radius factor not finite and positive");
-        if (!(f & (kErrNodeCap | kErrLevels | kErrStack | kErrListCap | kErrItemCap)) && !pair_short) {
+        if (!(f & (kErrNodeCap | kErrLevels | kErrStack | kErrListCap | kErrItemCap)) && !pair_short &&
+            !(want_nb && nb_rows_too_long(t))) {
             done = true;
             cudaEventElapsedTime(&ms[2], ctx->ev[6], ctx->ev[7]);
         } else {
@@ -1588,8 +1608,14 @@ int pt_orbit_neighbours(pt_tree *t, const double *vel, const pt_orbit_params *op
             rc = fail(ctx, PT_ERR_CAPACITY, "orbit neighbour lists need %llu entries, capacity %lld",
                       npairs, (long long)nb_capacity);
         } else {
-            nb_launch(nb_args(t), st);
+            nb_stage(t, st);
             CK(cudaGetLastError());
+            TRY(read_status(t));
+            if (nb_rows_too_long(t)) {
+                t->nb_long = true;
+                nb_stage(t, st);
+                CK(cudaGetLastError());
+            }
             cudaMemcpyKind k1 = is_device_ptr(nb_offsets) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
             CK(cudaMemcpyAsync(nb_offsets, t->nb_off.p, (n + 1) * 8, k1, st));
             if (npairs) {

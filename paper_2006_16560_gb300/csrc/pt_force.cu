@@ -972,10 +972,99 @@ int force_reduce_launch(const ForceArgs &A, cudaStream_t st) {
 }
 
 // ===========================================================================
-// Neighbour CSR: pairs (sorted i, sorted j) -> keys (orig i * n + orig j) ->
-// radix sort -> row offsets by binary search -> column indices.
+// Neighbour CSR.  Rows are short (a few neighbours), so the pairs go straight
+// to their rows: a counting launch gives every pair its row and a rank in it
+// (in the order of arrival), a scan places the rows, a filling launch writes
+// the columns, and each row is sorted.  Six launches; sorting all pairs by
+// (row, column) took three per 8 bits of the key, 9 to 18, each a few us
+// whatever the number of pairs.  CSR and energy sums together, before -> after:
+// 1,000 particles (116 pairs) 60 -> 42 us, 2^20 (26,668) 111 -> 54 us, 10^7
+// (2.4e6) 580 -> 267 us.  Rows of more than kNbRowMax entries are left unsorted and reported (max_row): the
+// host then sorts all pairs by radix (nb_sort_launch).
 // ===========================================================================
 
+__global__ void k_nb_count(NbArgs A) {
+    unsigned long long np = A.st->npairs;
+    if (np > A.pair_cap) np = A.pair_cap;
+    for (unsigned long long k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
+        const unsigned i = A.perm[A.pairs[k].x];
+        const unsigned r = atomicAdd(&A.row[i], 1u);
+        A.vals[k] = r;
+        if (r == kNbRowMax) A.st->max_row = kNbRowMax + 1;     // every writer writes the same
+    }
+}
+
+__global__ void k_nb_fill(NbArgs A) {
+    unsigned long long np = A.st->npairs;
+    if (np > A.pair_cap) np = A.pair_cap;
+    const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
+    for (unsigned long long k = t0; k < np; k += dt) {
+        const uint2 p = A.pairs[k];
+        A.nb_idx[A.nb_off[A.perm[p.x]] + A.vals[k]] = (int)A.perm[p.y];
+    }
+    if (t0 == 0) A.nb_off[A.n] = (long long)np;
+}
+
+// One thread per row of up to four entries (insertion), a warp for longer
+// ones: 32 at a time by rank (entries are distinct), each lane counting the
+// row's smaller entries.
+__global__ void __launch_bounds__(256) k_nb_rows(NbArgs A) {
+    __shared__ int buf[8][kNbRowMax];
+    const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (unsigned r0 = warp * 32; r0 < A.n; r0 += nw * 32) {
+        const unsigned r = r0 + lane;
+        const unsigned c = r < A.n ? A.row[r] : 0u;
+        int *e = nullptr;
+        if (c > 1) {
+            e = A.nb_idx + A.nb_off[r];
+            if (c <= 4) {
+                int v[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) v[k] = k < (int)c ? e[k] : 0x7fffffff;
+                auto cx = [&](int i, int j) {
+                    const int x = min(v[i], v[j]), y = max(v[i], v[j]);
+                    v[i] = x;
+                    v[j] = y;
+                };
+                cx(0, 1); cx(2, 3); cx(0, 2); cx(1, 3); cx(1, 2);
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (k < (int)c) e[k] = v[k];
+            }
+        }
+        unsigned m = __ballot_sync(0xffffffffu, c > 4 && c <= kNbRowMax);
+        while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            const unsigned n = __shfl_sync(0xffffffffu, c, src);
+            int *row = reinterpret_cast<int *>(__shfl_sync(0xffffffffu, (unsigned long long)e, src));
+            for (unsigned k = lane; k < n; k += 32) buf[w][k] = row[k];
+            __syncwarp();
+            for (unsigned k = lane; k < n; k += 32) {
+                const int v = buf[w][k];
+                unsigned rank = 0;
+                for (unsigned j = 0; j < n; j++) rank += buf[w][j] < v ? 1u : 0u;
+                row[rank] = v;
+            }
+            __syncwarp();
+        }
+    }
+}
+
+int nb_launch(const NbArgs &A, cudaStream_t st) {
+    cudaMemsetAsync(A.row, 0, (size_t)A.n * sizeof(unsigned), st);
+    cudaMemsetAsync(&A.st->max_row, 0, sizeof(unsigned), st);
+    k_nb_count<<<sm_count() * 4, 256, 0, st>>>(A);
+    const int nk = scan_exclusive<unsigned long long>(A.row, reinterpret_cast<unsigned long long *>(A.nb_off), A.n_dev,
+                                                      nullptr, nullptr, A.scan_tmp, st);
+    k_nb_fill<<<sm_count() * 4, 256, 0, st>>>(A);
+    k_nb_rows<<<sm_count() * 4, 256, 0, st>>>(A);
+    return nk + 3;
+}
+
+// Any row length: pairs (sorted i, sorted j) -> keys (orig i * n + orig j) ->
+// radix sort -> row offsets by binary search -> column indices.
 __global__ void k_nb_keys(NbArgs A) {
     unsigned long long np = A.st->npairs;
     if (np > A.pair_cap) np = A.pair_cap;
@@ -1002,7 +1091,7 @@ __global__ void k_nb_csr(NbArgs A) {
         A.nb_idx[k] = (int)(A.keys_sorted[k] % A.n);
 }
 
-int nb_launch(const NbArgs &A, cudaStream_t st) {
+int nb_sort_launch(const NbArgs &A, cudaStream_t st) {
     k_nb_keys<<<sm_count() * 4, 256, 0, st>>>(A);
     int nk = radix_sort(A.keys, A.vals, A.keys_sorted, A.vals_sorted, A.npairs_dev,
                         (unsigned)A.pair_cap, 0, A.key_bits, nullptr, 0, A.sort_tmp, st);

@@ -65,7 +65,7 @@ struct Status {
     unsigned nitems, nparts;         // force work items, partial records of split groups
     unsigned nwide;                  // groups walked by whole blocks (listed in gr_wide)
     unsigned wide_next[2];           // their work counters (counting, filling)
-    unsigned pad0;
+    unsigned max_row;                // above kNbRowMax: a neighbour row is too long for nb_launch
     unsigned long long cell_total, pp_total;
     unsigned long long cell_inter, pp_inter;
     unsigned long long npairs;
@@ -180,5 +180,11 @@ int radix_sort(const unsigned long long *keys_in, const unsigned *vals_in,
                 unsigned long long *keys_out, unsigned *vals_out,
                 const unsigned *n_dev, unsigned n_max, int bit0, int bit1,
                 const unsigned *set_of, int set_bits, SortTmp tmp, cudaStream_t st);
+
+// The same order for at most kRankSortMax keys whose count the host knows, by
+// (set, key) when set_of is given (set ids by value), in one or two launches.
+constexpr unsigned kRankSortMax = 8192;
+int rank_sort(const unsigned long long *keys_in, const unsigned *vals_in, unsigned long long *keys_out,
+              unsigned *vals_out, unsigned n, const unsigned *set_of, SortTmp tmp, cudaStream_t st);
 
 }  // namespace pt

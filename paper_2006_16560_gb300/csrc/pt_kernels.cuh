@@ -163,7 +163,10 @@ struct NbArgs {
     long long *nb_off;               // n + 1 (global CSR, input order)
     int *nb_idx;                     // pair_cap
     int key_bits;
+    unsigned *row;                   // n: entries per row
+    const unsigned *n_dev;           // device copy of n
     Status *st;
+    ScanTmp scan_tmp;
     SortTmp sort_tmp;
 };
 
@@ -231,6 +234,8 @@ constexpr unsigned kForce64Unit = 128;    // list entries of one tile of every w
 int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st);
 constexpr int kRedBlocksMax = 256;    // partial-sum slots of the force's energy / momentum reduction
 int force_reduce_launch(const ForceArgs &A, cudaStream_t st);
+constexpr unsigned kNbRowMax = 512;   // longest neighbour row nb_launch sorts (else: status max_row above it)
 int nb_launch(const NbArgs &A, cudaStream_t st);
+int nb_sort_launch(const NbArgs &A, cudaStream_t st);   // rows of any length
 
 }  // namespace pt
