@@ -901,8 +901,11 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     if (A.nsets > 1) {
         while ((1 << set_bits) < A.nsets) set_bits++;
     }
-    nk += radix_sort(A.keys_in, A.vals_in, A.skey, A.perm, A.n_dev, n, 0, 3 * kBits, set_of,
-                     set_bits, A.sort_tmp, st);
+    if (n <= kRankSortMax)
+        nk += rank_sort(A.keys_in, A.vals_in, A.skey, A.perm, n, set_of, A.sort_tmp, st);
+    else
+        nk += radix_sort(A.keys_in, A.vals_in, A.skey, A.perm, A.n_dev, n, 0, 3 * kBits, set_of,
+                         set_bits, A.sort_tmp, st);
     k_gather<<<grid_for(n, kT, gmax), kT, 0, st>>>(A.pos, A.mass, n, A.perm, A.qbuf, scale, A.ssc,
                                                    A.sp64, A.spH, A.spL, A.sq, S);
     // topology
