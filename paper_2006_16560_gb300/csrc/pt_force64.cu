@@ -35,38 +35,46 @@ namespace pt {
 
 constexpr int kFfTile = 32;        // list entries per warp tile: one gathered by each lane
 constexpr int kFfFold = 2;         // tiles between folds of the float32 sums into float64
-constexpr unsigned kFfFewCells = 2048;   // cell lists below this take the full products (see ff_cells)
+constexpr unsigned kFfFewCells = 4096;   // cell lists below this take the full products (see ff_cells)
 constexpr int kFfQueue = 8;        // near pairs a lane may hold before the warp evaluates them
 constexpr float kFfTinyR2 = 0x1p-46f;   // smallest scaled r^2 evaluated in float32 expansions
 
+// Every value is a packed pair (f32x2), one for each of a lane's two targets:
+// half the instructions, so that the pipe and not the issue of dependent
+// instructions bounds the loops at 12 to 16 warps per SM (scalar float32, two
+// targets interleaved by the compiler: 150,001 particles 28.6 ms; packed 24.1
+// ms with four blocks per SM, which spill, and 23.5 ms with three).
+__device__ __forceinline__ f2x neg2(f2x a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2x dup2(float a) { return pk2(a, a); }
+
 struct ff {            // h + l
-    float h, l;
+    f2x h, l;
 };
 struct ft {            // h + l + e, |l| <= ulp(h) / 2, e ~ the rounding of l
-    float h, l, e;
+    f2x h, l, e;
 };
 
-__device__ __forceinline__ ff ff_two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+__device__ __forceinline__ ff ff_two_sum(f2x a, f2x b) {
+    const f2x s = add2(a, b), bb = sub2(s, a);
+    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
 }
-__device__ __forceinline__ ff ff_fast(float a, float b) {      // |a| >= |b| or a = 0
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+__device__ __forceinline__ ff ff_fast(f2x a, f2x b) {      // |a| >= |b| or a = 0
+    const f2x s = add2(a, b);
+    return {s, sub2(b, sub2(s, a))};
 }
-__device__ __forceinline__ ff ff_prod(float a, float b) {      // exact
-    const float p = __fmul_rn(a, b);
-    return {p, __fmaf_rn(a, b, -p)};
+__device__ __forceinline__ ff ff_prod(f2x a, f2x b) {      // exact
+    const f2x p = mul2(a, b);
+    return {p, fma2(a, b, neg2(p))};
 }
 
 // ---- two float32 (quadrupole terms); low parts are not renormalised
 __device__ __forceinline__ ff ff_mul(ff a, ff b) {
     const ff p = ff_prod(a.h, b.h);
-    return {p.h, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l))};
+    return {p.h, fma2(a.l, b.h, fma2(a.h, b.l, p.l))};
 }
 __device__ __forceinline__ ff ff_sum3(ff x, ff y, ff z) {
     const ff s = ff_two_sum(x.h, y.h), t = ff_two_sum(s.h, z.h);
-    return ff_fast(t.h, __fadd_rn(__fadd_rn(__fadd_rn(x.l, y.l), z.l), __fadd_rn(s.l, t.l)));
+    return ff_fast(t.h, add2(add2(add2(x.l, y.l), z.l), add2(s.l, t.l)));
 }
 
 // ---- three float32
@@ -74,8 +82,8 @@ __device__ __forceinline__ ff ff_sum3(ff x, ff y, ff z) {
 __device__ __forceinline__ ft ft_mul_raw(ft a, ft b) {         // h not renormalised against l
     const ff p = ff_prod(a.h, b.h), q = ff_prod(a.h, b.l), r = ff_prod(a.l, b.h);
     const ff c = ff_two_sum(q.h, r.h), d = ff_two_sum(p.l, c.h);
-    const float w = __fadd_rn(__fadd_rn(c.l, d.l), __fadd_rn(q.l, r.l));
-    return {p.h, d.h, __fmaf_rn(a.h, b.e, __fmaf_rn(a.e, b.h, __fmaf_rn(a.l, b.l, w)))};
+    const f2x w = add2(add2(c.l, d.l), add2(q.l, r.l));
+    return {p.h, d.h, fma2(a.h, b.e, fma2(a.e, b.h, fma2(a.l, b.l, w)))};
 }
 __device__ __forceinline__ ft ft_mul(ft a, ft b) {
     const ft x = ft_mul_raw(a, b);
@@ -84,19 +92,19 @@ __device__ __forceinline__ ft ft_mul(ft a, ft b) {
 }
 // the same with the cross terms rounded (~2^-49): cells
 __device__ __forceinline__ ft ft_mul_cell(ft a, ft b) {
-    const ff p = ff_prod(a.h, b.h), d = ff_two_sum(p.l, __fmaf_rn(a.l, b.h, __fmul_rn(a.h, b.l)));
+    const ff p = ff_prod(a.h, b.h), d = ff_two_sum(p.l, fma2(a.l, b.h, mul2(a.h, b.l)));
     const ff s = ff_fast(p.h, d.h);
-    return {s.h, s.l, __fmaf_rn(a.h, b.e, __fmaf_rn(a.e, b.h, __fmaf_rn(a.l, b.l, d.l)))};
+    return {s.h, s.l, fma2(a.h, b.e, fma2(a.e, b.h, fma2(a.l, b.l, d.l)))};
 }
 // running sum of x.h + x.l + x.e
 __device__ __forceinline__ void ft_acc(ft &a, ft x) {
     const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l), u = ff_two_sum(t.h, x.l);
-    a = {s.h, u.h, __fadd_rn(a.e, __fadd_rn(__fadd_rn(t.l, u.l), x.e))};
+    a = {s.h, u.h, add2(a.e, add2(add2(t.l, u.l), x.e))};
 }
 // the same with x.l added to the third word (~2^-49 of x): cells
 __device__ __forceinline__ void ft_acc_cell(ft &a, ff x) {
     const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l);
-    a = {s.h, t.h, __fadd_rn(a.e, __fadd_rn(t.l, x.l))};
+    a = {s.h, t.h, add2(a.e, add2(t.l, x.l))};
 }
 // float32 to float64 on the integer pipe (finite values; subnormals are 0)
 __device__ __forceinline__ double ff_widen(float f) {
@@ -108,8 +116,8 @@ __device__ __forceinline__ double ff_widen(float f) {
 // Separation of two coordinates from their limbs: the limb differences are
 // exact (each limb is an integer of at most 21 bits in its unit), and each is
 // zero or at least as large as the next (FastTwoSum's condition).
-__device__ __forceinline__ ft ft_sep(float aj, float bj, float cj, float ai, float bi, float ci) {
-    const ff s = ff_fast(__fsub_rn(aj, ai), __fsub_rn(bj, bi)), t = ff_fast(s.l, __fsub_rn(cj, ci));
+__device__ __forceinline__ ft ft_sep(f2x aj, f2x bj, f2x cj, f2x ai, f2x bi, f2x ci) {
+    const ff s = ff_fast(sub2(aj, ai), sub2(bj, bi)), t = ff_fast(s.l, sub2(cj, ci));
     const ff r = ff_fast(s.h, t.h);
     return {r.h, r.l, t.l};
 }
@@ -118,20 +126,20 @@ __device__ __forceinline__ ft ft_sep(float aj, float bj, float cj, float ai, flo
 __device__ __forceinline__ ft ft_norm2(ft x, ft y, ft z) {
     const ft d[3] = {x, y, z};
     ff p[3], c[3];
-    float w[3];
+    f2x w[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         p[k] = ff_prod(d[k].h, d[k].h);
-        const float t = __fadd_rn(d[k].h, d[k].h);
+        const f2x t = add2(d[k].h, d[k].h);
         const ff q = ff_prod(t, d[k].l);
         c[k] = ff_two_sum(p[k].l, q.h);
-        w[k] = __fadd_rn(c[k].l, __fmaf_rn(t, d[k].e, __fmaf_rn(d[k].l, d[k].l, q.l)));
+        w[k] = add2(c[k].l, fma2(t, d[k].e, fma2(d[k].l, d[k].l, q.l)));
     }
     const ff s = ff_two_sum(p[0].h, p[1].h), t = ff_two_sum(s.h, p[2].h);
     const ff a = ff_two_sum(c[0].h, c[1].h), b = ff_two_sum(c[2].h, s.l), e = ff_two_sum(a.h, b.h);
     const ff g = ff_two_sum(e.h, t.l), r = ff_fast(t.h, g.h);
-    return {r.h, r.l, __fadd_rn(__fadd_rn(__fadd_rn(w[0], w[1]), w[2]),
-                                __fadd_rn(__fadd_rn(a.l, b.l), __fadd_rn(e.l, g.l)))};
+    return {r.h, r.l, add2(add2(add2(w[0], w[1]), w[2]),
+                                add2(add2(a.l, b.l), add2(e.l, g.l)))};
 }
 
 // 1 / sqrt(r2): the float32 approximation, one float32 Newton step (so that
@@ -139,16 +147,17 @@ __device__ __forceinline__ ft ft_norm2(ft x, ft y, ft z) {
 // on the residual d = 1 - r2 y^2, whose leading part 1 - fl(r2.h y^2) is
 // exact.
 __device__ __forceinline__ ft ft_rsqrt(ft r2) {
-    float y = rsqrtf(r2.h);
-    const float h0 = __fmul_rn(0.5f, y);
-    y = __fmaf_rn(h0, __fmaf_rn(-r2.h, __fmul_rn(y, y), 1.0f), y);
+    const float2 s = up2(r2.h);
+    f2x y = pk2(rsqrtf(s.x), rsqrtf(s.y));
+    const f2x one = dup2(1.0f), half = dup2(0.5f);
+    y = fma2(mul2(half, y), sub2(one, mul2(mul2(r2.h, y), y)), y);
     const ff q = ff_prod(y, y), p = ff_prod(r2.h, q.h), u = ff_prod(r2.h, q.l), v = ff_prod(r2.l, q.h);
-    const ff g = ff_two_sum(u.h, v.h), k = ff_two_sum(g.h, p.l), d = ff_two_sum(__fsub_rn(1.0f, p.h), -k.h);
-    const float de = __fsub_rn(d.l, __fadd_rn(__fadd_rn(__fadd_rn(g.l, k.l), __fadd_rn(u.l, v.l)),
-                                              __fmaf_rn(r2.l, q.l, __fmul_rn(r2.e, q.h))));
-    const ff l = ff_prod(__fmul_rn(0.5f, y), d.h);
+    const ff g = ff_two_sum(u.h, v.h), k = ff_two_sum(g.h, p.l), d = ff_two_sum(sub2(one, p.h), neg2(k.h));
+    const f2x de = sub2(d.l, add2(add2(add2(g.l, k.l), add2(u.l, v.l)), fma2(r2.l, q.l, mul2(r2.e, q.h))));
+    const f2x hy = mul2(half, y);
+    const ff l = ff_prod(hy, d.h);
     const ff r = ff_fast(y, l.h);
-    return {r.h, r.l, __fmaf_rn(__fmul_rn(0.5f, y), de, __fmaf_rn(__fmul_rn(l.h, 0.75f), d.h, l.l))};
+    return {r.h, r.l, fma2(hy, de, fma2(mul2(l.h, dup2(0.75f)), d.h, l.l))};
 }
 
 // ---------------------------------------------------------------------------
@@ -240,8 +249,8 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
 // Force kernel
 // ---------------------------------------------------------------------------
 
-struct FfTarget {
-    float ax, ay, az, bx, by, bz, cx, cy, cz;
+struct FfTarget {         // limbs of the lane's two targets
+    f2x ax, ay, az, bx, by, bz, cx, cy, cz;
 };
 
 struct FfGroup {          // per group, formed by one thread
@@ -255,68 +264,65 @@ struct FfGroup {          // per group, formed by one thread
 // u = d/r and q = u.Q.u (the unit-vector form keeps Q's products in range).
 // FULL: the monopole keeps three float32 throughout (short lists, whose few
 // terms do not average the cheaper products' rounding).
-template <int NI, int ORDER, bool FULL>
-__device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int cnt, const FfTarget (&T)[NI],
-                                         ft (&acc)[NI][4]) {
-    for (int j = 0; j < cnt; j++) {
+// The lane takes cells s, s + J, .. of the tile.
+template <int J, int ORDER, bool FULL>
+__device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int s, int cnt, const FfTarget &T, ft (&acc)[4]) {
+    for (int j = s; j < cnt; j += J) {
         const float4 A = sT[0][j], B = sT[1][j], Cc = sT[2][j];
+        const ft d[3] = {ft_sep(dup2(A.x), dup2(B.x), dup2(Cc.x), T.ax, T.bx, T.cx),
+                         ft_sep(dup2(A.y), dup2(B.y), dup2(Cc.y), T.ay, T.by, T.cy),
+                         ft_sep(dup2(A.z), dup2(B.z), dup2(Cc.z), T.az, T.bz, T.cz)};
+        const ft ri = ft_rsqrt(ft_norm2(d[0], d[1], d[2]));
+        const ft m = {dup2(A.w), dup2(B.w), dup2(Cc.w)};
+        const ft ri2 = FULL ? ft_mul(ri, ri) : ft_mul_cell(ri, ri), mr = FULL ? ft_mul(m, ri) : ft_mul_cell(m, ri);
+        ft f = FULL ? ft_mul(mr, ri2) : ft_mul_cell(mr, ri2), pot = mr;
+        ff w[3];
+        if (ORDER == 2) {
+            const float4 Q = sT[3][j], Ql = sT[4][j], Q2 = sT[5][j];
+            const ff xx = {dup2(Q.x), dup2(Ql.x)}, yy = {dup2(Q.y), dup2(Ql.y)}, zz = {dup2(Q.z), dup2(Ql.z)};
+            const ff xy = {dup2(Q.w), dup2(Ql.w)}, xz = {dup2(Q2.x), dup2(Q2.y)}, yz = {dup2(Q2.z), dup2(Q2.w)};
+            const ff r1 = {ri.h, ri.l}, r2 = {ri2.h, ri2.l};
+            const ff ux = ff_mul({d[0].h, d[0].l}, r1), uy = ff_mul({d[1].h, d[1].l}, r1);
+            const ff uz = ff_mul({d[2].h, d[2].l}, r1);
+            w[0] = ff_sum3(ff_mul(xx, ux), ff_mul(xy, uy), ff_mul(xz, uz));
+            w[1] = ff_sum3(ff_mul(xy, ux), ff_mul(yy, uy), ff_mul(yz, uz));
+            w[2] = ff_sum3(ff_mul(xz, ux), ff_mul(yz, uy), ff_mul(zz, uz));
+            const ff q3 = ff_mul(ff_sum3(ff_mul(ux, w[0]), ff_mul(uy, w[1]), ff_mul(uz, w[2])),
+                                 ff_mul(r2, r1));                            // q / r^3
+            const f2x half = dup2(0.5f), c25 = dup2(2.5f);
+            const ff s2 = ff_two_sum(pot.h, mul2(half, q3.h));
+            const ff v = ff_two_sum(pot.l, fma2(half, q3.l, s2.l));
+            pot = {s2.h, v.h, add2(pot.e, v.l)};
+            const ff t = ff_mul(q3, r2);                                     // q / r^5
+            const ff t25 = ff_prod(c25, t.h), g = ff_two_sum(f.h, t25.h);
+            const ff z = ff_two_sum(f.l, add2(g.l, fma2(c25, t.l, t25.l)));
+            const ff h = ff_fast(g.h, z.h);
+            f = {h.h, h.l, add2(f.e, z.l)};
+            const ff r4 = ff_mul(r2, r2);
 #pragma unroll
-        for (int k = 0; k < NI; k++) {
-            const ft d[3] = {ft_sep(A.x, B.x, Cc.x, T[k].ax, T[k].bx, T[k].cx),
-                             ft_sep(A.y, B.y, Cc.y, T[k].ay, T[k].by, T[k].cy),
-                             ft_sep(A.z, B.z, Cc.z, T[k].az, T[k].bz, T[k].cz)};
-            const ft ri = ft_rsqrt(ft_norm2(d[0], d[1], d[2]));
-            const ft m = {A.w, B.w, Cc.w};
-            const ft ri2 = FULL ? ft_mul(ri, ri) : ft_mul_cell(ri, ri), mr = FULL ? ft_mul(m, ri) : ft_mul_cell(m, ri);
-            ft f = FULL ? ft_mul(mr, ri2) : ft_mul_cell(mr, ri2), pot = mr;
-            ff w[3];
-            if (ORDER == 2) {
-                const float4 Q = sT[3][j], Ql = sT[4][j], Q2 = sT[5][j];
-                const ff xx = {Q.x, Ql.x}, yy = {Q.y, Ql.y}, zz = {Q.z, Ql.z}, xy = {Q.w, Ql.w};
-                const ff xz = {Q2.x, Q2.y}, yz = {Q2.z, Q2.w};
-                const ff r1 = {ri.h, ri.l}, r2 = {ri2.h, ri2.l};
-                const ff ux = ff_mul({d[0].h, d[0].l}, r1), uy = ff_mul({d[1].h, d[1].l}, r1);
-                const ff uz = ff_mul({d[2].h, d[2].l}, r1);
-                w[0] = ff_sum3(ff_mul(xx, ux), ff_mul(xy, uy), ff_mul(xz, uz));
-                w[1] = ff_sum3(ff_mul(xy, ux), ff_mul(yy, uy), ff_mul(yz, uz));
-                w[2] = ff_sum3(ff_mul(xz, ux), ff_mul(yz, uy), ff_mul(zz, uz));
-                const ff q3 = ff_mul(ff_sum3(ff_mul(ux, w[0]), ff_mul(uy, w[1]), ff_mul(uz, w[2])),
-                                     ff_mul(r2, r1));                        // q / r^3
-                const ff s = ff_two_sum(pot.h, 0.5f * q3.h);
-                const ff v = ff_two_sum(pot.l, __fmaf_rn(0.5f, q3.l, s.l));
-                pot = {s.h, v.h, __fadd_rn(pot.e, v.l)};
-                const ff t = ff_mul(q3, r2);                                 // q / r^5
-                const ff t25 = ff_prod(2.5f, t.h), g = ff_two_sum(f.h, t25.h);
-                const ff z = ff_two_sum(f.l, __fadd_rn(g.l, __fmaf_rn(2.5f, t.l, t25.l)));
-                const ff h = ff_fast(g.h, z.h);
-                f = {h.h, h.l, __fadd_rn(f.e, z.l)};
-                const ff r4 = ff_mul(r2, r2);
-#pragma unroll
-                for (int c = 0; c < 3; c++) w[c] = ff_mul(w[c], r4);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                if (FULL) {
-                    ft x = ft_mul_raw(f, d[c]);
-                    if (ORDER == 2) {
-                        const ff s = ff_two_sum(x.h, -w[c].h), v = ff_two_sum(x.l, __fsub_rn(s.l, w[c].l));
-                        x = {s.h, v.h, __fadd_rn(x.e, v.l)};
-                    }
-                    ft_acc(acc[k][c], x);
-                } else {
-                    const ff p = ff_prod(f.h, d[c].h);
-                    ff x = {p.h, __fmaf_rn(f.l, d[c].h, __fmaf_rn(f.h, d[c].l,
-                                 __fmaf_rn(f.h, d[c].e, __fmaf_rn(f.e, d[c].h, p.l))))};
-                    if (ORDER == 2) {
-                        const ff s = ff_two_sum(p.h, -w[c].h);
-                        x = {s.h, __fadd_rn(x.l, __fsub_rn(s.l, w[c].l))};
-                    }
-                    ft_acc_cell(acc[k][c], x);
-                }
-            }
-            if (FULL) ft_acc(acc[k][3], pot);
-            else ft_acc_cell(acc[k][3], {pot.h, __fadd_rn(pot.l, pot.e)});
+            for (int c = 0; c < 3; c++) w[c] = ff_mul(w[c], r4);
         }
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            if (FULL) {
+                ft x = ft_mul_raw(f, d[c]);
+                if (ORDER == 2) {
+                    const ff s2 = ff_two_sum(x.h, neg2(w[c].h)), v = ff_two_sum(x.l, sub2(s2.l, w[c].l));
+                    x = {s2.h, v.h, add2(x.e, v.l)};
+                }
+                ft_acc(acc[c], x);
+            } else {
+                const ff p = ff_prod(f.h, d[c].h);
+                ff x = {p.h, fma2(f.l, d[c].h, fma2(f.h, d[c].l, fma2(f.h, d[c].e, fma2(f.e, d[c].h, p.l))))};
+                if (ORDER == 2) {
+                    const ff s2 = ff_two_sum(p.h, neg2(w[c].h));
+                    x = {s2.h, add2(x.l, sub2(s2.l, w[c].l))};
+                }
+                ft_acc_cell(acc[c], x);
+            }
+        }
+        if (FULL) ft_acc(acc[3], pot);
+        else ft_acc_cell(acc[3], {pot.h, add2(pot.l, pot.e)});
     }
 }
 
@@ -324,15 +330,15 @@ __device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int cnt, c
 // neighbour test and changeover (Sec. 6.1, Eqs. 15-17), into the lane's
 // float64 sums.  K = W = 0 beyond r_out, so a pair queued by the conservative
 // float32 bound is exact as well.
-template <int NI, bool MD>
+template <bool MD>
 __device__ __forceinline__ void ff_near(const ForceArgs &A, const FfGroup &G, const unsigned *queue, int &qn,
-                                        const unsigned (&pid)[NI], double (*sD)[4][32]) {
+                                        const unsigned (&pid)[2], double (*sD)[4][32]) {
     const int lane = threadIdx.x & 31;
     for (int e = 0; __any_sync(0xffffffffu, e < qn); e++) {
         if (e >= qn) continue;
         const unsigned code = queue[e * 32 + lane];
-        const int k = NI > 1 ? (int)(code >> 31) : 0;
-        const unsigned pj = code & 0x7fffffffu, pi = NI > 1 && k ? pid[NI - 1] : pid[0];
+        const int k = (int)(code >> 31);
+        const unsigned pj = code & 0x7fffffffu, pi = pid[k ? 1 : 0];
         const double4 xi = A.sp64[pi], xj = A.sp64[pj];
         const double dx = __dsub_rn(xj.x, xi.x), dy = __dsub_rn(xj.y, xi.y), dz = __dsub_rn(xj.z, xi.z);
         const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
@@ -370,40 +376,43 @@ __device__ __forceinline__ void ff_near(const ForceArgs &A, const FfGroup &G, co
 // Particle pairs outside r_out: a += m d/r^3, P += m/r.  Closer ones (and
 // those below kFfTinyR2) are queued for ff_near and weigh nothing here; the
 // target's own entry is skipped.
-template <int NI, bool MD>
+template <int J, bool MD>
 __device__ __forceinline__ void ff_pairs(const ForceArgs &A, const FfGroup &G, const float4 (*sT)[kFfTile],
-                                         const unsigned *sI, const float *sW, int cnt, const FfTarget (&T)[NI],
-                                         const float (&invs)[NI], const unsigned (&pid)[NI],
-                                         const bool (&valid)[NI], unsigned *queue, int &qn,
-                                         double (*sD)[4][32], ft (&acc)[NI][4]) {
+                                         const unsigned *sI, const float *sW, int s, int cnt, const FfTarget &T,
+                                         const float (&invs)[2], const unsigned (&pid)[2], const bool (&valid)[2],
+                                         unsigned *queue, int &qn, double (*sD)[4][32], ft (&acc)[4]) {
     const int lane = threadIdx.x & 31;
-    for (int j = 0; j < cnt; j++) {
+    for (int j0 = 0; j0 < cnt; j0 += J) {         // uniform across the warp (it votes)
+        const bool real = J == 1 || j0 + s < cnt;
+        const int j = real ? j0 + s : j0;
         const float4 P = sT[0][j], B = sT[1][j], Cc = sT[2][j];
         const unsigned pj = sI[j];
-#pragma unroll
-        for (int k = 0; k < NI; k++) {
-            const ft dx = ft_sep(P.x, B.x, Cc.x, T[k].ax, T[k].bx, T[k].cx);
-            const ft dy = ft_sep(P.y, B.y, Cc.y, T[k].ay, T[k].by, T[k].cy);
-            const ft dz = ft_sep(P.z, B.z, Cc.z, T[k].az, T[k].bz, T[k].cz);
-            ft r2 = ft_norm2(dx, dy, dz);
-            float q2 = r2.h;
-            if (MD) {
-                const float w = fminf(invs[k], sW[j]);        // 1 / s_ij
-                q2 *= w * w;
-            }
-            const bool hit = q2 < G.hit2 || r2.h < kFfTinyR2;
-            if (hit && pj != pid[k] && valid[k]) queue[qn++ * 32 + lane] = pj | (k ? 0x80000000u : 0u);
-            r2.h = hit ? 1.0f : r2.h;
-            const ft m = {hit ? 0.0f : P.w, hit ? 0.0f : B.w, hit ? 0.0f : Cc.w};
-            const ft ri = ft_rsqrt(r2);
-            const ft mr = ft_mul(m, ri);
-            const ft f = ft_mul(mr, ft_mul(ri, ri));
-            ft_acc(acc[k][0], ft_mul_raw(f, dx));
-            ft_acc(acc[k][1], ft_mul_raw(f, dy));
-            ft_acc(acc[k][2], ft_mul_raw(f, dz));
-            ft_acc(acc[k][3], mr);
+        const ft dx = ft_sep(dup2(P.x), dup2(B.x), dup2(Cc.x), T.ax, T.bx, T.cx);
+        const ft dy = ft_sep(dup2(P.y), dup2(B.y), dup2(Cc.y), T.ay, T.by, T.cy);
+        const ft dz = ft_sep(dup2(P.z), dup2(B.z), dup2(Cc.z), T.az, T.bz, T.cz);
+        ft r2 = ft_norm2(dx, dy, dz);
+        const float2 rh = up2(r2.h);
+        float2 q2 = rh;
+        if (MD) {
+            const float w0 = fminf(invs[0], sW[j]), w1 = fminf(invs[1], sW[j]);   // 1 / s_ij
+            q2.x *= w0 * w0;
+            q2.y *= w1 * w1;
         }
-        if (__any_sync(0xffffffffu, qn > kFfQueue - NI)) ff_near<NI, MD>(A, G, queue, qn, pid, sD);
+        const bool hit0 = q2.x < G.hit2 || rh.x < kFfTinyR2, hit1 = q2.y < G.hit2 || rh.y < kFfTinyR2;
+        if (hit0 && real && pj != pid[0] && valid[0]) queue[qn++ * 32 + lane] = pj;
+        if (hit1 && real && pj != pid[1] && valid[1]) queue[qn++ * 32 + lane] = pj | 0x80000000u;
+        const bool none0 = hit0 || !real, none1 = hit1 || !real;
+        r2.h = pk2(none0 ? 1.0f : rh.x, none1 ? 1.0f : rh.y);
+        const ft m = {pk2(none0 ? 0.0f : P.w, none1 ? 0.0f : P.w), pk2(none0 ? 0.0f : B.w, none1 ? 0.0f : B.w),
+                      pk2(none0 ? 0.0f : Cc.w, none1 ? 0.0f : Cc.w)};
+        const ft ri = ft_rsqrt(r2);
+        const ft mr = ft_mul(m, ri);
+        const ft f = ft_mul(mr, ft_mul(ri, ri));
+        ft_acc(acc[0], ft_mul_raw(f, dx));
+        ft_acc(acc[1], ft_mul_raw(f, dy));
+        ft_acc(acc[2], ft_mul_raw(f, dz));
+        ft_acc(acc[3], mr);
+        if (__any_sync(0xffffffffu, qn > kFfQueue - 2)) ff_near<MD>(A, G, queue, qn, pid, sD);
     }
 }
 
@@ -418,41 +427,46 @@ struct FfShared {
     unsigned g;
 };
 
-// One pass over up to 32 NI targets; every warp takes every fourth tile of
-// each list segment.  Leaves the warps' float64 sums in S.D.
-template <int NI, int ORDER, bool MD>
+// One pass over up to 64 / J targets, two per lane: the warp's lanes form J
+// sub-streams that take every J-th list entry, so that a group of few targets
+// still fills them.  Every warp takes every fourth tile of each list segment.
+// Leaves the lanes' float64 sums in S.D.
+template <int J, int ORDER, bool MD>
 __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, unsigned lo,
                                         unsigned hi, FfShared &S) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    FfTarget T[NI];
-    float invs[NI];
-    unsigned pid[NI];
-    bool valid[NI];
-    ft acc[NI][4];
+    constexpr int L = 32 / J;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, s = lane / L;
+    float invs[2];
+    unsigned pid[2];
+    bool valid[2];
+    float4 a[2], b[2], c[2];
 #pragma unroll
-    for (int k = 0; k < NI; k++) {
-        const unsigned idx = i0 + lane + 32 * k;
+    for (int k = 0; k < 2; k++) {
+        const unsigned idx = i0 + lane % L + L * k;
         valid[k] = idx < gr.y;
         pid[k] = gr.x + (valid[k] ? idx : 0u);
-        const float4 a = A.ffp[3ull * pid[k]], b = A.ffp[3ull * pid[k] + 1], c = A.ffp[3ull * pid[k] + 2];
-        T[k] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z};
+        a[k] = A.ffp[3ull * pid[k]];
+        b[k] = A.ffp[3ull * pid[k] + 1];
+        c[k] = A.ffp[3ull * pid[k] + 2];
         invs[k] = MD ? A.spL[pid[k]].w : 1.0f;
 #pragma unroll
-        for (int q = 0; q < 4; q++) acc[k][q] = {0.0f, 0.0f, 0.0f};
-    }
-#pragma unroll
-    for (int k = 0; k < 2; k++)
-#pragma unroll
         for (int q = 0; q < 4; q++) S.D[w][k][q][lane] = 0.0;
+    }
+    const FfTarget T = {pk2(a[0].x, a[1].x), pk2(a[0].y, a[1].y), pk2(a[0].z, a[1].z),
+                        pk2(b[0].x, b[1].x), pk2(b[0].y, b[1].y), pk2(b[0].z, b[1].z),
+                        pk2(c[0].x, c[1].x), pk2(c[0].y, c[1].y), pk2(c[0].z, c[1].z)};
+    ft acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) acc[q] = {0ull, 0ull, 0ull};
     const FfGroup &G = S.G;
     auto fold = [&]() {
 #pragma unroll
-        for (int k = 0; k < NI; k++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                S.D[w][k][q][lane] += ff_widen(acc[k][q].h) + (ff_widen(acc[k][q].l) + ff_widen(acc[k][q].e));
-                acc[k][q] = {0.0f, 0.0f, 0.0f};
-            }
+        for (int q = 0; q < 4; q++) {
+            const float2 x = up2(acc[q].h), y = up2(acc[q].l), z = up2(acc[q].e);
+            S.D[w][0][q][lane] += ff_widen(x.x) + (ff_widen(y.x) + ff_widen(z.x));
+            S.D[w][1][q][lane] += ff_widen(x.y) + (ff_widen(y.y) + ff_widen(z.y));
+            acc[q] = {0ull, 0ull, 0ull};
+        }
     };
     int tiles = 0, qn = 0;
     {
@@ -470,8 +484,8 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
                 for (int r = 0; r < (ORDER == 2 ? 6 : 3); r++) S.T[w][r][lane] = o[r];
             }
             __syncwarp();
-            if (nc < kFfFewCells) ff_cells<NI, ORDER, true>(S.T[w], cnt, T, acc);
-            else ff_cells<NI, ORDER, false>(S.T[w], cnt, T, acc);
+            if (nc < kFfFewCells) ff_cells<J, ORDER, true>(S.T[w], s, cnt, T, acc);
+            else ff_cells<J, ORDER, false>(S.T[w], s, cnt, T, acc);
             __syncwarp();
             if (++tiles % kFfFold == 0) fold();
         }
@@ -493,12 +507,12 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
                 for (int r = 0; r < 3; r++) S.T[w][r][lane] = A.ffp[3ull * p + r];
             }
             __syncwarp();
-            ff_pairs<NI, MD>(A, G, S.T[w], S.I[w], S.W[w], cnt, T, invs, pid, valid, S.queue[w], qn, S.D[w], acc);
+            ff_pairs<J, MD>(A, G, S.T[w], S.I[w], S.W[w], s, cnt, T, invs, pid, valid, S.queue[w], qn, S.D[w], acc);
             __syncwarp();
             if (++tiles % kFfFold == 0) fold();
         }
     }
-    ff_near<NI, MD>(A, G, S.queue[w], qn, pid, S.D[w]);
+    ff_near<MD>(A, G, S.queue[w], qn, pid, S.D[w]);
     fold();
 }
 
@@ -518,7 +532,7 @@ __device__ __forceinline__ void ff_write(const ForceArgs &A, unsigned p, const d
 }
 
 template <int ORDER, bool MD, bool TAIL>
-__global__ void __launch_bounds__(kFThreads, 4) k_force_ff(ForceArgs A) {
+__global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
     __shared__ FfShared S;
     // lists left unusable by the walk (one-pass arrays exhausted, stack
     // overflow): do nothing, the host re-runs the walk and the force
@@ -565,19 +579,23 @@ __global__ void __launch_bounds__(kFThreads, 4) k_force_ff(ForceArgs A) {
         __syncthreads();
         double ep[4] = {0, 0, 0, 0};
         const unsigned t = threadIdx.x;
-        for (unsigned i0 = 0; i0 < gr.y; i0 += 64) {
-            if (gr.y - i0 > 32) ff_pass<2, ORDER, MD>(A, g, gr, i0, lo, hi, S);
-            else ff_pass<1, ORDER, MD>(A, g, gr, i0, lo, hi, S);
+        for (unsigned i0 = 0; i0 < gr.y;) {
+            const unsigned left = gr.y - i0, L = left > 32 ? 32u : left > 16 ? 16u : 8u;     // targets per sub-stream / 2
+            if (L == 32) ff_pass<1, ORDER, MD>(A, g, gr, i0, lo, hi, S);
+            else if (L == 16) ff_pass<2, ORDER, MD>(A, g, gr, i0, lo, hi, S);
+            else ff_pass<4, ORDER, MD>(A, g, gr, i0, lo, hi, S);
             __syncthreads();
-            if (t < 64 && i0 + t < gr.y) {                   // fixed-order sums over the warps
+            if (t < 2 * L && t < left) {                     // fixed-order sums over warps and sub-streams
                 double s[4] = {0, 0, 0, 0};
                 for (int w = 0; w < kFWarps; w++)
-                    for (int c = 0; c < 4; c++) s[c] += S.D[w][t >> 5][c][t & 31];
+                    for (unsigned l = t % L; l < 32; l += L)
+                        for (int c = 0; c < 4; c++) s[c] += S.D[w][t / L][c][l];
                 for (int c = 0; c < 4; c++) s[c] *= c < 3 ? S.G.sa : S.G.sp;
                 if (parts == 1) ff_write(A, gr.x + i0 + t, s, ep);
                 else store_part(A, g, part, i0 + t, s);
             }
             __syncthreads();
+            i0 += 2 * L;
         }
         if (parts > 1) {
             if (!last_part(A, g, parts, &S.g)) continue;
