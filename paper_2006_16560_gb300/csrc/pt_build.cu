@@ -10,6 +10,10 @@ namespace pt {
 
 constexpr int kT = 256;
 constexpr unsigned kTopoBig = 16;     // nodes above this size get a warp in the topology count
+// Largest set whose topology and multipole levels run in one block each: build
+// of 1,000 particles 215 -> 177 us, of 4,096 252 -> 250 us (one block's rounds
+// over a level then cost what the launches did), of 16,384 319 -> 379 us.
+constexpr unsigned kSmallBuild = 2048;
 
 // ---------------------------------------------------------------------------
 // Sets (clusters) and the root box
@@ -257,9 +261,8 @@ __device__ __forceinline__ void level_range(const Status *st, int l, unsigned ca
     if (c > cap - b) c = cap - b;
 }
 
-__global__ void k_topo_roots(const SetInfo *sets, int nsets, uint4 *nd_a, uint4 *nd_b,
-                             uint2 *nd_r, Status *st) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void topo_roots(int s, const SetInfo *sets, int nsets, uint4 *nd_a, uint4 *nd_b,
+                                           uint2 *nd_r, Status *st) {
     if (s < nsets) {
         nd_r[s] = make_uint2(sets[s].begin, sets[s].n);
         nd_a[s] = make_uint4(0, 0, 0, make_meta(0, 0, 0));
@@ -276,6 +279,10 @@ __global__ void k_topo_roots(const SetInfo *sets, int nsets, uint4 *nd_a, uint4 
         for (int b = 0; b < kLeafBuckets; b++) st->leaf_hist[b] = st->leaf_fill[b] = 0;
         st->nwide = 0;
     }
+}
+
+__global__ void k_topo_roots(const SetInfo *sets, int nsets, uint4 *nd_a, uint4 *nd_b, uint2 *nd_r, Status *st) {
+    topo_roots(blockIdx.x * blockDim.x + threadIdx.x, sets, nsets, nd_a, nd_b, nd_r, st);
 }
 
 // lcp[p] = number of leading key digits (levels) that sorted keys p - 1 and
@@ -376,12 +383,11 @@ __device__ __forceinline__ void topo_chunk(unsigned cnt, unsigned &k0, unsigned 
 // thread; larger ones a warp, whose lanes 1..7 bisect for the seven digit
 // boundaries at once (a thread doing them one after another waits on ~140
 // dependent loads at the top levels).
-__global__ void __launch_bounds__(kT) k_topo_count(int l, const unsigned long long *skey,
-                                                   const unsigned char *lcp, uint4 *nd_a,
-                                                   const uint2 *nd_r, unsigned *nch, uint4 *bnd,
-                                                   unsigned *bsum, int n_leaf, int levels, unsigned cap,
-                                                   Status *st) {
-    __shared__ unsigned sh[kT / 32];
+__device__ __forceinline__ void topo_count(int l, const unsigned long long *skey,
+                                           const unsigned char *lcp, uint4 *nd_a,
+                                           const uint2 *nd_r, unsigned *nch, uint4 *bnd,
+                                           unsigned *bsum, int n_leaf, int levels, unsigned cap,
+                                           Status *st, unsigned *sh) {
     unsigned b0, cnt, k0, k1;
     level_range(st, l, cap, b0, cnt);
     topo_chunk(cnt, k0, k1);
@@ -449,17 +455,25 @@ __global__ void __launch_bounds__(kT) k_topo_count(int l, const unsigned long lo
     if (threadIdx.x == 0) bsum[blockIdx.x] = s;
 }
 
+__global__ void __launch_bounds__(kT) k_topo_count(int l, const unsigned long long *skey,
+                                                   const unsigned char *lcp, uint4 *nd_a,
+                                                   const uint2 *nd_r, unsigned *nch, uint4 *bnd,
+                                                   unsigned *bsum, int n_leaf, int levels, unsigned cap,
+                                                   Status *st) {
+    __shared__ unsigned sh[kT / 32];
+    topo_count(l, skey, lcp, nd_a, nd_r, nch, bnd, bsum, n_leaf, levels, cap, st, sh);
+}
+
 // Creates the children of level l's split nodes and lists the split nodes
 // themselves, in any order, in nd_int from lvl_begin[l] on (the multipole
 // pass then takes one internal node per thread with no leaves in between:
 // float64 instructions cost the same for a warp with few lanes).  A block's
 // children follow those of the blocks before it (the sum of their bsum) in
 // the order of its chunk (a block scan), so level l+1 is in key order.
-__global__ void __launch_bounds__(kT) k_topo_emit(int l, const uint4 *bnd,
-                                                  uint4 *nd_a, uint4 *nd_b, uint2 *nd_r,
-                                                  const unsigned *nch, const unsigned *bsum,
-                                                  unsigned *nd_int, unsigned cap, Status *st) {
-    __shared__ unsigned sh[kT / 32];
+__device__ __forceinline__ void topo_emit(int l, const uint4 *bnd,
+                                          uint4 *nd_a, uint4 *nd_b, uint2 *nd_r,
+                                          const unsigned *nch, const unsigned *bsum,
+                                          unsigned *nd_int, unsigned cap, Status *st, unsigned *sh) {
     unsigned b0, cnt, k0, k1;
     level_range(st, l, cap, b0, cnt);
     topo_chunk(cnt, k0, k1);
@@ -517,7 +531,15 @@ __global__ void __launch_bounds__(kT) k_topo_emit(int l, const uint4 *bnd,
     }
 }
 
-__global__ void k_topo_finish(Status *st, unsigned cap) {
+__global__ void __launch_bounds__(kT) k_topo_emit(int l, const uint4 *bnd,
+                                                  uint4 *nd_a, uint4 *nd_b, uint2 *nd_r,
+                                                  const unsigned *nch, const unsigned *bsum,
+                                                  unsigned *nd_int, unsigned cap, Status *st) {
+    __shared__ unsigned sh[kT / 32];
+    topo_emit(l, bnd, nd_a, nd_b, nd_r, nch, bsum, nd_int, cap, st, sh);
+}
+
+__device__ __forceinline__ void topo_finish(Status *st, unsigned cap) {
     unsigned total = 0, maxl = 0;
     for (int l = 0; l < kLevels; l++) {
         if (st->lvl_count[l]) maxl = (unsigned)l;
@@ -529,6 +551,29 @@ __global__ void k_topo_finish(Status *st, unsigned cap) {
     }
     st->nnodes = total;
     st->max_level = maxl;
+}
+
+__global__ void k_topo_finish(Status *st, unsigned cap) { topo_finish(st, cap); }
+
+// Small sets: the whole topology in one block (the same steps, a barrier in
+// place of a launch between them; a level of a few hundred nodes costs a
+// launch and the latency of a few dependent loads, whatever the grid), up to
+// the tree's own depth.
+__global__ void __launch_bounds__(kT) k_topo_small(const SetInfo *sets, int nsets, const unsigned long long *skey,
+                                                   const unsigned char *lcp, uint4 *nd_a, uint4 *nd_b, uint2 *nd_r,
+                                                   unsigned *nch, uint4 *bnd, unsigned *bsum, unsigned *nd_int,
+                                                   int n_leaf, unsigned cap, Status *st) {
+    __shared__ unsigned sh[kT / 32];
+    for (int s = threadIdx.x; s < nsets; s += kT) topo_roots(s, sets, nsets, nd_a, nd_b, nd_r, st);
+    __syncthreads();
+    for (int l = 0; l <= kMaxLevel; l++) {
+        topo_count(l, skey, lcp, nd_a, nd_r, nch, bnd, bsum, n_leaf, kMaxLevel, cap, st, sh);
+        __syncthreads();
+        if (l == kMaxLevel || bsum[0] == 0) break;        // no node of this level was split
+        topo_emit(l, bnd, nd_a, nd_b, nd_r, nch, bsum, nd_int, cap, st, sh);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) topo_finish(st, cap);
 }
 
 // ---------------------------------------------------------------------------
@@ -772,6 +817,21 @@ __global__ void __launch_bounds__(kT) k_moments_level(int l, const uint4 *sq, ui
         internal_moments(nd_int[b0 + k], sq, nd_a, nd_b, nd_r, nd_c, nd_q, nd_t, nd_f, sets, nd_thr, cap);
 }
 
+// Small sets: all levels in one block, as k_topo_small.
+__global__ void __launch_bounds__(kT) k_moments_small(const uint4 *sq, uint4 *nd_a, uint4 *nd_b, const uint2 *nd_r,
+                                                      double4 *nd_c, double4 *nd_q, double4 *nd_t, float4 *nd_f,
+                                                      const SetInfo *sets, long long *nd_thr, const unsigned *nd_int,
+                                                      unsigned cap, const Status *st) {
+    for (int l = (int)st->max_level - 1; l >= 0; l--) {
+        unsigned b0, cnt;
+        level_range(st, l, cap, b0, cnt);
+        const unsigned ni = min(st->lvl_int[l], cnt);
+        for (unsigned k = threadIdx.x; k < ni; k += kT)
+            internal_moments(nd_int[b0 + k], sq, nd_a, nd_b, nd_r, nd_c, nd_q, nd_t, nd_f, sets, nd_thr, cap);
+        __syncthreads();
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Groups: mark the first particle of every group, compact, then describe.
 // A node with at most n_group particles (or a leaf) is a group; a larger
@@ -911,19 +971,26 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     // topology
     k_lcp<<<grid_for(n, kT, gmax), kT, 0, st>>>(A.skey, A.n_dev, A.lcp);
     nk++;
-    k_topo_roots<<<(A.nsets + 127) / 128, 128, 0, st>>>(A.sets, A.nsets, A.nd_a, A.nd_b, A.nd_r, S);
-    nk += 2;
-    for (int l = 0; l <= A.levels; l++) {
-        k_topo_count<<<gmax, kT, 0, st>>>(l, A.skey, A.lcp, A.nd_a, A.nd_r, A.tmp_u32a, A.nd_bnd,
-                                          A.topo_bsum, A.n_leaf, A.levels, A.cap_nodes, S);
-        nk++;
-        if (l == A.levels) break;
-        k_topo_emit<<<gmax, kT, 0, st>>>(l, A.nd_bnd, A.nd_a, A.nd_b, A.nd_r, A.tmp_u32a, A.topo_bsum,
-                                         A.nd_int, A.cap_nodes, S);
+    const bool small = n <= kSmallBuild;
+    if (small) {
+        k_topo_small<<<1, kT, 0, st>>>(A.sets, A.nsets, A.skey, A.lcp, A.nd_a, A.nd_b, A.nd_r, A.tmp_u32a, A.nd_bnd,
+                                       A.topo_bsum, A.nd_int, A.n_leaf, A.cap_nodes, S);
+        nk += 2;
+    } else {
+        k_topo_roots<<<(A.nsets + 127) / 128, 128, 0, st>>>(A.sets, A.nsets, A.nd_a, A.nd_b, A.nd_r, S);
+        nk += 2;
+        for (int l = 0; l <= A.levels; l++) {
+            k_topo_count<<<gmax, kT, 0, st>>>(l, A.skey, A.lcp, A.nd_a, A.nd_r, A.tmp_u32a, A.nd_bnd,
+                                              A.topo_bsum, A.n_leaf, A.levels, A.cap_nodes, S);
+            nk++;
+            if (l == A.levels) break;
+            k_topo_emit<<<gmax, kT, 0, st>>>(l, A.nd_bnd, A.nd_a, A.nd_b, A.nd_r, A.tmp_u32a, A.topo_bsum,
+                                             A.nd_int, A.cap_nodes, S);
+            nk++;
+        }
+        k_topo_finish<<<1, 1, 0, st>>>(S, A.cap_nodes);
         nk++;
     }
-    k_topo_finish<<<1, 1, 0, st>>>(S, A.cap_nodes);
-    nk++;
     long long *thr = A.massdep ? A.nd_thr : nullptr;
     k_leaf_hist<<<gmax, kT, 0, st>>>(A.nd_a, A.nd_r, A.cap_nodes, S);
     k_leaf_scatter<<<gmax, kT, 0, st>>>(A.nd_a, A.nd_r, A.cap_nodes, A.tmp_u32a, S);
@@ -931,13 +998,19 @@ int build_launch(const BuildArgs &A, cudaStream_t st) {
     k_moments_leaves<<<gmax, kT, 0, st>>>(A.sp64, A.sq, A.nd_a, A.nd_b, A.nd_r, A.nd_c, A.nd_q, A.nd_t,
                                           A.nd_f, A.ssc, A.sets, thr, A.tmp_u32a, A.cap_nodes, S);
     nk++;
-    // two blocks per SM: the kernel's 120 registers allow no more resident
-    // ones, and a level's internal nodes are few (the larger grid ran in
-    // waves of idle blocks)
-    const int mgrid = sm_count() * 2;
-    for (int l = A.levels - 1; l >= 0; l--, nk++)
-        k_moments_level<<<mgrid, kT, 0, st>>>(l, A.sq, A.nd_a, A.nd_b, A.nd_r, A.nd_c, A.nd_q, A.nd_t,
-                                             A.nd_f, A.sets, thr, A.nd_int, A.cap_nodes, S);
+    if (small) {
+        k_moments_small<<<1, kT, 0, st>>>(A.sq, A.nd_a, A.nd_b, A.nd_r, A.nd_c, A.nd_q, A.nd_t, A.nd_f, A.sets, thr,
+                                          A.nd_int, A.cap_nodes, S);
+        nk++;
+    } else {
+        // two blocks per SM: the kernel's 120 registers allow no more resident
+        // ones, and a level's internal nodes are few (the larger grid ran in
+        // waves of idle blocks)
+        const int mgrid = sm_count() * 2;
+        for (int l = A.levels - 1; l >= 0; l--, nk++)
+            k_moments_level<<<mgrid, kT, 0, st>>>(l, A.sq, A.nd_a, A.nd_b, A.nd_r, A.nd_c, A.nd_q, A.nd_t,
+                                                 A.nd_f, A.sets, thr, A.nd_int, A.cap_nodes, S);
+    }
     // groups
     cudaMemsetAsync(A.gflag, 0, (size_t)n * sizeof(unsigned), st);
     k_group_mark<<<gmax, kT, 0, st>>>(A.nd_a, A.nd_b, A.nd_r, A.gflag, A.n_group, S);
