@@ -426,7 +426,7 @@ int read_status(pt_tree *t) {
 }
 
 // Build over t->n particles in t->nsets sets; pos/mass are device pointers.
-// Enqueues the build between events ev[0] and ev[1]. Its ~105 short kernels
+// Enqueues the build between events ev[0] and ev[1]. Its dozens of short kernels
 // are bound by the host's launch rate, so a build whose arguments equal the
 // previous one's is captured into a CUDA graph (on the context's private
 // stream) and replayed from then on.
@@ -538,9 +538,10 @@ WalkArgs walk_args(pt_tree *t) {
     return A;
 }
 
-// Targets per partial record of a split group (a walk group holds at most
-// n_group particles; larger depth-capped leaves are never split).
-unsigned part_stride(const pt_tree *t) { return (unsigned)std::min(t->prm.n_group, 1 << 16); }
+// Targets per partial record of a split group: the most a walk group holds,
+// n_group; groups of more than 256 (a larger n_group, a depth-capped leaf)
+// take several passes anyway and are never split.
+unsigned part_stride(const pt_tree *t) { return (unsigned)std::min(t->prm.n_group, 256); }
 
 // Room for the force work items: one per group (at most n) and the extra
 // parts of the split groups, as many as the last step's with a quarter and 64

@@ -1,18 +1,18 @@
-// pt_force.cu -- the P3T long-range force kernels, fused neighbour
-// extraction, the energy / momentum sums and the neighbour CSR.
+// pt_force.cu -- the mixed-precision P3T long-range force kernel with fused
+// neighbour extraction, the work items of both force kernels (the float64
+// one is in pt_force64.cu), the energy / momentum sums and the neighbour CSR.
 //
-// One CTA (4 warps) evaluates one walk group at a time, taking groups from
-// an atomic work counter in the order k_group_order writes (largest pass
-// configuration first).  Every warp holds all of the group's targets (two or
-// three per lane) and streams its own quarter of the group's lists: it
-// gathers a tile of list entries into shared memory (128 in the mixed
-// kernel, 64 in the float64 one), then every lane reads them by broadcast and
-// accumulates.  The four warps' partial sums are reduced in float64 at the
-// end of the group, in a fixed order.  Four warps per group rather than one
-// keep small sets (a few thousand particles, a few hundred groups) spread
-// over the whole GPU.  A group has one cell list and two PP segments: near
-// (leaves within r_out of the group's box: changeover and neighbour tests)
-// and far (every pair at least r_out apart: plain Newtonian pairs).
+// One CTA (4 warps) evaluates one item: a walk group, or for a group with
+// long lists one part of them (see pt_force.cuh), in the order k_items_write
+// lists them.  Every warp holds all of the group's targets (two or three per
+// lane) and streams its own quarter of the lists: it gathers a tile of 128
+// list entries into shared memory, then every lane reads them by broadcast
+// and accumulates.  The four warps' partial sums are added in float-float at
+// the end, in a fixed order.  Four warps per group rather than one keep small
+// sets (a few thousand particles, a few hundred groups) spread over the whole
+// GPU.  A group has one cell list and two PP segments: near (leaves within
+// r_out of the group's box: changeover and neighbour tests) and far (every
+// pair at least r_out apart: plain Newtonian pairs).
 //
 // Pair force (Sec. 5.1, Eq. 11; Sec. 6.1, Eqs. 15-17), for x_ij > 0:
 //   a_i += m_j (x_j - x_i) (1 - K(x)) / r^3,  P_i += m_j (1 - W(x)) / r

@@ -118,7 +118,7 @@ struct ForceArgs {
     double4 *parts;                  // partial sums: part_stride targets per record
     unsigned part_stride;
     unsigned item_cap, part_cap;     // items the launch can take, records in parts
-    unsigned part_shift;             // log2 of the part length's unit: see part_entries
+    unsigned part_shift;             // scale of the part length by precision: see part_entries
     const unsigned *cells, *pp;
     const double4 *sp64;
     const float4 *spH, *spL;
