@@ -944,8 +944,7 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
         nk += batch_gather_launch(dtab, dsets, C, n, ip, im, isc, st);
     }
     CK(cudaMemsetAsync(dS, 0, sizeof(Status), st));
-    nk += build_launch(build_args(t, ip, im), st);
-    CK(cudaMemsetAsync(&dS->flags, 0, sizeof(unsigned), st));
+    nk += build_launch(build_args(t, ip, im), st);       // its flags stay for the host (kErrBuild)
     WalkArgs W = walk_args(t);
     nk += walk_launch(W, 2, st);              // one pass (arrays sized before the capture)
     ForceArgs F = force_args(t, t->d_acc.as<double>(), t->d_pot.as<double>(), want_nb);

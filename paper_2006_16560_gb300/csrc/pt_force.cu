@@ -621,9 +621,9 @@ __global__ void __launch_bounds__(kFThreads, PT_FORCE_MIN_BLOCKS) k_force_mixed(
     // (float64 divisions and a square root: slow on this part's FP64 pipe)
     __shared__ ChgF sC;
     __shared__ double sRout2, sRout, sC2;
-    // lists left unusable by the walk (one-pass arrays exhausted, stack
-    // overflow): do nothing, the host re-runs the walk and the force
-    if (A.st->flags & (kErrListCap | kErrStack | kErrItemCap)) return;
+    // lists left unusable by the build or the walk (one-pass arrays exhausted,
+    // stack overflow): do nothing, the host reports it or runs them again
+    if (A.st->flags & (kErrBuild | kErrListCap | kErrStack | kErrItemCap)) return;
     const unsigned ni = A.st->nitems;
     for (unsigned it = 0;; it++) {
         unsigned gi;
@@ -799,8 +799,8 @@ __global__ void __launch_bounds__(32) k_force_reduce(const double4 *red_e, const
 constexpr int kItemThreads = 256;
 
 // Parts and item class of group g.  A group larger than a partial record (a
-// leaf at the depth limit) is never split, nor is any when the walk left the
-// lists unusable.
+// leaf at the depth limit) is never split, nor is any when the build or the
+// walk left the lists unusable.
 __device__ __forceinline__ unsigned group_parts(const ForceArgs &A, unsigned g, unsigned unit, bool usable, int &cls) {
     const unsigned n = A.gr_r[g].y, L = A.gr_nc[g] + A.gr_np[g] + A.gr_nf[g];
     const unsigned most = part_entries(A.sets[A.gr_a[g].w].n, A.part_shift);
@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(kItemThreads) k_items_count(ForceArgs A, unsig
     __shared__ unsigned sh[kItemClasses];
     if (threadIdx.x < kItemClasses) sh[threadIdx.x] = 0;
     __syncthreads();
-    const bool usable = (A.st->flags & (kErrListCap | kErrStack)) == 0;
+    const bool usable = (A.st->flags & (kErrBuild | kErrListCap | kErrStack)) == 0;
     unsigned b, e;
     item_chunk(A.st->ngroups, b, e);
     for (unsigned g = b + threadIdx.x; g < e; g += kItemThreads) {
@@ -866,7 +866,7 @@ __global__ void __launch_bounds__(kItemThreads) k_items_write(ForceArgs A, unsig
             if (sum > A.item_cap || tot[0] > A.part_cap) atomicOr(&A.st->flags, kErrItemCap);
         }
     }
-    const bool usable = (A.st->flags & (kErrListCap | kErrStack)) == 0;
+    const bool usable = (A.st->flags & (kErrBuild | kErrListCap | kErrStack)) == 0;
     unsigned b, e;
     item_chunk(A.st->ngroups, b, e);
     for (unsigned r = b; r < e; r += kItemThreads) {          // uniform across the block

@@ -534,9 +534,9 @@ __device__ __forceinline__ void ff_write(const ForceArgs &A, unsigned p, const d
 template <int ORDER, bool MD, bool TAIL>
 __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
     __shared__ FfShared S;
-    // lists left unusable by the walk (one-pass arrays exhausted, stack
-    // overflow): do nothing, the host re-runs the walk and the force
-    if (A.st->flags & (kErrListCap | kErrStack | kErrItemCap)) return;
+    // lists left unusable by the build or the walk (one-pass arrays exhausted,
+    // stack overflow): do nothing, the host reports it or runs them again
+    if (A.st->flags & (kErrBuild | kErrListCap | kErrStack | kErrItemCap)) return;
     const unsigned ni = A.st->nitems;
     for (unsigned it = 0;; it++) {
         unsigned gi;

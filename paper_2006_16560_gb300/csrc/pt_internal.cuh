@@ -43,6 +43,11 @@ enum : unsigned {
     kErrBadScale = 1u << 7,   // radius factor not finite and positive
     kErrLevels = 1u << 9,     // a node above n_leaf particles at the deepest level launched
     kErrItemCap = 1u << 8,    // more force work items or partial records than the launch holds
+    // a build whose tree is not to be walked: its input was refused, or it ran
+    // out of nodes (links to children past the arrays) or levels.  A batch
+    // enqueues the walk and the force without reading the status in between;
+    // they then do nothing, and the host sees the flag at the end
+    kErrBuild = kErrNonFinite | kErrNegMass | kErrBadScale | kErrNodeCap | kErrLevels,
 };
 
 // Per-set (cluster) table entry.

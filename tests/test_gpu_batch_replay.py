@@ -1,0 +1,92 @@
+"""Replayed batch graphs on inputs unlike those they were captured on.
+
+A captured step fixes its launches and array sizes; a replay whose tree, lists
+or rows do not fit must be noticed and computed again, and refused inputs must
+be refused as in an uncaptured call.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_helpers import run_gpu
+from paper_2006_16560_gb300 import binding as B
+from paper_2006_16560_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _cuda(x):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+def _batch(sizes, r_out=0.02, nb_factor=8):
+    sets = []
+    for k, n in enumerate(sizes):
+        d = inputs.plummer(n, 40 + k, masses="kroupa")
+        sets.append({"pos": _cuda(d["pos"]), "mass": _cuda(d["mass"]), "r_in": 0.1 * r_out, "r_out": r_out})
+    return B.Batch(sets, nb_factor=nb_factor)
+
+
+def _assert_equals_single_sets(b, prm):
+    ctx = B.Context(0)
+    for k, s in enumerate(b.sets):
+        p = B.Params(**{**prm.__dict__, "r_in": s["r_in"], "r_out": s["r_out"]})
+        g = run_gpu(ctx, s["pos"].cpu().numpy(), s["mass"].cpu().numpy(), p)
+        assert np.array_equal(b.acc[k].cpu().numpy(), g["acc"]) and np.array_equal(b.pot[k].cpu().numpy(), g["pot"])
+        assert np.array_equal(b.nb_off[k].cpu().numpy(), g["nb_off"])
+        assert np.array_equal(b.nb_idx[k][: len(g["nb_idx"])].cpu().numpy(), g["nb_idx"])
+        g["tree"].free()
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_leaf", [1, 8])
+@pytest.mark.parametrize("precision", [B.PT_FP64, B.PT_MIXED])
+def test_replay_on_a_deeper_tree(n_leaf, precision):
+    prm = B.Params(theta=0.5, n_leaf=n_leaf, n_group=64, order=2, precision=precision)
+    ctx = B.Context(0)
+    b = _batch([3000, 1500])
+    for _ in range(2):
+        shallow = b.run(ctx, prm, graph=True)
+    pos = b.sets[0]["pos"].cpu().numpy()
+    pos[:12] = pos[0] + 1e-8 * np.random.default_rng(2).random((12, 3))      # a clump far below the captured depth
+    b.sets[0]["pos"].copy_(_cuda(pos))
+    for _ in range(2):                                                       # the replay, and the graph captured anew
+        st = b.run(ctx, prm, graph=True)
+        assert st["max_level"] >= shallow["max_level"] + 5
+        _assert_equals_single_sets(b, prm)
+    ctx.close()
+
+
+def test_replay_out_of_nodes():
+    prm = B.Params(theta=0.5, n_leaf=1, n_group=64, order=2, precision=B.PT_MIXED)
+    ctx = B.Context(0)
+    b = _batch([3000])
+    for _ in range(2):
+        b.run(ctx, prm, graph=True)
+    pos = b.sets[0]["pos"].cpu().numpy()
+    pos[1::2] = pos[::2] + 1e-7                        # tight pairs: a chain of single children above each
+    b.sets[0]["pos"].copy_(_cuda(pos))
+    for _ in range(2):
+        assert b.run(ctx, prm, graph=True)["nodes"] > 4 * len(pos)
+        _assert_equals_single_sets(b, prm)
+    ctx.close()
+
+
+@pytest.mark.parametrize("what", ["nan", "inf", "negative mass"])
+def test_replay_refuses_bad_input(what):
+    prm = B.Params(theta=0.5, n_leaf=8, n_group=64, order=2, precision=B.PT_MIXED)
+    ctx = B.Context(0)
+    b = _batch([1000, 2500])
+    for _ in range(2):
+        b.run(ctx, prm, graph=True)
+    t = b.sets[1]["mass"] if what == "negative mass" else b.sets[1]["pos"][:, 1]
+    good = t[7].item()
+    t[7] = {"nan": float("nan"), "inf": float("inf"), "negative mass": -good}[what]
+    with pytest.raises(B.PTError) as e:
+        b.run(ctx, prm, graph=True)
+    assert e.value.code == B.PT_ERR_ARG
+    t[7] = good
+    b.run(ctx, prm, graph=True)
+    _assert_equals_single_sets(b, prm)
+    ctx.close()
