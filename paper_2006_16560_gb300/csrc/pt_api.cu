@@ -200,6 +200,7 @@ struct pt_tree {
     // sizes its arrays from them (0: no estimate yet, walk in two passes)
     unsigned long long est_cells = 0, est_pp = 0;
     bool nb_long = false;                      // a neighbour row was too long for nb_launch
+    bool graph_nb_long = false;                // what gexec holds: nb_sort_launch or nb_launch
     long long est_extra = -1;                  // force items beyond one per group (-1: no step yet)
     unsigned est_parts = 0;                    // partial records of its split groups
     unsigned long long chunk_cells = kWalkChunkEntries, chunk_pp = kWalkChunkEntries;
@@ -643,7 +644,8 @@ NbArgs nb_args(pt_tree *t) {
 int nb_stage(pt_tree *t, cudaStream_t st) {
     return t->nb_long ? nb_sort_launch(nb_args(t), st) : nb_launch(nb_args(t), st);
 }
-bool nb_rows_too_long(pt_tree *t) { return !t->nb_long && t->h.max_row > kNbRowMax; }
+// Whether the CSR just made holds rows that nb_launch left unsorted.
+bool nb_rows_too_long(const pt_tree *t, bool sorted) { return !sorted && t->h.max_row > kNbRowMax; }
 
 int alloc_pairs(pt_tree *t, unsigned long long cap) {
     pt_ctx *ctx = t->ctx;
@@ -758,7 +760,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             t->est_extra = (long long)t->h.nitems - (long long)t->h.ngroups;
             t->est_parts = t->h.nparts;
             if (!(t->h.flags & kErrItemCap)) {
-                if (want_nb && nb_rows_too_long(t)) {
+                if (want_nb && nb_rows_too_long(t, t->nb_long)) {
                     t->nb_long = true;
                     t->launches_force += nb_stage(t, st);
                     CK(cudaGetLastError());
@@ -1085,7 +1087,7 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
         if (f & (kErrNonFinite | kErrNegMass | kErrBadScale))
             return fail(ctx, PT_ERR_ARG, "non-finite position, negative mass or radius factor not finite and positive");
         if (!(f & (kErrNodeCap | kErrLevels | kErrStack | kErrListCap | kErrItemCap)) && !pair_short &&
-            !(want_nb && nb_rows_too_long(t))) {
+            !(want_nb && nb_rows_too_long(t, t->graph_nb_long))) {
             done = true;
             cudaEventElapsedTime(&ms[2], ctx->ev[6], ctx->ev[7]);
         } else {
@@ -1158,6 +1160,7 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
                 t->gexec = nullptr;
                 return fail(ctx, PT_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ec));
             }
+            t->graph_nb_long = t->nb_long;
             t->gkey_mode = mode;
             t->gkey_p = *params;
             t->gkey_n.resize(C);
@@ -1611,7 +1614,7 @@ int pt_orbit_neighbours(pt_tree *t, const double *vel, const pt_orbit_params *op
             nb_stage(t, st);
             CK(cudaGetLastError());
             TRY(read_status(t));
-            if (nb_rows_too_long(t)) {
+            if (nb_rows_too_long(t, t->nb_long)) {
                 t->nb_long = true;
                 nb_stage(t, st);
                 CK(cudaGetLastError());

@@ -90,3 +90,35 @@ def test_replay_refuses_bad_input(what):
     b.run(ctx, prm, graph=True)
     _assert_equals_single_sets(b, prm)
     ctx.close()
+
+
+def _clump(b, members):
+    """Moves the first particles of the first set together: rows of members - 1 neighbours."""
+    pos = b.sets[0]["pos"].cpu().numpy()
+    pos[:members] = np.array([3.0, 1.0, 2.0]) + 1e-3 * np.random.default_rng(members).random((members, 3))
+    b.sets[0]["pos"].copy_(_cuda(pos))
+
+
+def _assert_rows(b):
+    for k, s in enumerate(b.sets):
+        off, idx = oracle.neighbours(s["pos"].cpu().numpy(), s["r_out"])
+        assert np.array_equal(b.nb_off[k].cpu().numpy(), off)
+        assert np.array_equal(b.nb_idx[k][: len(idx)].cpu().numpy(), idx)
+
+
+def test_replay_with_rows_longer_than_captured():
+    prm = B.Params(theta=0.5, n_leaf=8, n_group=64, order=0, precision=B.PT_MIXED)
+    ctx = B.Context(0)
+    b, other = _batch([2500, 1000], nb_factor=200), _batch([3000], nb_factor=200)
+    for _ in range(2):
+        b.run(ctx, prm, graph=True)
+        _assert_rows(b)
+    _clump(other, 700)
+    other.run(ctx, prm)                                # rows too long for the captured way, in an uncaptured call
+    _assert_rows(other)
+    for members in (600, 40, 600, 300, 20):
+        _clump(b, members)
+        for _ in range(2):
+            b.run(ctx, prm, graph=True)
+            _assert_rows(b)
+    ctx.close()
