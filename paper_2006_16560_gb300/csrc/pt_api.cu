@@ -199,7 +199,8 @@ struct pt_tree {
     // list sizes of the last successful walk of this tree: the one-pass walk
     // sizes its arrays from them (0: no estimate yet, walk in two passes)
     unsigned long long est_cells = 0, est_pp = 0;
-    bool nb_long = false;                      // a neighbour row was too long for nb_launch
+    // the last lists' rows were too long for nb_launch (force, orbit search)
+    bool nb_long = false, orb_nb_long = false;
     bool graph_nb_long = false;                // what gexec holds: nb_sort_launch or nb_launch
     long long est_extra = -1;                  // force items beyond one per group (-1: no step yet)
     unsigned est_parts = 0;                    // partial records of its split groups
@@ -639,10 +640,10 @@ NbArgs nb_args(pt_tree *t) {
     return A;
 }
 
-// Neighbour CSR of the tree's pairs: rows of any length by sorting all pairs
-// once a row has been too long for the direct way (nb_long).
-int nb_stage(pt_tree *t, cudaStream_t st) {
-    return t->nb_long ? nb_sort_launch(nb_args(t), st) : nb_launch(nb_args(t), st);
+// Neighbour CSR of the tree's pairs: by sorting all pairs (rows of any length)
+// when the last lists' rows were too long for the direct way.
+int nb_stage(pt_tree *t, bool sorted, cudaStream_t st) {
+    return sorted ? nb_sort_launch(nb_args(t), st) : nb_launch(nb_args(t), st);
 }
 // Whether the CSR just made holds rows that nb_launch left unsorted.
 bool nb_rows_too_long(const pt_tree *t, bool sorted) { return !sorted && t->h.max_row > kNbRowMax; }
@@ -751,7 +752,7 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             CK(cudaEventRecord(ctx->ev[4], st));
             TRY(copy_out());
             nk += force_reduce_launch(F, st);
-            if (want_nb) nk += nb_stage(t, st);
+            if (want_nb) nk += nb_stage(t, t->nb_long, st);
             t->launches_force = nk;
             CK(cudaGetLastError());
             CK(cudaEventRecord(ctx->ev[5], st));
@@ -760,11 +761,13 @@ int run_force(pt_tree *t, double *acc, double *pot, bool want_nb, unsigned long 
             t->est_extra = (long long)t->h.nitems - (long long)t->h.ngroups;
             t->est_parts = t->h.nparts;
             if (!(t->h.flags & kErrItemCap)) {
-                if (want_nb && nb_rows_too_long(t, t->nb_long)) {
-                    t->nb_long = true;
-                    t->launches_force += nb_stage(t, st);
-                    CK(cudaGetLastError());
-                    CK(cudaStreamSynchronize(st));
+                if (want_nb) {
+                    if (nb_rows_too_long(t, t->nb_long)) {
+                        t->launches_force += nb_stage(t, true, st);
+                        CK(cudaGetLastError());
+                        CK(cudaStreamSynchronize(st));
+                    }
+                    t->nb_long = t->h.max_row > kNbRowMax;
                 }
                 return PT_OK;
             }
@@ -958,7 +961,7 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
     nk += force_launch(F, t->prm.precision, t->n, st);
     nk += force_reduce_launch(F, st);
     if (want_nb) {
-        nk += nb_stage(t, st);
+        nk += nb_stage(t, t->nb_long, st);
         nk += batch_nb_launch(dtab, dsets, C, n, t->nb_off.as<long long>(), t->nb_idx.as<int>(),
                               t->d_totals.as<long long>(), !host_io, st);
     }
@@ -1611,14 +1614,14 @@ int pt_orbit_neighbours(pt_tree *t, const double *vel, const pt_orbit_params *op
             rc = fail(ctx, PT_ERR_CAPACITY, "orbit neighbour lists need %llu entries, capacity %lld",
                       npairs, (long long)nb_capacity);
         } else {
-            nb_stage(t, st);
+            nb_stage(t, t->orb_nb_long, st);
             CK(cudaGetLastError());
             TRY(read_status(t));
-            if (nb_rows_too_long(t, t->nb_long)) {
-                t->nb_long = true;
-                nb_stage(t, st);
+            if (nb_rows_too_long(t, t->orb_nb_long)) {
+                nb_stage(t, true, st);
                 CK(cudaGetLastError());
             }
+            t->orb_nb_long = t->h.max_row > kNbRowMax;
             cudaMemcpyKind k1 = is_device_ptr(nb_offsets) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
             CK(cudaMemcpyAsync(nb_offsets, t->nb_off.p, (n + 1) * 8, k1, st));
             if (npairs) {

@@ -944,8 +944,9 @@ int force_reduce_launch(const ForceArgs &A, cudaStream_t st) {
 // (row, column) took three per 8 bits of the key, 9 to 18, each a few us
 // whatever the number of pairs.  CSR and energy sums together, before -> after:
 // 1,000 particles (116 pairs) 60 -> 42 us, 2^20 (26,668) 111 -> 54 us, 10^7
-// (2.4e6) 580 -> 267 us.  Rows of more than kNbRowMax entries are left unsorted and reported (max_row): the
-// host then sorts all pairs by radix (nb_sort_launch).
+// (2.4e6) 580 -> 267 us.  Rows of more than kNbRowMax entries are reported after
+// the counting launch (max_row), and the others then do nothing: the host
+// sorts all pairs by radix (nb_sort_launch), now and until rows are shorter.
 // ===========================================================================
 
 __global__ void k_nb_count(NbArgs A) {
@@ -960,6 +961,7 @@ __global__ void k_nb_count(NbArgs A) {
 }
 
 __global__ void k_nb_fill(NbArgs A) {
+    if (A.st->max_row > kNbRowMax) return;
     unsigned long long np = A.st->npairs;
     if (np > A.pair_cap) np = A.pair_cap;
     const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
@@ -975,6 +977,7 @@ __global__ void k_nb_fill(NbArgs A) {
 // row's smaller entries.
 __global__ void __launch_bounds__(256) k_nb_rows(NbArgs A) {
     __shared__ int buf[8][kNbRowMax];
+    if (A.st->max_row > kNbRowMax) return;
     const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (unsigned r0 = warp * 32; r0 < A.n; r0 += nw * 32) {
@@ -1052,11 +1055,18 @@ __global__ void k_nb_csr(NbArgs A) {
         }
         A.nb_off[i] = (long long)lo;
     }
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x)
-        A.nb_idx[k] = (int)(A.keys_sorted[k] % A.n);
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
+        const unsigned long long key = A.keys_sorted[k];
+        const unsigned j = (unsigned)(key % A.n);
+        A.nb_idx[k] = (int)j;
+        // a row of more than kNbRowMax / 2 entries is reported as too long for nb_launch: rows
+        // that vary around kNbRowMax would else be made twice every other time
+        if (k >= kNbRowMax / 2 && A.keys_sorted[k - kNbRowMax / 2] >= key - j) A.st->max_row = kNbRowMax + 1;
+    }
 }
 
 int nb_sort_launch(const NbArgs &A, cudaStream_t st) {
+    cudaMemsetAsync(&A.st->max_row, 0, sizeof(unsigned), st);
     k_nb_keys<<<sm_count() * 4, 256, 0, st>>>(A);
     int nk = radix_sort(A.keys, A.vals, A.keys_sorted, A.vals_sorted, A.npairs_dev,
                         (unsigned)A.pair_cap, 0, A.key_bits, nullptr, 0, A.sort_tmp, st);

@@ -71,6 +71,7 @@ struct Status {
     unsigned nwide;                  // groups walked by whole blocks (listed in gr_wide)
     unsigned wide_next[2];           // their work counters (counting, filling)
     unsigned max_row;                // above kNbRowMax: a neighbour row is too long for nb_launch
+                                     // (after nb_sort_launch: for the next lists to take it)
     unsigned long long cell_total, pp_total;
     unsigned long long cell_inter, pp_inter;
     unsigned long long npairs;

@@ -84,3 +84,43 @@ def test_row_lengths():
             assert np.array_equal(idx[:total].cpu().numpy(), want_idx)
     t.free()
     ctx.close()
+
+
+def test_long_rows_are_forgotten():
+    """After lists with a row above 512 a tree makes short rows the short way again,
+    and a tree's neighbour search along orbits does not decide for its force."""
+    import torch
+
+    from paper_2006_16560_gb300 import binding as B
+    ctx = B.Context(0)
+    rng = np.random.default_rng(5)
+    n = 1500
+    short = rng.normal(size=(n, 3))
+    long = short.copy()
+    long[:600] = 5.0 + 1e-3 * rng.random((600, 3))
+    mass = _cuda(np.full(n, 1.0 / n))
+    p = B.Params(theta=0.5, r_in=0.001, r_out=0.01, n_leaf=8, n_group=64, order=0, precision=B.PT_MIXED)
+    acc, pot = torch.empty((n, 3), dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda")
+    off, idx = torch.empty(n + 1, dtype=torch.int64, device="cuda"), torch.empty(n * n, dtype=torch.int32, device="cuda")
+    t = B.Tree(ctx, _cuda(short), mass, p)
+
+    def step(pos):
+        t.rebuild(_cuda(pos), mass)
+        total, st, _ = t.force(acc, pot, off, idx, n * n)
+        want_off, want_idx = oracle.neighbours(pos, p.r_out)
+        assert np.array_equal(off.cpu().numpy(), want_off) and np.array_equal(idx[:total].cpu().numpy(), want_idx)
+        return st.launches_force
+
+    step(short)
+    usual = step(short)
+    assert step(long) > usual                             # made again by sorting
+    assert step(long) > usual                             # by sorting at once
+    step(short)
+    assert step(short) == usual
+    vel = _cuda(np.zeros((n, 3)))
+    vel[0, 0] = 1.0
+    o, i, _ = t.orbit_neighbours(vel, dt=10.0, C_v=1e9)    # one particle's radius covers the set
+    assert int(np.diff(o.cpu().numpy()).max()) > 512
+    assert step(short) == usual
+    t.free()
+    ctx.close()
