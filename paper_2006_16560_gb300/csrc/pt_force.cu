@@ -1054,15 +1054,12 @@ __global__ void k_nb_csr(NbArgs A) {
             if (A.keys_sorted[mid] < key) lo = mid + 1; else hi = mid;
         }
         A.nb_off[i] = (long long)lo;
-    }
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
-        const unsigned long long key = A.keys_sorted[k];
-        const unsigned j = (unsigned)(key % A.n);
-        A.nb_idx[k] = (int)j;
         // a row of more than kNbRowMax / 2 entries is reported as too long for nb_launch: rows
         // that vary around kNbRowMax would else be made twice every other time
-        if (k >= kNbRowMax / 2 && A.keys_sorted[k - kNbRowMax / 2] >= key - j) A.st->max_row = kNbRowMax + 1;
+        if (np - lo > kNbRowMax / 2 && A.keys_sorted[lo + kNbRowMax / 2] < key + A.n) A.st->max_row = kNbRowMax + 1;
     }
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x)
+        A.nb_idx[k] = (int)(A.keys_sorted[k] % A.n);
 }
 
 int nb_sort_launch(const NbArgs &A, cudaStream_t st) {

@@ -124,3 +124,21 @@ def test_long_rows_are_forgotten():
     assert step(short) == usual
     t.free()
     ctx.close()
+
+
+def test_many_long_rows_side_by_side():
+    """Clumps of adjacent particles whose rows lie around the warp's tiles (32 and 128 entries)."""
+    from paper_2006_16560_gb300 import binding as B
+    rng = np.random.default_rng(6)
+    pos = [rng.normal(size=(500, 3))]
+    for k, clump in enumerate((5, 33, 34, 64, 65, 66, 128, 129, 130, 131, 257, 258, 512, 513)):
+        pos.append(np.array([10.0 + k, 0.0, 0.0]) + 1e-3 * rng.random((clump, 3)))
+    pos = np.concatenate(pos)
+    n = len(pos)
+    ctx = B.Context(0)
+    for precision in (B.PT_MIXED, B.PT_FP64):
+        p = B.Params(theta=0.5, r_in=0.001, r_out=0.01, n_leaf=8, n_group=64, order=0, precision=precision)
+        _, _, off, idx, _ = B.longrange_force(ctx, _cuda(pos), _cuda(np.full(n, 1.0 / n)), p, nb_capacity=n * n)
+        want_off, want_idx = oracle.neighbours(pos, p.r_out)
+        assert np.array_equal(off.cpu().numpy(), want_off) and np.array_equal(idx.cpu().numpy(), want_idx)
+    ctx.close()
