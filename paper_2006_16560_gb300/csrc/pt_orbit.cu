@@ -122,10 +122,14 @@ __device__ __forceinline__ int orbit_pair(const OrbitArgs &A, unsigned pi, unsig
 }
 
 constexpr int kOrbChunk = 128;     // opened-leaf particles staged per warp
-// Warps that share a wide group (walk_wide: its box overlaps much of the tree,
-// so its members are tested against most of the set): each walks the whole
-// tree and tests every kOrbParts-th staged chunk.  One warp alone took as long
-// as the rest of the search (250,007 Kroupa Plummer particles: 2.85 -> 1.27 ms).
+// Warps that share a wide group at most (walk_wide: its box overlaps much of
+// the tree, so its members are tested against most of the set): each walks the
+// whole tree and tests its share of the staged chunks.  One warp alone took as
+// long as the rest of the search (250,007 Kroupa Plummer particles, 65 wide
+// groups: 2.85 -> 1.27 ms).  No more parts than the launch has warps for them:
+// nearly all groups of a uniform set of up to 10^5 particles are wide (a
+// uniform sphere of 100,003, 1,500 wide groups, whole call: 624 us in sixteen
+// parts each, 364 in as many as there are warps).
 constexpr unsigned kOrbParts = 16;
 
 // Candidate tests of the staged particles against every member of group g:
@@ -196,19 +200,26 @@ __global__ void __launch_bounds__(kOrbThreads) k_orbit_search(OrbitArgs A) {
     const unsigned ng = A.st->ngroups;
     unsigned *stk = ostack + (size_t)w * A.stack_cap;
     const int cap = (int)A.stack_cap;
-    // items: kOrbParts parts of every wide group, then the groups
-    const unsigned nparts = A.st->nwide * kOrbParts;
+    // items: the parts of every wide group, then the groups
+    const unsigned nwide = A.st->nwide;
+    const unsigned per = max(1u, min(kOrbParts, gridDim.x * kOrbWarps / max(nwide, 1u)));
+    const unsigned nparts = nwide * per;
     for (;;) {
         unsigned i = 0;
         if (lane == 0) i = (unsigned)atomicAdd(&A.ctr[0], 1ull);
         i = __shfl_sync(0xffffffffu, i, 0);
         if (i >= nparts + ng) break;
-        const unsigned g = i < nparts ? A.gr_wide[i / kOrbParts] : i - nparts;
+        const unsigned g = i < nparts ? A.gr_wide[i / per] : i - nparts;
         const uint4 ga = A.gr_a[g], gb = A.gr_b[g];
         if (i >= nparts && walk_wide(ga, gb, A.sets[ga.w].n)) continue;
-        const unsigned part = i < nparts ? i % kOrbParts : 0u;
-        unsigned chunk = 0;          // staged chunks so far (a wide group's part takes every kOrbParts-th)
-        auto mine = [&]() { return i >= nparts || chunk++ % kOrbParts == part; };
+        // staged chunks to the next one that is this part's (it takes every per-th)
+        unsigned skip = i < nparts ? i % per : 0u;
+        auto mine = [&]() {
+            if (i >= nparts) return true;
+            const bool m = skip == 0;
+            skip = m ? per - 1 : skip - 1;
+            return m;
+        };
         const uint2 gr = A.gr_r[g];
         const long long gthr = A.gr_thr[g];
         unsigned long long ncand = 0;

@@ -136,3 +136,14 @@ def test_full_size_sampled_rows(ctx):
     b = idx.astype(np.int64) * n + rows
     assert np.array_equal(np.sort(a), np.sort(b))
     assert off[-1] <= cand
+
+
+@pytest.mark.parametrize("n_group", [8, 24, 64])
+def test_uniform_set_of_wide_groups(ctx, n_group):
+    """Nearly every group of a uniform set is shared by warps: about 300 groups of
+    64 in several parts each, 2,500 of 8 in one, more than the launch's warps."""
+    rng = np.random.default_rng(n_group)
+    n = 20000
+    d = {"pos": rng.random((n, 3)), "vel": rng.normal(size=(n, 3)), "mass": rng.uniform(0.5, 1.5, n) / n}
+    r_out = 0.01
+    _check(ctx, d, r_out, 0.3 * r_out, 0, B.PT_ORBIT_ROUT, n_leaf=8, n_group=n_group)[0].free()
