@@ -342,9 +342,9 @@ int alloc_build(pt_tree *t, unsigned n, int nsets) {
     TRY(ensure(ctx, t->gpart, N * 32));
     TRY(ensure(ctx, t->red_part, (size_t)kRedBlocksMax * 48));     // reduction partials, one per block
     TRY(ensure(ctx, t->ssc, N * 8));
-    if (t->prm.precision == PT_FP64) {       // double-float records of the float64 force kernel
-        TRY(ensure(ctx, t->ffp, N * 48));
-        TRY(ensure(ctx, t->ffn, C * 96));
+    if (t->prm.precision == PT_FP64) {       // records of the float64 force kernel
+        TRY(ensure(ctx, t->ffp, N * 64));
+        TRY(ensure(ctx, t->ffn, C * 112));
     }
     TRY(ensure(ctx, t->set_mean, S * 8));
     if (t->prm.mass_dependent) {

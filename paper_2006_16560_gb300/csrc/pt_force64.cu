@@ -12,10 +12,16 @@
 // float64 operations, take float64 instructions.
 //
 // Precision.  Coordinates enter as 63-bit fixed point relative to the
-// coordinate origin (exact for |x| >= 2^-9 of the largest coordinate, within
-// 2^-63 of it below), cut into three 21-bit limbs held as float32.  Limb
-// differences are exact, so a pair's separation is correct to ~2^-70 of
-// itself however close the pair is and wherever the group lies.  r^2, 1/r and
+// coordinate origin, in units of each axis' largest coordinate, cut into three
+// 21-bit limbs held as float32, and the float32 remainder: exact for |x| >=
+// 2^-33 of that coordinate, within 2^-87 of it below.  (Without the remainder
+// the core of a set with an escaper loses bits: 3,000 Plummer particles and
+// one at 10^4 / 10^5 core radii, accelerations 7e-14 / 3e-13 rms from an
+// extended-precision sum of the same lists, against 5e-16 with float64
+// instructions and 2e-16 with the remainder.)  Limb differences are
+// exact, so the separation of a pair or of a cell evaluated here (2^-23 box
+// sides or more) is correct to ~2^-63 of itself wherever the group lies.
+// r^2, 1/r and
 // the products and sums of particle pairs and of short cell lists keep three
 // float32 (~2^-64); in a list of thousands of cells each cell's products keep
 // two and a half (~2^-49, averaged over the list), and a quadrupole term, at
@@ -113,13 +119,15 @@ __device__ __forceinline__ double ff_widen(float f) {
     return __hiloint2double(e ? (int)hi : 0, e ? (int)(u << 29) : 0);
 }
 
-// Separation of two coordinates from their limbs: the limb differences are
-// exact (each limb is an integer of at most 21 bits in its unit), and each is
-// zero or at least as large as the next (FastTwoSum's condition).
-__device__ __forceinline__ ft ft_sep(f2x aj, f2x bj, f2x cj, f2x ai, f2x bi, f2x ci) {
+// Separation of two coordinates from their limbs and remainders: the limb
+// differences are exact (each limb is an integer of at most 21 bits in its
+// unit), and each is zero or at least as large as the next (FastTwoSum's
+// condition); the remainders, below half the last limb's unit, only enter the
+// third word.
+__device__ __forceinline__ ft ft_sep(f2x aj, f2x bj, f2x cj, f2x dj, f2x ai, f2x bi, f2x ci, f2x di) {
     const ff s = ff_fast(sub2(aj, ai), sub2(bj, bi)), t = ff_fast(s.l, sub2(cj, ci));
     const ff r = ff_fast(s.h, t.h);
-    return {r.h, r.l, t.l};
+    return {r.h, r.l, add2(t.l, sub2(dj, di))};
 }
 
 // dx^2 + dy^2 + dz^2
@@ -162,35 +170,46 @@ __device__ __forceinline__ ft ft_rsqrt(ft r2) {
 
 // ---------------------------------------------------------------------------
 // Records of the float32 expansions, written once per force call from the
-// sorted float64 arrays (48 B per particle, 96 B per node)
+// sorted float64 arrays (64 B per particle, 112 B per node)
 // ---------------------------------------------------------------------------
 
-// Exponents of a set's units: X = 2^ex above every |coordinate|, lengths in
-// 2^es >= box side (for coincident particles, whose box side is a stand-in,
+// Exponents of a set's units: 2^ex above every |coordinate| of an axis, lengths
+// in 2^es >= box side (for coincident particles, whose box side is a stand-in,
 // not below 2^(ex - 60): the limbs then stay in range), masses in 2^em.
 struct FfUnits {
-    int ex, es, em;
+    int ex[3], es, em;
 };
 __device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M) {
-    double X = S.S * 0x1p-60;
-    for (int d = 0; d < 3; d++) X = fmax(X, fmax(fabs(S.origin[d]), fabs(S.origin[d] + S.S)));
     FfUnits u;
-    u.ex = ilogb(X) + 1;
-    u.es = max(ilogb(S.S) + 1, u.ex - 60);
+    u.es = ilogb(S.S) + 1;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const double X = fmax(S.S * 0x1p-60, fmax(fabs(S.origin[d]), fabs(S.origin[d] + S.S)));
+        u.ex[d] = ilogb(X) + 1;
+        u.es = max(u.es, u.ex[d] - 60);
+    }
     u.em = M > 0.0 ? ilogb(M) + 1 : 0;
     return u;
 }
 
-// The three limbs of x in units of 2^es: rounded to a multiple of 2^(ex - 62),
-// then cut 21 bits at a time, each limb rounded to nearest.
-__device__ __forceinline__ void ff_limbs(double x, const FfUnits &u, float &a, float &b, float &c) {
-    const long long f = __double2ll_rn(scalbn(x, 62 - u.ex));
+// The three limbs of x in units of 2^es, rounded to a multiple of 2^(ex - 62)
+// and cut 21 bits at a time, each limb rounded to nearest, and what that
+// rounding left (a double of 2^52 or more in those units leaves nothing).
+__device__ __forceinline__ void ff_limbs(double x, int ex, int es, float &a, float &b, float &c, float &d) {
+    const double w = scalbn(x, 62 - ex);
+    const long long f = __double2ll_rn(w);
     const long long ia = (f + (1ll << 41)) >> 42, rem = f - (ia << 42);
     const long long ib = (rem + (1ll << 20)) >> 21, ic = rem - (ib << 21);
-    const int k = u.ex - u.es;
+    const int k = ex - es;
     a = scalbnf((float)ia, k - 20);
     b = scalbnf((float)ib, k - 41);
     c = scalbnf((float)ic, k - 62);
+    d = scalbnf(__double2float_rn(w - (double)f), k - 62);
+}
+__device__ __forceinline__ void ff_position(double4 P, const FfUnits &u, float4 &a, float4 &b, float4 &c, float4 &d) {
+    ff_limbs(P.x, u.ex[0], u.es, a.x, b.x, c.x, d.x);
+    ff_limbs(P.y, u.ex[1], u.es, a.y, b.y, c.y, d.y);
+    ff_limbs(P.z, u.ex[2], u.es, a.z, b.z, c.z, d.z);
 }
 
 __device__ __forceinline__ float ff_split(double v, int k, float &h, float &l) {   // returns the third word
@@ -206,29 +225,30 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
         const unsigned set = A.sq[p].w;
         const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
         const double4 P = A.sp64[p];
-        float4 a, b, c;
-        ff_limbs(P.x, u, a.x, b.x, c.x);
-        ff_limbs(P.y, u, a.y, b.y, c.y);
-        ff_limbs(P.z, u, a.z, b.z, c.z);
+        float4 a, b, c, d;
+        ff_position(P, u, a, b, c, d);
         c.w = ff_split(P.w, -u.em, a.w, b.w);
-        A.ffp[3ull * p] = a;
-        A.ffp[3ull * p + 1] = b;
-        A.ffp[3ull * p + 2] = c;
+        d.w = 0.0f;
+        float4 *o = A.ffp + 4ull * p;
+        o[0] = a;
+        o[1] = b;
+        o[2] = c;
+        o[3] = d;
     }
     const unsigned nn = A.st->nnodes;
     for (unsigned v = t0; v < nn; v += dt) {
         const unsigned set = A.sq[A.nd_r[v].x].w;
         const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
         const double4 P = A.nd_c[v];
-        float4 a, b, c;
-        ff_limbs(P.x, u, a.x, b.x, c.x);
-        ff_limbs(P.y, u, a.y, b.y, c.y);
-        ff_limbs(P.z, u, a.z, b.z, c.z);
+        float4 a, b, c, d;
+        ff_position(P, u, a, b, c, d);
         c.w = ff_split(P.w, -u.em, a.w, b.w);
-        float4 *o = A.ffn + 6ull * v;
+        d.w = 0.0f;
+        float4 *o = A.ffn + 7ull * v;
         o[0] = a;
         o[1] = b;
         o[2] = c;
+        o[3] = d;
         if (A.order == 2) {                  // Qxx Qyy Qzz Qxy | their low parts | Qxz, Qyz (high, low)
             const double4 q0 = A.nd_q[2 * v], q1 = A.nd_q[2 * v + 1];
             const int k = -u.em - 2 * u.es;
@@ -238,9 +258,9 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
             ff_split(q0.w, k, a.w, b.w);
             ff_split(q1.x, k, c.x, c.y);
             ff_split(q1.y, k, c.z, c.w);
-            o[3] = a;
-            o[4] = b;
-            o[5] = c;
+            o[4] = a;
+            o[5] = b;
+            o[6] = c;
         }
     }
 }
@@ -249,8 +269,8 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
 // Force kernel
 // ---------------------------------------------------------------------------
 
-struct FfTarget {         // limbs of the lane's two targets
-    f2x ax, ay, az, bx, by, bz, cx, cy, cz;
+struct FfTarget {         // limbs and remainders of the lane's two targets
+    f2x ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz;
 };
 
 struct FfGroup {          // per group, formed by one thread
@@ -268,17 +288,17 @@ struct FfGroup {          // per group, formed by one thread
 template <int J, int ORDER, bool FULL>
 __device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int s, int cnt, const FfTarget &T, ft (&acc)[4]) {
     for (int j = s; j < cnt; j += J) {
-        const float4 A = sT[0][j], B = sT[1][j], Cc = sT[2][j];
-        const ft d[3] = {ft_sep(dup2(A.x), dup2(B.x), dup2(Cc.x), T.ax, T.bx, T.cx),
-                         ft_sep(dup2(A.y), dup2(B.y), dup2(Cc.y), T.ay, T.by, T.cy),
-                         ft_sep(dup2(A.z), dup2(B.z), dup2(Cc.z), T.az, T.bz, T.cz)};
+        const float4 A = sT[0][j], B = sT[1][j], Cc = sT[2][j], D = sT[3][j];
+        const ft d[3] = {ft_sep(dup2(A.x), dup2(B.x), dup2(Cc.x), dup2(D.x), T.ax, T.bx, T.cx, T.dx),
+                         ft_sep(dup2(A.y), dup2(B.y), dup2(Cc.y), dup2(D.y), T.ay, T.by, T.cy, T.dy),
+                         ft_sep(dup2(A.z), dup2(B.z), dup2(Cc.z), dup2(D.z), T.az, T.bz, T.cz, T.dz)};
         const ft ri = ft_rsqrt(ft_norm2(d[0], d[1], d[2]));
         const ft m = {dup2(A.w), dup2(B.w), dup2(Cc.w)};
         const ft ri2 = FULL ? ft_mul(ri, ri) : ft_mul_cell(ri, ri), mr = FULL ? ft_mul(m, ri) : ft_mul_cell(m, ri);
         ft f = FULL ? ft_mul(mr, ri2) : ft_mul_cell(mr, ri2), pot = mr;
         ff w[3];
         if (ORDER == 2) {
-            const float4 Q = sT[3][j], Ql = sT[4][j], Q2 = sT[5][j];
+            const float4 Q = sT[4][j], Ql = sT[5][j], Q2 = sT[6][j];
             const ff xx = {dup2(Q.x), dup2(Ql.x)}, yy = {dup2(Q.y), dup2(Ql.y)}, zz = {dup2(Q.z), dup2(Ql.z)};
             const ff xy = {dup2(Q.w), dup2(Ql.w)}, xz = {dup2(Q2.x), dup2(Q2.y)}, yz = {dup2(Q2.z), dup2(Q2.w)};
             const ff r1 = {ri.h, ri.l}, r2 = {ri2.h, ri2.l};
@@ -385,11 +405,11 @@ __device__ __forceinline__ void ff_pairs(const ForceArgs &A, const FfGroup &G, c
     for (int j0 = 0; j0 < cnt; j0 += J) {         // uniform across the warp (it votes)
         const bool real = J == 1 || j0 + s < cnt;
         const int j = real ? j0 + s : j0;
-        const float4 P = sT[0][j], B = sT[1][j], Cc = sT[2][j];
+        const float4 P = sT[0][j], B = sT[1][j], Cc = sT[2][j], D = sT[3][j];
         const unsigned pj = sI[j];
-        const ft dx = ft_sep(dup2(P.x), dup2(B.x), dup2(Cc.x), T.ax, T.bx, T.cx);
-        const ft dy = ft_sep(dup2(P.y), dup2(B.y), dup2(Cc.y), T.ay, T.by, T.cy);
-        const ft dz = ft_sep(dup2(P.z), dup2(B.z), dup2(Cc.z), T.az, T.bz, T.cz);
+        const ft dx = ft_sep(dup2(P.x), dup2(B.x), dup2(Cc.x), dup2(D.x), T.ax, T.bx, T.cx, T.dx);
+        const ft dy = ft_sep(dup2(P.y), dup2(B.y), dup2(Cc.y), dup2(D.y), T.ay, T.by, T.cy, T.dy);
+        const ft dz = ft_sep(dup2(P.z), dup2(B.z), dup2(Cc.z), dup2(D.z), T.az, T.bz, T.cz, T.dz);
         ft r2 = ft_norm2(dx, dy, dz);
         const float2 rh = up2(r2.h);
         float2 q2 = rh;
@@ -417,7 +437,7 @@ __device__ __forceinline__ void ff_pairs(const ForceArgs &A, const FfGroup &G, c
 }
 
 struct FfShared {
-    float4 T[kFWarps][6][kFfTile];
+    float4 T[kFWarps][7][kFfTile];
     unsigned I[kFWarps][kFfTile];
     float W[kFWarps][kFfTile];             // 1 / s_j (mass-dependent radii)
     unsigned queue[kFWarps][kFfQueue * 32];
@@ -439,22 +459,25 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
     float invs[2];
     unsigned pid[2];
     bool valid[2];
-    float4 a[2], b[2], c[2];
+    float4 a[2], b[2], c[2], d[2];
 #pragma unroll
     for (int k = 0; k < 2; k++) {
         const unsigned idx = i0 + lane % L + L * k;
         valid[k] = idx < gr.y;
         pid[k] = gr.x + (valid[k] ? idx : 0u);
-        a[k] = A.ffp[3ull * pid[k]];
-        b[k] = A.ffp[3ull * pid[k] + 1];
-        c[k] = A.ffp[3ull * pid[k] + 2];
+        const float4 *o = A.ffp + 4ull * pid[k];
+        a[k] = o[0];
+        b[k] = o[1];
+        c[k] = o[2];
+        d[k] = o[3];
         invs[k] = MD ? A.spL[pid[k]].w : 1.0f;
 #pragma unroll
         for (int q = 0; q < 4; q++) S.D[w][k][q][lane] = 0.0;
     }
     const FfTarget T = {pk2(a[0].x, a[1].x), pk2(a[0].y, a[1].y), pk2(a[0].z, a[1].z),
                         pk2(b[0].x, b[1].x), pk2(b[0].y, b[1].y), pk2(b[0].z, b[1].z),
-                        pk2(c[0].x, c[1].x), pk2(c[0].y, c[1].y), pk2(c[0].z, c[1].z)};
+                        pk2(c[0].x, c[1].x), pk2(c[0].y, c[1].y), pk2(c[0].z, c[1].z),
+                        pk2(d[0].x, d[1].x), pk2(d[0].y, d[1].y), pk2(d[0].z, d[1].z)};
     ft acc[4];
 #pragma unroll
     for (int q = 0; q < 4; q++) acc[q] = {0ull, 0ull, 0ull};
@@ -479,9 +502,9 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
             if (t >= ce) break;
             const int cnt = (int)min(q, ce - t);
             if (lane < cnt) {
-                const float4 *o = A.ffn + 6ull * A.cells[co + t + lane];
+                const float4 *o = A.ffn + 7ull * A.cells[co + t + lane];
 #pragma unroll
-                for (int r = 0; r < (ORDER == 2 ? 6 : 3); r++) S.T[w][r][lane] = o[r];
+                for (int r = 0; r < (ORDER == 2 ? 7 : 4); r++) S.T[w][r][lane] = o[r];
             }
             __syncwarp();
             if (nc < kFfFewCells) ff_cells<J, ORDER, true>(S.T[w], s, cnt, T, acc);
@@ -504,7 +527,7 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
                 S.I[w][lane] = p;
                 if (MD) S.W[w][lane] = A.spL[p].w;
 #pragma unroll
-                for (int r = 0; r < 3; r++) S.T[w][r][lane] = A.ffp[3ull * p + r];
+                for (int r = 0; r < 4; r++) S.T[w][r][lane] = A.ffp[4ull * p + r];
             }
             __syncwarp();
             ff_pairs<J, MD>(A, G, S.T[w], S.I[w], S.W[w], s, cnt, T, invs, pid, valid, S.queue[w], qn, S.D[w], acc);

@@ -126,7 +126,7 @@ struct ForceArgs {
     const float4 *nd_f;
     const uint2 *nd_r;
     const uint4 *sq;
-    float4 *ffp, *ffn;               // float64 kernel: double-float records (3 per particle, 6 per node)
+    float4 *ffp, *ffn;               // float64 kernel: float32 expansions (4 per particle, 7 per node)
     const SetInfo *sets;
     const unsigned *perm;
     const double *ssc;               // sorted radius factors (massdep)

@@ -1,0 +1,113 @@
+"""Rounding errors of the float64 force kernel against float64 instructions.
+
+The library's own tree and lists are summed on the host twice, in extended
+precision (64 bits of significand or more) and in float64 as a float64 kernel
+sums them (four accumulators, one list entry after another).  The kernel's
+results must be no further from the extended sums than the float64 ones, in
+the root mean square and at the 99th percentile of the targets.  r_out is so
+small that no pair lies within it: those are float64 instructions anyway.
+"""
+import numpy as np
+import pytest
+
+from paper_2006_16560_gb300 import binding as B
+from paper_2006_16560_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _sums(dtype, x, cells, parts, order):
+    """Accelerations (three) and potential at x of cells (M, com, Q) and particles (m, pos)."""
+    x = x.astype(dtype)
+    M, com, Q = (v.astype(dtype) for v in cells)
+    m, pos = (v.astype(dtype) for v in parts)
+    d = com - x
+    r2 = (d * d).sum(1)
+    rinv = 1 / np.sqrt(r2)
+    f = M * rinv * rinv * rinv
+    phi = M * rinv
+    a = f[:, None] * d
+    if order == 2:
+        qd = np.stack([Q[:, 0] * d[:, 0] + Q[:, 3] * d[:, 1] + Q[:, 4] * d[:, 2],
+                       Q[:, 3] * d[:, 0] + Q[:, 1] * d[:, 1] + Q[:, 5] * d[:, 2],
+                       Q[:, 4] * d[:, 0] + Q[:, 5] * d[:, 1] + Q[:, 2] * d[:, 2]], 1)
+        r5 = rinv * rinv * rinv * rinv * rinv
+        t = (d * qd).sum(1) * r5
+        a = (f + dtype(2.5) * t * rinv * rinv)[:, None] * d - qd * r5[:, None]
+        phi = phi + t / 2
+    e = pos - x
+    s = 1 / np.sqrt((e * e).sum(1))
+    terms = np.concatenate([np.concatenate([a, (m * s * s * s)[:, None] * e]), np.concatenate([phi, m * s])[:, None]], 1)
+    if dtype is np.longdouble:
+        return terms.sum(0)
+    # entry after entry in four accumulators (64 entries each in turn), as four warps do
+    pad = np.concatenate([terms, np.zeros((-len(terms) % 256, 4))]).reshape(-1, 4, 64, 4)
+    return sum(np.cumsum(pad[:, w].reshape(-1, 4), 0)[-1] for w in range(4))
+
+
+def _errors(pos, mass, theta, order, n_leaf=16, targets=64, seed=0):
+    import torch
+    n = len(mass)
+    ctx = B.Context(0)
+    r_out = 1e-12 * float(np.ptp(pos, axis=0).max())
+    t = B.Tree(ctx, torch.from_numpy(np.ascontiguousarray(pos)).cuda(), torch.from_numpy(mass).cuda(),
+               B.Params(theta=theta, r_in=0.1 * r_out, r_out=r_out, n_leaf=n_leaf, n_group=64, order=order,
+                        precision=B.PT_FP64))
+    acc = torch.empty((n, 3), dtype=torch.float64, device="cuda")
+    pot = torch.empty(n, dtype=torch.float64, device="cuda")
+    off = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+    idx = torch.empty(64, dtype=torch.int32, device="cuda")
+    total, st, _ = t.force(acc, pot, off, idx, 64)
+    assert total == 0
+    got = np.concatenate([acc.cpu().numpy(), -pot.cpu().numpy()[:, None]], 1)
+    nodes, groups, (_, perm) = t.nodes(), t.groups(), t.keys()
+    co, cells, po, pp = t.lists(st.cell_list_total, st.pp_list_total)
+    ps, ms = pos[perm], mass[perm]
+    at = np.sort(np.random.default_rng(seed).choice(n, targets, replace=False))
+    err = {"kernel": [], "float64": []}
+    longest = 0
+    for k in at:
+        g = int(np.searchsorted(groups["begin"], k, side="right")) - 1
+        c, p = cells[co[g]:co[g + 1]], pp[po[g]:po[g + 1]]
+        p = p[p != k]
+        longest = max(longest, len(c))
+        lists = ((nodes["mass"][c], nodes["com"][c], nodes["quad"][c]), (ms[p], ps[p]))
+        ref = _sums(np.longdouble, ps[k], *lists, order)
+        for name, v in (("kernel", got[perm[k]]), ("float64", _sums(np.float64, ps[k], *lists, order))):
+            d = v.astype(np.longdouble) - ref
+            err[name].append((float(np.sqrt((d[:3] ** 2).sum() / (ref[:3] ** 2).sum())), float(abs(d[3] / ref[3]))))
+    t.free()
+    ctx.close()
+    return np.array(err["kernel"]), np.array(err["float64"]), longest
+
+
+def _assert_no_further(pos, mass, *args, **kw):
+    k, f, longest = _errors(pos, mass, *args, **kw)
+    rms, p99 = (lambda e: np.sqrt((e * e).mean(0))), (lambda e: np.percentile(e, 99, axis=0))
+    print("rms", rms(k), "float64", rms(f), "p99", p99(k), "float64", p99(f))
+    assert (rms(k) <= rms(f)).all() and (p99(k) <= p99(f)).all()
+    return longest
+
+
+@pytest.mark.parametrize("order", [0, 2])
+@pytest.mark.parametrize("reach", [1e2, 1e3, 1e4, 1e5, 1e6])
+def test_core_with_an_escaper(order, reach):
+    """A core of unit size around the origin and one particle `reach` away, which sets the box."""
+    d = inputs.plummer(3000, 5, masses="kroupa")
+    pos = d["pos"].copy()
+    pos[0] = [reach, 0.3 * reach, -0.1 * reach]
+    _assert_no_further(pos, d["mass"], 0.4, order)
+
+
+@pytest.mark.parametrize("shift", [(1e6, 0.0, 0.0), (0.0, -1e9, 1e3), (2e5, 2e5, 2e5)])
+def test_sets_far_from_the_origin(shift):
+    """Each axis by itself: coordinates near zero on one beside large ones on another."""
+    d = inputs.plummer(2000, 6, masses="kroupa")
+    _assert_no_further(d["pos"] + np.array(shift), d["mass"], 0.5, 2)
+
+
+def test_flat_set():
+    """A disc a millionth as thick as wide."""
+    rng = np.random.default_rng(8)
+    pos = rng.normal(size=(3000, 3)) * np.array([1.0, 1.0, 1e-6])
+    _assert_no_further(pos, rng.uniform(0.5, 1.5, 3000) / 3000, 0.5, 2)
