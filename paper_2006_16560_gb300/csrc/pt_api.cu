@@ -344,7 +344,7 @@ int alloc_build(pt_tree *t, unsigned n, int nsets) {
     TRY(ensure(ctx, t->ssc, N * 8));
     if (t->prm.precision == PT_FP64) {       // records of the float64 force kernel
         TRY(ensure(ctx, t->ffp, N * 64));
-        TRY(ensure(ctx, t->ffn, C * 112));
+        TRY(ensure(ctx, t->ffn, C * 144));
     }
     TRY(ensure(ctx, t->set_mean, S * 8));
     if (t->prm.mass_dependent) {
@@ -600,6 +600,7 @@ ForceArgs force_args(pt_tree *t, double *acc, double *pot, bool want_nb) {
     A.acc = acc;
     A.pot = pot;
     A.G = t->prm.G;
+    A.theta = t->prm.theta;
     A.order = t->prm.order;
     A.want_nb = want_nb ? 1 : 0;
     A.pairs = t->pairs.as<uint2>();

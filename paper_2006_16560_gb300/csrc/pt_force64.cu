@@ -7,7 +7,8 @@
 // apart than its changeover radius -- all cells and all but a few particle
 // pairs -- is evaluated in unevaluated sums of two or three float32 built
 // from error-free transformations (Knuth's TwoSum, Dekker's FastTwoSum, FMA
-// products): ~600 float32 instructions per cell and ~410 per particle pair.
+// products): 655 float32 operations per cell (414 without a quadrupole, 1,326
+// at wide opening angles, see kFfQuad2Theta) and 414 per particle pair.
 // Only pairs within r_out, whose changeover and neighbour test are defined in
 // float64 operations, take float64 instructions.
 //
@@ -21,15 +22,17 @@
 // instructions and 2e-16 with the remainder.)  Limb differences are
 // exact, so the separation of a pair or of a cell evaluated here (2^-23 box
 // sides or more) is correct to ~2^-63 of itself wherever the group lies.
-// r^2, 1/r and
-// the products and sums of particle pairs and of short cell lists keep three
-// float32 (~2^-64); in a list of thousands of cells each cell's products keep
-// two and a half (~2^-49, averaged over the list), and a quadrupole term, at
-// most a few percent of its cell's monopole, always two.  The
-// sums are folded into float64 every 64 list entries.  Two float32 throughout
-// (~2^-47 per pair) were measured first: three times faster on the same
-// lists, but with results 2-5 times further from an extended-precision sum
-// than float64 instructions give, and so not used.
+// r^2, 1/r and the products and sums of cells and pairs keep three float32
+// (~2^-64).  Products of two and a half (~2^-49) in lists of thousands of cells
+// were used at first: their rounding averages out in a Plummer sphere, but not
+// where one cell is most of the sum (a body with half the mass in 60,000: p99
+// 4.9e-15 against 2.5e-15 with float64 instructions, 3.1e-16 with three words;
+// the force of 150,001 particles takes 27.4 ms instead of 25.1).  Quadrupole
+// terms keep two words (~2^-47 of the term) up to an opening angle of 0.6,
+// where they are a fraction of their cells' monopoles, and three above it.
+// The sums are folded into float64 every 64 list entries.  Two float32
+// throughout (~2^-47 per pair) were measured first, with results 2-5 times
+// further from an extended-precision sum than float64 instructions give.
 //
 // Lengths are scaled by the power of two at or above the root box side and
 // masses by that of the set's mass, so no power up to r^-5 leaves float32's
@@ -41,8 +44,14 @@ namespace pt {
 
 constexpr int kFfTile = 32;        // list entries per warp tile: one gathered by each lane
 constexpr int kFfFold = 2;         // tiles between folds of the float32 sums into float64
-constexpr unsigned kFfFewCells = 4096;   // cell lists below this take the full products (see ff_cells)
 constexpr int kFfQueue = 8;        // near pairs a lane may hold before the warp evaluates them
+// Opening angles up to this take quadrupole terms in two words: rms errors of
+// accelerations 0.3 to 0.7 of float64 instructions' in sets of massive pairs whose
+// quadrupoles dominate (theta 0.3 to 0.6), but 1.3 times at 1.0, and 15 times in
+// a Plummer sphere at 1.5, where cells' quadrupoles reach their monopoles.  Three
+// words: 0.2 at any angle, at twice the operations (force of 100,003 Plummer
+// particles at theta 1.0: 3.3 ms, 2.0 with two words, 31 with float64 instructions).
+constexpr double kFfQuad2Theta = 0.6;
 constexpr float kFfTinyR2 = 0x1p-46f;   // smallest scaled r^2 evaluated in float32 expansions
 
 // Every value is a packed pair (f32x2), one for each of a lane's two targets:
@@ -96,21 +105,15 @@ __device__ __forceinline__ ft ft_mul(ft a, ft b) {
     const ff s = ff_fast(x.h, x.l);
     return {s.h, s.l, x.e};
 }
-// the same with the cross terms rounded (~2^-49): cells
-__device__ __forceinline__ ft ft_mul_cell(ft a, ft b) {
-    const ff p = ff_prod(a.h, b.h), d = ff_two_sum(p.l, fma2(a.l, b.h, mul2(a.h, b.l)));
-    const ff s = ff_fast(p.h, d.h);
-    return {s.h, s.l, fma2(a.h, b.e, fma2(a.e, b.h, fma2(a.l, b.l, d.l)))};
+__device__ __forceinline__ ft ft_sum3(ft x, ft y, ft z) {
+    const ff s = ff_two_sum(x.h, y.h), t = ff_two_sum(s.h, z.h), a = ff_two_sum(x.l, y.l), b = ff_two_sum(z.l, s.l);
+    const ff c = ff_two_sum(a.h, b.h), g = ff_two_sum(c.h, t.l), r = ff_fast(t.h, g.h);
+    return {r.h, r.l, add2(add2(add2(x.e, y.e), z.e), add2(add2(a.l, b.l), add2(c.l, g.l)))};
 }
 // running sum of x.h + x.l + x.e
 __device__ __forceinline__ void ft_acc(ft &a, ft x) {
     const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l), u = ff_two_sum(t.h, x.l);
     a = {s.h, u.h, add2(a.e, add2(add2(t.l, u.l), x.e))};
-}
-// the same with x.l added to the third word (~2^-49 of x): cells
-__device__ __forceinline__ void ft_acc_cell(ft &a, ff x) {
-    const ff s = ff_two_sum(a.h, x.h), t = ff_two_sum(a.l, s.l);
-    a = {s.h, t.h, add2(a.e, add2(t.l, x.l))};
 }
 // float32 to float64 on the integer pipe (finite values; subnormals are 0)
 __device__ __forceinline__ double ff_widen(float f) {
@@ -219,7 +222,10 @@ __device__ __forceinline__ float ff_split(double v, int k, float &h, float &l) {
     return __double2float_rn((w - (double)h) - (double)l);
 }
 
-__global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
+// Rows (float4) of a cell's record, by the float32 words of its quadrupole.
+__host__ __device__ constexpr int ff_rows(int quad) { return quad == 0 ? 4 : quad == 2 ? 7 : 9; }
+
+__global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n, int quad) {
     const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
     for (unsigned p = t0; p < n; p += dt) {
         const unsigned set = A.sq[p].w;
@@ -244,23 +250,28 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n) {
         ff_position(P, u, a, b, c, d);
         c.w = ff_split(P.w, -u.em, a.w, b.w);
         d.w = 0.0f;
-        float4 *o = A.ffn + 7ull * v;
+        float4 *o = A.ffn + (size_t)ff_rows(quad) * v;
         o[0] = a;
         o[1] = b;
         o[2] = c;
         o[3] = d;
-        if (A.order == 2) {                  // Qxx Qyy Qzz Qxy | their low parts | Qxz, Qyz (high, low)
+        if (quad) {          // Qxx Qyy Qzz Qxy | their low parts | Qxz, Qyz (high, low) | third words
             const double4 q0 = A.nd_q[2 * v], q1 = A.nd_q[2 * v + 1];
             const int k = -u.em - 2 * u.es;
-            ff_split(q0.x, k, a.x, b.x);
-            ff_split(q0.y, k, a.y, b.y);
-            ff_split(q0.z, k, a.z, b.z);
-            ff_split(q0.w, k, a.w, b.w);
-            ff_split(q1.x, k, c.x, c.y);
-            ff_split(q1.y, k, c.z, c.w);
+            float4 e, g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            e.x = ff_split(q0.x, k, a.x, b.x);
+            e.y = ff_split(q0.y, k, a.y, b.y);
+            e.z = ff_split(q0.z, k, a.z, b.z);
+            e.w = ff_split(q0.w, k, a.w, b.w);
+            g.x = ff_split(q1.x, k, c.x, c.y);
+            g.y = ff_split(q1.y, k, c.z, c.w);
             o[4] = a;
             o[5] = b;
             o[6] = c;
+            if (quad == 3) {
+                o[7] = e;
+                o[8] = g;
+            }
         }
     }
 }
@@ -280,12 +291,22 @@ struct FfGroup {          // per group, formed by one thread
     Chg C;
 };
 
+// The three words of a cell's quadrupole.
+__device__ __forceinline__ void ff_quad3(const float4 (*sT)[kFfTile], int j, ft (&Q)[6]) {
+    const float4 a = sT[4][j], b = sT[5][j], c = sT[6][j], e = sT[7][j], g = sT[8][j];
+    Q[0] = {dup2(a.x), dup2(b.x), dup2(e.x)};
+    Q[1] = {dup2(a.y), dup2(b.y), dup2(e.y)};
+    Q[2] = {dup2(a.z), dup2(b.z), dup2(e.z)};
+    Q[3] = {dup2(a.w), dup2(b.w), dup2(e.w)};
+    Q[4] = {dup2(c.x), dup2(c.y), dup2(g.x)};
+    Q[5] = {dup2(c.z), dup2(c.w), dup2(g.y)};
+}
+
 // A cell: a += (m/r^3 + 5/2 q/r^5) d - Q u/r^4, P += m/r + 1/2 q/r^3, with
 // u = d/r and q = u.Q.u (the unit-vector form keeps Q's products in range).
-// FULL: the monopole keeps three float32 throughout (short lists, whose few
-// terms do not average the cheaper products' rounding).
+// QUAD: float32 words of the quadrupole terms (0: none).
 // The lane takes cells s, s + J, .. of the tile.
-template <int J, int ORDER, bool FULL>
+template <int J, int QUAD>
 __device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int s, int cnt, const FfTarget &T, ft (&acc)[4]) {
     for (int j = s; j < cnt; j += J) {
         const float4 A = sT[0][j], B = sT[1][j], Cc = sT[2][j], D = sT[3][j];
@@ -294,16 +315,16 @@ __device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int s, int
                          ft_sep(dup2(A.z), dup2(B.z), dup2(Cc.z), dup2(D.z), T.az, T.bz, T.cz, T.dz)};
         const ft ri = ft_rsqrt(ft_norm2(d[0], d[1], d[2]));
         const ft m = {dup2(A.w), dup2(B.w), dup2(Cc.w)};
-        const ft ri2 = FULL ? ft_mul(ri, ri) : ft_mul_cell(ri, ri), mr = FULL ? ft_mul(m, ri) : ft_mul_cell(m, ri);
-        ft f = FULL ? ft_mul(mr, ri2) : ft_mul_cell(mr, ri2), pot = mr;
-        ff w[3];
-        if (ORDER == 2) {
+        const ft ri2 = ft_mul(ri, ri), mr = ft_mul(m, ri);
+        ft f = ft_mul(mr, ri2), pot = mr;
+        if (QUAD == 2) {
             const float4 Q = sT[4][j], Ql = sT[5][j], Q2 = sT[6][j];
             const ff xx = {dup2(Q.x), dup2(Ql.x)}, yy = {dup2(Q.y), dup2(Ql.y)}, zz = {dup2(Q.z), dup2(Ql.z)};
             const ff xy = {dup2(Q.w), dup2(Ql.w)}, xz = {dup2(Q2.x), dup2(Q2.y)}, yz = {dup2(Q2.z), dup2(Q2.w)};
             const ff r1 = {ri.h, ri.l}, r2 = {ri2.h, ri2.l};
             const ff ux = ff_mul({d[0].h, d[0].l}, r1), uy = ff_mul({d[1].h, d[1].l}, r1);
             const ff uz = ff_mul({d[2].h, d[2].l}, r1);
+            ff w[3];
             w[0] = ff_sum3(ff_mul(xx, ux), ff_mul(xy, uy), ff_mul(xz, uz));
             w[1] = ff_sum3(ff_mul(xy, ux), ff_mul(yy, uy), ff_mul(yz, uz));
             w[2] = ff_sum3(ff_mul(xz, ux), ff_mul(yz, uy), ff_mul(zz, uz));
@@ -320,29 +341,38 @@ __device__ __forceinline__ void ff_cells(const float4 (*sT)[kFfTile], int s, int
             f = {h.h, h.l, add2(f.e, z.l)};
             const ff r4 = ff_mul(r2, r2);
 #pragma unroll
-            for (int c = 0; c < 3; c++) w[c] = ff_mul(w[c], r4);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            if (FULL) {
-                ft x = ft_mul_raw(f, d[c]);
-                if (ORDER == 2) {
-                    const ff s2 = ff_two_sum(x.h, neg2(w[c].h)), v = ff_two_sum(x.l, sub2(s2.l, w[c].l));
-                    x = {s2.h, v.h, add2(x.e, v.l)};
-                }
-                ft_acc(acc[c], x);
-            } else {
-                const ff p = ff_prod(f.h, d[c].h);
-                ff x = {p.h, fma2(f.l, d[c].h, fma2(f.h, d[c].l, fma2(f.h, d[c].e, fma2(f.e, d[c].h, p.l))))};
-                if (ORDER == 2) {
-                    const ff s2 = ff_two_sum(p.h, neg2(w[c].h));
-                    x = {s2.h, add2(x.l, sub2(s2.l, w[c].l))};
-                }
-                ft_acc_cell(acc[c], x);
+            for (int c = 0; c < 3; c++) {
+                const ff y = ff_mul(w[c], r4);
+                const ft x = ft_mul_raw(f, d[c]);
+                const ff e = ff_two_sum(x.h, neg2(y.h)), v2 = ff_two_sum(x.l, sub2(e.l, y.l));
+                ft_acc(acc[c], {e.h, v2.h, add2(x.e, v2.l)});
             }
+        } else if (QUAD == 3) {
+            ft Q[6];                                                         // xx yy zz xy xz yz
+            ff_quad3(sT, j, Q);
+            const ft u[3] = {ft_mul(d[0], ri), ft_mul(d[1], ri), ft_mul(d[2], ri)};
+            const ft w[3] = {ft_sum3(ft_mul(Q[0], u[0]), ft_mul(Q[3], u[1]), ft_mul(Q[4], u[2])),
+                             ft_sum3(ft_mul(Q[3], u[0]), ft_mul(Q[1], u[1]), ft_mul(Q[5], u[2])),
+                             ft_sum3(ft_mul(Q[4], u[0]), ft_mul(Q[5], u[1]), ft_mul(Q[2], u[2]))};
+            const ft q3 = ft_mul(ft_sum3(ft_mul(u[0], w[0]), ft_mul(u[1], w[1]), ft_mul(u[2], w[2])), ft_mul(ri2, ri));
+            const f2x half = dup2(0.5f);
+            ft_acc(pot, {mul2(half, q3.h), mul2(half, q3.l), mul2(half, q3.e)});
+            ft_acc(f, ft_mul({dup2(2.5f), 0ull, 0ull}, ft_mul(q3, ri2)));    // 5/2 q / r^5
+            const ff h = ff_fast(f.h, f.l);
+            f = {h.h, h.l, f.e};
+            const ft r4 = ft_mul(ri2, ri2);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const ft y = ft_mul(w[c], r4);
+                ft x = ft_mul_raw(f, d[c]);
+                ft_acc(x, {neg2(y.h), neg2(y.l), neg2(y.e)});
+                ft_acc(acc[c], x);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 3; c++) ft_acc(acc[c], ft_mul_raw(f, d[c]));
         }
-        if (FULL) ft_acc(acc[3], pot);
-        else ft_acc_cell(acc[3], {pot.h, add2(pot.l, pot.e)});
+        ft_acc(acc[3], pot);
     }
 }
 
@@ -436,8 +466,9 @@ __device__ __forceinline__ void ff_pairs(const ForceArgs &A, const FfGroup &G, c
     }
 }
 
+template <int QUAD>
 struct FfShared {
-    float4 T[kFWarps][7][kFfTile];
+    float4 T[kFWarps][ff_rows(QUAD)][kFfTile];
     unsigned I[kFWarps][kFfTile];
     float W[kFWarps][kFfTile];             // 1 / s_j (mass-dependent radii)
     unsigned queue[kFWarps][kFfQueue * 32];
@@ -451,9 +482,9 @@ struct FfShared {
 // sub-streams that take every J-th list entry, so that a group of few targets
 // still fills them.  Every warp takes every fourth tile of each list segment.
 // Leaves the lanes' float64 sums in S.D.
-template <int J, int ORDER, bool MD>
+template <int J, int QUAD, bool MD>
 __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const uint2 gr, unsigned i0, unsigned lo,
-                                        unsigned hi, FfShared &S) {
+                                        unsigned hi, FfShared<QUAD> &S) {
     constexpr int L = 32 / J;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, s = lane / L;
     float invs[2];
@@ -502,13 +533,12 @@ __device__ __forceinline__ void ff_pass(const ForceArgs &A, unsigned g, const ui
             if (t >= ce) break;
             const int cnt = (int)min(q, ce - t);
             if (lane < cnt) {
-                const float4 *o = A.ffn + 7ull * A.cells[co + t + lane];
+                const float4 *o = A.ffn + (size_t)ff_rows(QUAD) * A.cells[co + t + lane];
 #pragma unroll
-                for (int r = 0; r < (ORDER == 2 ? 7 : 4); r++) S.T[w][r][lane] = o[r];
+                for (int r = 0; r < ff_rows(QUAD); r++) S.T[w][r][lane] = o[r];
             }
             __syncwarp();
-            if (nc < kFfFewCells) ff_cells<J, ORDER, true>(S.T[w], s, cnt, T, acc);
-            else ff_cells<J, ORDER, false>(S.T[w], s, cnt, T, acc);
+            ff_cells<J, QUAD>(S.T[w], s, cnt, T, acc);
             __syncwarp();
             if (++tiles % kFfFold == 0) fold();
         }
@@ -554,9 +584,9 @@ __device__ __forceinline__ void ff_write(const ForceArgs &A, unsigned p, const d
     ep[3] += m * az;
 }
 
-template <int ORDER, bool MD, bool TAIL>
+template <int QUAD, bool MD, bool TAIL>
 __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
-    __shared__ FfShared S;
+    __shared__ FfShared<QUAD> S;
     // lists left unusable by the build or the walk (one-pass arrays exhausted,
     // stack overflow): do nothing, the host reports it or runs them again
     if (A.st->flags & (kErrBuild | kErrListCap | kErrStack | kErrItemCap)) return;
@@ -604,9 +634,9 @@ __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
         const unsigned t = threadIdx.x;
         for (unsigned i0 = 0; i0 < gr.y;) {
             const unsigned left = gr.y - i0, L = left > 32 ? 32u : left > 16 ? 16u : 8u;     // targets per sub-stream / 2
-            if (L == 32) ff_pass<1, ORDER, MD>(A, g, gr, i0, lo, hi, S);
-            else if (L == 16) ff_pass<2, ORDER, MD>(A, g, gr, i0, lo, hi, S);
-            else ff_pass<4, ORDER, MD>(A, g, gr, i0, lo, hi, S);
+            if (L == 32) ff_pass<1, QUAD, MD>(A, g, gr, i0, lo, hi, S);
+            else if (L == 16) ff_pass<2, QUAD, MD>(A, g, gr, i0, lo, hi, S);
+            else ff_pass<4, QUAD, MD>(A, g, gr, i0, lo, hi, S);
             __syncthreads();
             if (t < 2 * L && t < left) {                     // fixed-order sums over warps and sub-streams
                 double s[4] = {0, 0, 0, 0};
@@ -632,21 +662,19 @@ __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
     }
 }
 
-template <bool TAIL>
+template <int QUAD, bool TAIL>
 static void force64_t(const ForceArgs &A, int blocks, cudaStream_t st) {
-    if (A.order == 2) {
-        if (A.massdep) k_force_ff<2, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        else k_force_ff<2, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-    } else {
-        if (A.massdep) k_force_ff<0, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-        else k_force_ff<0, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
-    }
+    if (A.massdep) k_force_ff<QUAD, true, TAIL><<<blocks, kFThreads, 0, st>>>(A);
+    else k_force_ff<QUAD, false, TAIL><<<blocks, kFThreads, 0, st>>>(A);
 }
 
 int force64_launch(const ForceArgs &A, unsigned n, int blocks, cudaStream_t st) {
-    k_ff_records<<<sm_count() * 8, 256, 0, st>>>(A, n);
-    if (A.count_hint && A.direct_items) force64_t<true>(A, blocks, st);
-    else force64_t<false>(A, blocks, st);
+    const int quad = A.order == 0 ? 0 : A.theta <= kFfQuad2Theta ? 2 : 3;
+    const bool tail = A.count_hint && A.direct_items;
+    k_ff_records<<<sm_count() * 8, 256, 0, st>>>(A, n, quad);
+    if (quad == 0) tail ? force64_t<0, true>(A, blocks, st) : force64_t<0, false>(A, blocks, st);
+    else if (quad == 2) tail ? force64_t<2, true>(A, blocks, st) : force64_t<2, false>(A, blocks, st);
+    else tail ? force64_t<3, true>(A, blocks, st) : force64_t<3, false>(A, blocks, st);
     return 2;
 }
 

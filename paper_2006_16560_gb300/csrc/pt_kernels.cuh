@@ -133,6 +133,7 @@ struct ForceArgs {
     int massdep;
     double *acc, *pot;               // input (caller) order, device
     double G;
+    double theta;                    // opening angle of the lists
     int order;                       // 0 or 2
     int want_nb;
     uint2 *pairs;                    // (sorted i, sorted j)

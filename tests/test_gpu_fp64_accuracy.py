@@ -111,3 +111,33 @@ def test_flat_set():
     rng = np.random.default_rng(8)
     pos = rng.normal(size=(3000, 3)) * np.array([1.0, 1.0, 1e-6])
     _assert_no_further(pos, rng.uniform(0.5, 1.5, 3000) / 3000, 0.5, 2)
+
+
+@pytest.mark.parametrize("theta", [0.3, 0.5, 0.6, 0.61, 0.8, 1.0, 1.5])
+def test_massive_pairs_at_any_opening_angle(theta):
+    """Quadrupoles that dominate: pairs of massive bodies, one cell each, and wide opening angles."""
+    d = inputs.plummer(20000, 3, masses="kroupa")
+    rng = np.random.default_rng(7)
+    pos, mass = d["pos"].copy(), d["mass"].copy()
+    for b in range(6):
+        v = rng.normal(size=3)
+        v *= 10.0 ** rng.uniform(-2.0, -0.3) / np.linalg.norm(v)
+        c = rng.normal(size=3)
+        pos[2 * b], pos[2 * b + 1] = c + v / 2, c - v / 2
+        mass[2 * b] = mass[2 * b + 1] = 0.3
+    _assert_no_further(pos, mass, theta, 2, targets=160)
+
+
+@pytest.mark.parametrize("order", [0, 2])
+def test_one_body_outweighs_a_long_list(order):
+    """Thousands of cells, one of which is most of the sum: its rounding is not averaged."""
+    d = inputs.plummer(60000, 4, masses="kroupa")
+    pos, mass = d["pos"].copy(), d["mass"].copy()
+    pos[0], mass[0] = [0.3, 0.1, -0.2], 1.0
+    assert _assert_no_further(pos, mass, 0.2, order, targets=32) > 5000
+
+
+def test_plummer_spheres_of_the_usual_parameters():
+    for n, theta, order in ((1000, 0.5, 0), (4096, 0.5, 0), (20000, 0.3, 2), (60000, 0.6, 2)):
+        d = inputs.plummer(n, n, masses="kroupa")
+        _assert_no_further(d["pos"], d["mass"], theta, order, n_leaf=8)
