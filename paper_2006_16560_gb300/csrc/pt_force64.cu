@@ -287,7 +287,7 @@ struct FfTarget {         // limbs and remainders of the lane's two targets
 struct FfGroup {          // per group, formed by one thread
     float hit2;           // scaled (r_out (1 + 2^-18))^2: a pair at or above it is outside r_out
     double sa, sp;        // units of acceleration (mass / length^2) and potential (mass / length)
-    double ua, up;        // 1 / sa, 1 / sp
+    double ua, up;        // 1 / sa, 1 / sp (at most 2^1023)
     Chg C;
 };
 
@@ -625,8 +625,10 @@ __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
             G.hit2 = __double2float_ru(fmin(h * h, 1e30));
             G.sa = scalbn(1.0, u.em - 2 * u.es);
             G.sp = scalbn(1.0, u.em - u.es);
-            G.ua = scalbn(1.0, 2 * u.es - u.em);
-            G.up = scalbn(1.0, u.es - u.em);
+            // finite: where the units' accelerations or potentials underflow, so do the near
+            // pairs' and zero times infinity must not come of it
+            G.ua = scalbn(1.0, min(2 * u.es - u.em, 1023));
+            G.up = scalbn(1.0, min(u.es - u.em, 1023));
             S.G = G;
         }
         __syncthreads();

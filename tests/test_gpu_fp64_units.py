@@ -68,3 +68,21 @@ def test_list_and_pass_edges(n, r_out):
         np.testing.assert_allclose(p, po, rtol=1e-10)
         oo, oi = oracle.neighbours(d["pos"], r_out)
         assert np.array_equal(off, oo) and np.array_equal(idx, oi)
+
+
+@pytest.mark.parametrize("k,j", [(400, -300), (480, -100), (320, -760)])
+def test_units_below_the_smallest_number(k, j):
+    """Units in which accelerations or potentials fall below float64's range: zero, as with
+    float64 instructions, not infinity times zero (near pairs are scaled by 1 / unit)."""
+    d = inputs.plummer(500, 5, masses="kroupa")
+    kw = dict(theta=0.5, n_leaf=8, n_group=64, order=2)
+    _, p0, o0, i0 = _run(d["pos"], d["mass"], r_in=0.05, r_out=0.5, **kw)
+    s = 2.0 ** k
+    a, p, o, i = _run(d["pos"] * s, d["mass"] * 2.0 ** j, r_in=0.05 * s, r_out=0.5 * s, **kw)
+    assert len(i0) > 500 and np.array_equal(o, o0) and np.array_equal(i, i0)
+    assert np.isfinite(a).all() and np.isfinite(p).all()
+    assert np.abs(a).max() <= 1e-300
+    if k - j < 1000:
+        assert np.array_equal(p, p0 * 2.0 ** (j - k))
+    else:
+        assert np.abs(p).max() <= 1e-300
