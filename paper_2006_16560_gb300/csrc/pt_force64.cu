@@ -35,9 +35,10 @@
 // further from an extended-precision sum than float64 instructions give.
 //
 // Lengths are scaled by the power of two at or above the root box side and
-// masses by that of the set's mass, so no power up to r^-5 leaves float32's
-// range whatever the caller's units: separations below 2^-23 box sides go to
-// the float64 path, and accepted cells are at least a grid cell (2^-21) away.
+// masses by one near the set's mass (see FfUnits), so no power up to r^-5
+// leaves float32's range whatever the caller's units: separations below 2^-23
+// box sides go to the float64 path, and accepted cells are at least a grid
+// cell (2^-21) away.
 #include "pt_force.cuh"
 
 namespace pt {
@@ -178,11 +179,15 @@ __device__ __forceinline__ ft ft_rsqrt(ft r2) {
 
 // Exponents of a set's units: 2^ex above every |coordinate| of an axis, lengths
 // in 2^es >= box side (for coincident particles, whose box side is a stand-in,
-// not below 2^(ex - 60): the limbs then stay in range), masses in 2^em.
+// not below 2^(ex - 60): the limbs then stay in range), masses in 2^em: the
+// set's mass is 2^50, so that bodies down to 1e-36 of it keep all their words
+// above float32's smallest number, and cells' m / r^3 below its largest (2^119
+// at 2^-23 box sides); 2^16 with opening angles above kFfQuad2Theta, where a
+// cell as wide as the box may be accepted at 2^-21 of it (Q / r^5 ~ 2^123).
 struct FfUnits {
     int ex[3], es, em;
 };
-__device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M) {
+__device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M, int quad) {
     FfUnits u;
     u.es = ilogb(S.S) + 1;
 #pragma unroll
@@ -191,7 +196,7 @@ __device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M) {
         u.ex[d] = ilogb(X) + 1;
         u.es = max(u.es, u.ex[d] - 60);
     }
-    u.em = M > 0.0 ? ilogb(M) + 1 : 0;
+    u.em = M > 0.0 ? ilogb(M) + 1 - (quad == 3 ? 16 : 50) : 0;
     return u;
 }
 
@@ -229,7 +234,7 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n, int
     const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
     for (unsigned p = t0; p < n; p += dt) {
         const unsigned set = A.sq[p].w;
-        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
+        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w, quad);
         const double4 P = A.sp64[p];
         float4 a, b, c, d;
         ff_position(P, u, a, b, c, d);
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__(256) k_ff_records(ForceArgs A, unsigned n, int
     const unsigned nn = A.st->nnodes;
     for (unsigned v = t0; v < nn; v += dt) {
         const unsigned set = A.sq[A.nd_r[v].x].w;
-        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w);
+        const FfUnits u = ff_units(A.sets[set], A.nd_c[set].w, quad);
         const double4 P = A.nd_c[v];
         float4 a, b, c, d;
         ff_position(P, u, a, b, c, d);
@@ -618,7 +623,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_force_ff(ForceArgs A) {
         const uint2 gr = A.gr_r[g];
         if (threadIdx.x == 0) {
             const SetInfo &I = A.sets[A.gr_a[g].w];
-            const FfUnits u = ff_units(I, A.nd_c[A.gr_b[g].w].w);
+            const FfUnits u = ff_units(I, A.nd_c[A.gr_b[g].w].w, QUAD);
             FfGroup G;
             G.C = make_chg(I);
             const double h = scalbn(I.r_out, -u.es) * (1.0 + 0x1p-18);

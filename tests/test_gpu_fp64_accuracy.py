@@ -45,7 +45,7 @@ def _sums(dtype, x, cells, parts, order):
     return sum(np.cumsum(pad[:, w].reshape(-1, 4), 0)[-1] for w in range(4))
 
 
-def _errors(pos, mass, theta, order, n_leaf=16, targets=64, seed=0):
+def _errors(pos, mass, theta, order, n_leaf=16, targets=64, seed=0, only=None):
     import torch
     n = len(mass)
     ctx = B.Context(0)
@@ -64,6 +64,8 @@ def _errors(pos, mass, theta, order, n_leaf=16, targets=64, seed=0):
     co, cells, po, pp = t.lists(st.cell_list_total, st.pp_list_total)
     ps, ms = pos[perm], mass[perm]
     at = np.sort(np.random.default_rng(seed).choice(n, targets, replace=False))
+    if only is not None:
+        at = np.nonzero(perm == only)[0]
     err = {"kernel": [], "float64": []}
     longest = 0
     for k in at:
@@ -81,11 +83,15 @@ def _errors(pos, mass, theta, order, n_leaf=16, targets=64, seed=0):
     return np.array(err["kernel"]), np.array(err["float64"]), longest
 
 
-def _assert_no_further(pos, mass, *args, **kw):
-    k, f, longest = _errors(pos, mass, *args, **kw)
+def _assert_errors_no_larger(k, f):
     rms, p99 = (lambda e: np.sqrt((e * e).mean(0))), (lambda e: np.percentile(e, 99, axis=0))
     print("rms", rms(k), "float64", rms(f), "p99", p99(k), "float64", p99(f))
     assert (rms(k) <= rms(f)).all() and (p99(k) <= p99(f)).all()
+
+
+def _assert_no_further(pos, mass, *args, **kw):
+    k, f, longest = _errors(pos, mass, *args, **kw)
+    _assert_errors_no_larger(k, f)
     return longest
 
 
@@ -141,3 +147,19 @@ def test_plummer_spheres_of_the_usual_parameters():
     for n, theta, order in ((1000, 0.5, 0), (4096, 0.5, 0), (20000, 0.3, 2), (60000, 0.6, 2)):
         d = inputs.plummer(n, n, masses="kroupa")
         _assert_no_further(d["pos"], d["mass"], theta, order, n_leaf=8)
+
+
+@pytest.mark.parametrize("light", [1e-12, 1e-24, 1e-31])
+def test_light_bodies_around_a_heavy_one(light):
+    """The heavy body's own acceleration comes from bodies many orders lighter."""
+    kernel, plain = [], []
+    for body in range(17, 33):
+        d = inputs.plummer(3000, 11, masses="kroupa")
+        pos, mass = d["pos"].copy(), light * d["mass"]
+        mass[body] = 1.0
+        if body == 17:
+            pos[body] = [0.01, -0.02, 0.03]
+        k, f, _ = _errors(pos, mass, 0.5, 2, only=body)
+        kernel.append(k[0])
+        plain.append(f[0])
+    _assert_errors_no_larger(np.array(kernel), np.array(plain))
