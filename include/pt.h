@@ -134,7 +134,8 @@ typedef struct {
                                    when any of its pairs is within r_out); the
                                    others used the plain Newtonian pair, which
                                    is exact beyond r_out (K = W = 0)         */
-    int64_t max_walk_stack;     /* deepest walk stack (pending nodes per warp) */
+    int64_t max_walk_stack;     /* deepest walk stack (pending nodes per warp; of
+                                   a group walked by a block its warps' share) */
     int64_t launches_build;     /* kernels launched by the last tree build   */
     int64_t launches_force;     /* kernels launched by the force call        */
 } pt_stats;

@@ -240,7 +240,8 @@ __device__ __noinline__ void walk_block(const WalkArgs &A, unsigned g, const lon
     }
     if (threadIdx.x == 0) {
         if (overflow) atomicOr(&A.st->flags, kErrStack);
-        if (!FILL || ONEPASS) atomicMax(&A.st->max_stack, (unsigned)max_sp);
+        // per warp, as an ordinary group's
+        if (!FILL || ONEPASS) atomicMax(&A.st->max_stack, (unsigned)(max_sp + kWalkWarps - 1) / kWalkWarps);
         if (!FILL) {                 // counting pass: gr_np holds the total for the scan
             A.gr_nc[g] = nc;
             A.gr_np[g] = nn + nf;

@@ -61,3 +61,23 @@ def test_block_walk_and_parts(n, order):
         assert np.array_equal(out[2], off) and np.array_equal(out[3], idx)
         t.free()
     ctx.close()
+
+
+def test_walk_stack_is_counted_per_warp():
+    """max_walk_stack means pending nodes per warp whether a warp or a block walks a group:
+    at most the 768 entries of a warp's stack."""
+    import torch
+
+    from paper_2006_16560_gb300 import binding as B
+    pos, mass = _set(32768, 40, 1)
+    ctx = B.Context(0)
+    dp, dm = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    acc = torch.empty((32768, 3), dtype=torch.float64, device="cuda")
+    pot = torch.empty(32768, dtype=torch.float64, device="cuda")
+    t = B.Tree(ctx, dp, dm, B.Params(theta=0.2, r_in=0.02, r_out=0.2, n_leaf=2, n_group=64, order=0,
+                                     precision=B.PT_MIXED))
+    for _ in range(2):
+        _, st, _ = t.force(acc, pot)
+        assert 32 <= st.max_walk_stack <= 768
+    t.free()
+    ctx.close()
