@@ -191,6 +191,8 @@ struct pt_tree {
     std::vector<unsigned> gkey_n;
     std::vector<double> gkey_r;
     pt_params gkey_p{};
+    std::vector<const void *> gkey_at;         // addresses() and cap_pairs at the capture
+    unsigned long long gkey_pairs = 0;
     int gkey_mode = -1;
     // last results
     Status h{};
@@ -210,24 +212,34 @@ struct pt_tree {
     float ms_build = 0.f;
     int launches_build = 0, launches_force = 0;
 
+    // every device buffer, and the pinned blocks
+    std::vector<Buf *> bufs() {
+        return {&status, &sets, &set_of, &bmin, &bmax, &n_dev, &in_pos, &in_mass, &keys_in,
+                &vals_in, &qbuf, &skey, &perm, &sp64, &spH, &spL, &sq, &nd_a, &nd_b, &nd_r,
+                &nd_c, &nd_q, &nd_t, &nd_f, &nd_bnd, &nd_int, &topo_bs, &tmp_a, &tmp_b, &lcp, &gflag, &gbegin, &gr_r, &gr_a,
+                &gr_b, &gr_nc, &gr_np, &gr_co, &gr_po, &gr_nf, &gr_fo, &gr_wide, &gr_pb, &items, &parts, &gpart, &red_part, &cells, &pp, &pairs,
+                &nb_keys, &nb_keys_s, &nb_vals, &nb_vals_s, &nb_off, &nb_idx, &npairs_dev,
+                &sort_k2, &sort_v2, &sort_counts, &scan_sums, &out_acc, &out_pot,
+                &ffp, &ffn, &in_scale, &scale_buf, &set_mean, &ssc, &nd_thr, &gr_thr, &orb_vel, &orb_sv, &orb_rnbf, &walk_spill,
+                &orb_ndr, &orb_ndthr, &orb_grthr, &orb_ctr, &orb_rnb, &d_tab, &d_totals, &d_acc, &d_pot};
+    }
+    std::vector<void *> pinned() const { return {h_tab, h_sets_pin, h_totals, h_n, h_io, h_nboff, h_nbidx}; }
+    // Where they all lie: a captured batch holds these addresses.
+    std::vector<const void *> addresses() {
+        std::vector<const void *> v;
+        for (Buf *b : bufs()) v.push_back(b->p);
+        for (void *q : pinned()) v.push_back(q);
+        return v;
+    }
+
     void release() {
-        Buf *all[] = {&status, &sets, &set_of, &bmin, &bmax, &n_dev, &in_pos, &in_mass, &keys_in,
-                      &vals_in, &qbuf, &skey, &perm, &sp64, &spH, &spL, &sq, &nd_a, &nd_b, &nd_r,
-                      &nd_c, &nd_q, &nd_t, &nd_f, &nd_bnd, &nd_int, &topo_bs, &tmp_a, &tmp_b, &lcp, &gflag, &gbegin, &gr_r, &gr_a,
-                      &gr_b, &gr_nc, &gr_np, &gr_co, &gr_po, &gr_nf, &gr_fo, &gr_wide, &gr_pb, &items, &parts, &gpart, &red_part, &cells, &pp, &pairs,
-                      &nb_keys, &nb_keys_s, &nb_vals, &nb_vals_s, &nb_off, &nb_idx, &npairs_dev,
-                      &sort_k2, &sort_v2, &sort_counts, &scan_sums, &out_acc, &out_pot,
-                      &ffp, &ffn, &in_scale, &scale_buf, &set_mean, &ssc, &nd_thr, &gr_thr, &orb_vel, &orb_sv, &orb_rnbf, &walk_spill,
-                      &orb_ndr, &orb_ndthr, &orb_grthr, &orb_ctr, &orb_rnb};
-        for (Buf *b : all) b->release();
-        d_tab.release(); d_totals.release(); d_acc.release(); d_pot.release();
+        for (Buf *b : bufs()) b->release();
         if (gexec) cudaGraphExecDestroy(gexec);
         gexec = nullptr;
         if (gbuild) cudaGraphExecDestroy(gbuild);
         gbuild = nullptr;
         have_last_build = false;
-        void *pinned[] = {h_tab, h_sets_pin, h_totals, h_n, h_io, h_nboff, h_nbidx};
-        for (void *q : pinned)
+        for (void *q : pinned())
             if (q) cudaFreeHost(q);
         h_tab = nullptr; h_sets_pin = nullptr; h_totals = nullptr; h_n = nullptr;
         h_io = nullptr; h_nboff = nullptr; h_nbidx = nullptr;
@@ -980,6 +992,9 @@ int enqueue_batch(pt_tree *t, cudaStream_t st, bool host_io, bool want_nb) {
     return PT_OK;
 }
 
+// The captured sequence is this call's: the same shape, and every buffer still
+// where it was (another call on the batch tree may have let it grow, and the
+// graph would then read and write the blocks given up).
 bool graph_matches(pt_tree *t, int C, const pt_cluster_desc *d, const pt_params *p, int mode) {
     if (!t->gexec || t->gkey_mode != mode || (int)t->gkey_n.size() != C) return false;
     if (std::memcmp(&t->gkey_p, p, sizeof(pt_params)) != 0) return false;
@@ -987,7 +1002,7 @@ bool graph_matches(pt_tree *t, int C, const pt_cluster_desc *d, const pt_params 
         if (t->gkey_n[c] != (unsigned)d[c].n || t->gkey_r[2 * c] != d[c].r_in ||
             t->gkey_r[2 * c + 1] != d[c].r_out)
             return false;
-    return true;
+    return t->gkey_pairs == t->cap_pairs && t->gkey_at == t->addresses();
 }
 
 int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, int flags,
@@ -1167,6 +1182,8 @@ int batch_impl(pt_ctx *ctx, int C, pt_cluster_desc *d, const pt_params *params, 
             t->graph_nb_long = t->nb_long;
             t->gkey_mode = mode;
             t->gkey_p = *params;
+            t->gkey_at = t->addresses();
+            t->gkey_pairs = t->cap_pairs;
             t->gkey_n.resize(C);
             t->gkey_r.resize(2 * C);
             for (int c = 0; c < C; c++) {

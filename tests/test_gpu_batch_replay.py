@@ -122,3 +122,30 @@ def test_replay_with_rows_longer_than_captured():
             b.run(ctx, prm, graph=True)
             _assert_rows(b)
     ctx.close()
+
+
+@pytest.mark.parametrize("device", [True, False])
+@pytest.mark.parametrize("larger", [[9000], [300] * 40])
+def test_replay_after_a_larger_batch(device, larger):
+    """A batch with more particles or more sets moves the buffers that a captured one uses."""
+    from test_gpu_batch import _clusters, _run_batch
+    prm = B.Params(theta=0.5, n_leaf=8, n_group=64, order=2, precision=B.PT_MIXED)
+    ctx = B.Context(0)
+    cl = _clusters(50, [1200, 2100])
+    for _ in range(2):
+        rc, _, _ = _run_batch(ctx, cl, prm, flags=B.PT_BATCH_GRAPH, device=device)
+        assert rc == B.PT_OK
+    assert _run_batch(ctx, _clusters(60, larger), prm, device=device)[0] == B.PT_OK
+    rng = np.random.default_rng(3)
+    for _ in range(3):
+        for c in cl:
+            c["pos"] = c["pos"] + 1e-3 * rng.normal(size=c["pos"].shape)
+        rc, got, _ = _run_batch(ctx, cl, prm, flags=B.PT_BATCH_GRAPH, device=device)
+        assert rc == B.PT_OK
+        for c, r in zip(cl, got):
+            p = B.Params(**{**prm.__dict__, "r_in": c["r_in"], "r_out": c["r_out"]})
+            g = run_gpu(ctx, c["pos"], c["mass"], p)
+            for k in ("acc", "pot", "nb_off", "nb_idx"):
+                assert np.array_equal(r[k], g[k]), k
+            g["tree"].free()
+    ctx.close()
