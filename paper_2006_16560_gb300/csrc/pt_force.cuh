@@ -83,9 +83,14 @@ __device__ __forceinline__ Chg make_chg(const SetInfo &S) {
 // length depends on the set's own size and on the precision only, so a set's
 // results do not depend on what else is in a batch or on the launch.
 //
-// Entries per part at most: about 1.5 times the mean list at the upper end of
-// each range of set sizes, so that ordinary groups of large sets stay whole
-// (a part costs its targets' loads and a reduction again).  The float64
+// Entries per part at most (times 64 in the mixed kernel), tuned on Plummer
+// spheres at theta 0.3.  Against their mean lists: 2,048 entries are 2 times
+// the mean of 1,000 particles and 0.45 of that of 8,191, where most groups are
+// split (such sets have fewer groups than the GPU has SMs); 8,192 are 1.4 to 1.1
+// times (16,384 to 32,767), 16,384 are 1.7 to 1.5 times (10^5 to 262,143) and
+// 65,536 are 5 times (10^6 and 10^7), so that ordinary groups of large sets
+// stay whole (a part costs its targets' loads and a reduction again).  At theta
+// 0.6 lists are 3 to 5 times shorter and hardly any is split.  The float64
 // kernel's entries cost ~15 times as much, so its parts are an eighth as long.
 __device__ __forceinline__ unsigned part_entries(unsigned n, unsigned shift) {
     return (n < 8192u ? 32u : n < 32768u ? 128u : n < 262144u ? 256u : 1024u) << shift;

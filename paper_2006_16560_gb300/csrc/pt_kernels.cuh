@@ -17,8 +17,12 @@ constexpr unsigned long long kWalkChunkEntries = 8192;   // one-pass list alloca
 // A group is wide when a side of its grid box is at least 2^-kWalkWideShift of
 // the root box: it is listed by the build and walked by a whole block (see
 // pt_walk.cu).  2^-4 finds the groups with many times the mean list (a box
-// that reaches the core from the halo) among about 2% of a Plummer sphere's
-// groups; 2^-5 lists twice as many at the same walk times.  Sets below
+// that reaches the core from the halo) among 9 to 1% of a Plummer sphere's
+// groups (16,384 to 250,007 particles); 2^-5 lists twice as many at the same
+// walk times.  In uniform sets nearly every group is wide up to 10^5 particles,
+// and their walks are no slower for it (one warp per group -> now: sphere of
+// 16,384 102 -> 72 us, of 100,003 204 -> 167, of 250,007 319 -> 294; cube of
+// 100,003 211 -> 168; a fractal of 100,003 143 -> 90).  Sets below
 // kWalkWideMin particles have none: their walks take a few dozen steps, and a
 // block's steps cost more than a warp's (1,000 particles: 39 against 32 us).
 constexpr unsigned kWalkWideShift = 4, kWalkWideMin = 2048;
@@ -60,8 +64,11 @@ struct BuildArgs {
     unsigned *gr_wide;               // groups with a wide box, in any order
     int n_leaf, n_group;
     // deepest level the launch sequence covers (kMaxLevel: every tree): the
-    // depth of the tree's last build and two more, since an empty level still
-    // costs its three kernels; a deeper tree is flagged (kErrLevels)
+    // depth of a recent build of the tree plus a margin (two at first, doubled
+    // whenever a tree was deeper, so that one that often is ends at every
+    // level), since an empty level still costs its three kernels; a deeper
+    // tree is flagged (kErrLevels) and built again.  Not used by sets small
+    // enough for one block (kSmallBuild in pt_build.cu)
     int levels;
     // mass-dependent changeover radii (Eq. 12): per-particle factors in input
     // order (NULL: computed from the masses when massdep, else all 1)
