@@ -184,6 +184,7 @@ __device__ __forceinline__ ft ft_rsqrt(ft r2) {
 // above float32's smallest number, and cells' m / r^3 below its largest (2^119
 // at 2^-23 box sides); 2^16 with opening angles above kFfQuad2Theta, where a
 // cell as wide as the box may be accepted at 2^-21 of it (Q / r^5 ~ 2^123).
+// Less where 1 / unit of acceleration or potential would pass 2^1023.
 struct FfUnits {
     int ex[3], es, em;
 };
@@ -196,7 +197,8 @@ __device__ __forceinline__ FfUnits ff_units(const SetInfo &S, double M, int quad
         u.ex[d] = ilogb(X) + 1;
         u.es = max(u.es, u.ex[d] - 60);
     }
-    u.em = M > 0.0 ? ilogb(M) + 1 - (quad == 3 ? 16 : 50) : 0;
+    const int em = M > 0.0 ? ilogb(M) + 1 : 0;
+    u.em = max(em - (quad == 3 ? 16 : 50), min(em, max(2 * u.es, u.es) - 1023));
     return u;
 }
 

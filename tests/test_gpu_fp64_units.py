@@ -86,3 +86,18 @@ def test_units_below_the_smallest_number(k, j):
         assert np.array_equal(p, p0 * 2.0 ** (j - k))
     else:
         assert np.abs(p).max() <= 1e-300
+
+
+@pytest.mark.parametrize("k,j", [(20, -950), (-30, -1005), (0, -1010)])
+def test_units_near_the_smallest_number(k, j):
+    """Accelerations and potentials just above float64's smallest normal number, near pairs among them."""
+    d = inputs.plummer(500, 5, masses="kroupa")
+    mass = np.ldexp(np.rint(np.ldexp(d["mass"], 24)), -24)      # few bits: exact in any unit
+    kw = dict(theta=0.0, n_leaf=8, n_group=64, order=0)
+    a0, p0, o0, i0 = _run(d["pos"], mass, r_in=0.05, r_out=0.5, **kw)
+    s = 2.0 ** k
+    a, p, o, i = _run(d["pos"] * s, mass * 2.0 ** j, r_in=0.05 * s, r_out=0.5 * s, **kw)
+    assert len(i0) > 500 and np.array_equal(o, o0) and np.array_equal(i, i0)
+    # near pairs lose bits where m / r^3 falls below the smallest normal number
+    assert np.abs(a * 2.0 ** 900 * 2.0 ** (2 * k - j - 900) - a0).max() <= 1e-10 * np.abs(a0).max()
+    assert np.abs(p * 2.0 ** 900 * 2.0 ** (k - j - 900) - p0).max() <= 1e-10 * np.abs(p0).max()
