@@ -72,8 +72,8 @@ def test_list_and_pass_edges(n, r_out):
 
 @pytest.mark.parametrize("k,j", [(400, -300), (480, -100), (320, -760)])
 def test_units_below_the_smallest_number(k, j):
-    """Units in which accelerations or potentials fall below float64's range: zero, as with
-    float64 instructions, not infinity times zero (near pairs are scaled by 1 / unit)."""
+    """Units in which accelerations or potentials fall below float64's range: zero, not
+    infinity times zero (near pairs are scaled by 1 / unit)."""
     d = inputs.plummer(500, 5, masses="kroupa")
     kw = dict(theta=0.5, n_leaf=8, n_group=64, order=2)
     _, p0, o0, i0 = _run(d["pos"], d["mass"], r_in=0.05, r_out=0.5, **kw)
